@@ -1,0 +1,37 @@
+"""Closest-pair kernels at the sizes where their tiling can go wrong, against
+the FP64 oracle (pairs equal, distances the rounded FP64 values: exact, since
+FP32 values only choose which pairs are recomputed in FP64)."""
+import math
+
+import numpy as np
+import pytest
+
+import datagen
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_2107_05537_gb300 as pm  # noqa: E402
+
+
+def _check(X, A, k, gamma, T, leaf):
+    ix = pm.Index(torch.from_numpy(X).cuda(), m=A.shape[0], leaf_size=leaf, proj=A)
+    t, _, _ = oracle.params(A.shape[0], 1.5, 1 / math.e)
+    got = ix.closest_pairs(k=k, gamma=gamma, T=T, t=t)
+    lay = ix.layout()
+    ix.close()
+    ref = oracle.cp_radius_filter(X, A, lay, k, t, gamma, T)
+    assert got["pairs"].tolist() == ref["pairs"].tolist()
+    assert np.array_equal(got["dists"], ref["dists"].astype(np.float32))
+    for f, g in (("count", "count"), ("lca_nodes", "nodes"), ("nodes_done", "nodes_done")):
+        assert got["stats"][f] == ref[g]
+    return got
+
+
+# rows of 1 to 9 steps of 32 coordinates: below, at and past a four-step round
+@pytest.mark.parametrize("d", [1, 31, 33, 96, 97, 128, 129, 257])
+def test_pair_distance_row_lengths(d):
+    X, _, _, _ = datagen.mixture(700, d, 7, 1.0, seed=d)
+    A = oracle.gen_projection(3, 15, d).astype(np.float32)
+    _check(X, A, 9, 2.0, 10 ** 9, 16)
