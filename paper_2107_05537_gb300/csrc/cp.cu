@@ -6,8 +6,9 @@
 //                   largest distance, the same arithmetic as the oracle
 //   [host]          FindLCA: maximal inner nodes with radius < R = gamma t ub,
 //                   sorted by (radius, node id)
-//   k_cp_node_pairs cross-leaf pairs of a node's subtree with projected
-//                   distance < t ub (FP32 with a proven band, FP64 inside it)
+//   k_cp_tiles      cross-leaf pairs of nodes' subtrees with projected distance
+//                   < t ub (FP32 with a proven band, FP64 inside it)
+//   k_cp_replay     the nodes of a batch in order, for one value of ub
 //   k_pair_*        exact top-k merges: radix select of an FP32 threshold,
 //                   guard set, FP64 distances, sort by (dist, i, j)
 #include <algorithm>
@@ -113,10 +114,6 @@ __global__ void k_node_ball(const double *__restrict__ O64, const int64_t *__res
     }
 }
 
-// Cross-leaf pairs of positions [lo, hi) whose FP64 projected distance is
-// < Rt (strict, Algorithm 4).  FP32: |sqrt(d'^2_32) - d'_64| <= eps, so
-// d'^2_32 < loT is surely in, > hiT surely out, and the rest is decided in
-// FP64.  Thread per first position a; loops over b > a.
 // Sec. 6.3, setting of gamma: for every pair (a, b), a < b, of the n
 // positions of a layout, R / ||o_a', o_b'|| with R the radius of their lowest
 // common node (descending from the root while both leaves lie in one child;
@@ -178,39 +175,118 @@ __global__ void k_gather_rows(const float *__restrict__ X, int ld, int d, const 
     for (int j = threadIdx.x; j < d; j += blockDim.x) S[i * d + j] = x[j];
 }
 
-__global__ void k_cp_node_pairs(const float *__restrict__ O32, const double *__restrict__ O64, int m,
-                                const int32_t *__restrict__ leafOfPos, int64_t lo, int64_t hi, float loT,
-                                float hiT, double Rt, PairCand *__restrict__ out, unsigned long long *cnt,
-                                unsigned long long cap, unsigned long long *fp64n)
+// Cross-leaf pairs (a, b), a < b, of node subtrees whose FP32 projected
+// squared distance is at most hiT, by tiles of CT x CT positions: a listed
+// tile (`tiles`), or, without a list, the tiles of the one node [lo, hi) by
+// the grid (x: columns, y: rows).  exact: only the pairs with FP64 projected
+// distance < Rt (strict, Algorithm 4): |sqrt(d'^2_32) - d'_64| <= eps, so
+// d'^2_32 < loT is surely in, > hiT surely out, and the rest is decided in
+// FP64 (counted in fp64n); else the superset up to hiT, with the tile's node
+// number beside each pair.
+// Bound by instruction issue (about 45 per pair).  A thread holds one row and
+// takes 16 columns out of shared memory; the kept pairs of a warp are counted
+// first and take one atomic on the output counter.  A thread per row walking
+// the whole node left most of the GPU idle: 1,265 nodes of 79 points on average
+// took 94 ms in 1,265 launches, 0.08 ms in two tiled ones.
+constexpr int CT = 64;
+struct PairTile {
+    int32_t a0, b0;   // first row and column position (b0 >= a0)
+    int32_t hi;       // end of the node's positions
+    int32_t node;     // number of the node in its batch
+};
+
+__global__ void __launch_bounds__(256)
+k_cp_tiles(const float *__restrict__ O32, const double *__restrict__ O64, int m, const int32_t *__restrict__ leafOf,
+           const PairTile *__restrict__ tiles, int64_t lo, int64_t hi, int exact, float loT, float hiT, double Rt,
+           PairCand *__restrict__ out, int32_t *__restrict__ outNode, unsigned long long *cnt, unsigned long long cap,
+           unsigned long long *fp64n)
 {
-    const int64_t a = lo + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (a >= hi) return;
-    float oa[PM_MP];
+    constexpr int NC = CT * CT / 256;   // columns per thread
+    __shared__ float4 sO[CT][PM_MP / 4];
+    __shared__ int sLeaf[CT];
+    const int t = threadIdx.x, lane = t & 31, r = t & (CT - 1), part = t / CT;
+    const int64_t rows = tiles ? 1 : (hi - lo + CT - 1) / CT;
+    for (int64_t ty = blockIdx.y; ty < rows; ty += gridDim.y) {
+        int64_t a0, b0, end;
+        int node = 0;
+        if (tiles) {
+            const PairTile T = tiles[blockIdx.x];
+            a0 = T.a0;
+            b0 = T.b0;
+            end = T.hi;
+            node = T.node;
+        } else {
+            a0 = lo + ty * CT;
+            b0 = lo + (int64_t)blockIdx.x * CT;
+            end = hi;
+            if (b0 < a0) continue;   // block-uniform
+        }
+        __syncthreads();
+        {
+            // CT columns of four float4 each: one per thread
+            const int64_t b = b0 + (t >> 2);
+            sO[t >> 2][t & 3] = b < end ? ((const float4 *)(O32 + b * PM_MP))[t & 3] : make_float4(0.f, 0.f, 0.f, 0.f);
+            if (t < CT) sLeaf[t] = b0 + t < end ? leafOf[b0 + t] : -1;
+        }
+        __syncthreads();
+        const int64_t a = a0 + r;
+        const bool av = a < end;
+        float oa[PM_MP];
 #pragma unroll
-    for (int j = 0; j < PM_MP; j++) oa[j] = O32[a * PM_MP + j];
-    const int la = leafOfPos[a];
-    for (int64_t b = a + 1; b < hi; b++) {
-        if (leafOfPos[b] == la) continue;
-        const float v = pm_pd2_32(oa, O32 + b * PM_MP);
-        bool in = v < loT;
-        if (!in && v <= hiT) {
-            atomicAdd(fp64n, 1ull);
-            in = pm_pdist64(O64 + a * PM_MP, O64 + b * PM_MP, m) < Rt;
+        for (int j4 = 0; j4 < PM_MP / 4; j4++) {
+            const float4 v = av ? ((const float4 *)(O32 + a * PM_MP))[j4] : make_float4(0.f, 0.f, 0.f, 0.f);
+            oa[4 * j4] = v.x;
+            oa[4 * j4 + 1] = v.y;
+            oa[4 * j4 + 2] = v.z;
+            oa[4 * j4 + 3] = v.w;
         }
-        if (in) {
-            unsigned long long slot = atomicAdd(cnt, 1ull);
-            if (slot < cap) {
-                PairCand pc;
-                pc.key = v;
-                pc.a = (int32_t)a;
-                pc.b = (int32_t)b;
-                out[slot] = pc;
+        const int la = av ? leafOf[a] : -1;
+        float v[NC];
+        unsigned keep = 0u;
+#pragma unroll
+        for (int c = 0; c < NC; c++) {
+            const int cc = part * NC + c;
+            v[c] = pm_pd2_32(oa, (const float *)sO[cc]);
+            const int64_t b = b0 + cc;
+            const int lb = sLeaf[cc];
+            if (av && b > a && b < end && lb != la && v[c] <= hiT) keep |= 1u << c;
+        }
+        if (exact) {
+#pragma unroll
+            for (int c = 0; c < NC; c++)
+                if (((keep >> c) & 1u) && !(v[c] < loT)) {
+                    atomicAdd(fp64n, 1ull);
+                    if (!(pm_pdist64(O64 + a * PM_MP, O64 + (b0 + part * NC + c) * PM_MP, m) < Rt)) keep &= ~(1u << c);
+                }
+        }
+        const int mine = __popc(keep);
+        int incl = mine;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += x;
+        }
+        const int total = __shfl_sync(0xffffffffu, incl, 31);
+        unsigned long long base = 0;
+        if (lane == 0 && total) base = atomicAdd(cnt, (unsigned long long)total);
+        base = __shfl_sync(0xffffffffu, base, 0) + (unsigned long long)(incl - mine);
+#pragma unroll
+        for (int c = 0; c < NC; c++)
+            if ((keep >> c) & 1u) {
+                if (base < cap) {
+                    PairCand pc;
+                    pc.key = v[c];
+                    pc.a = (int32_t)a;
+                    pc.b = (int32_t)(b0 + part * NC + c);
+                    out[base] = pc;
+                    if (outNode) outNode[base] = node;
+                }
+                base++;
             }
-        }
     }
 }
 
-// Original-space FP32 squared distances of candidate pairs (overwrites key).
+// Original-space FP32 squared distances of candidate pairs, into dst [n] or, if
+// that is null, over the pairs' keys.
 // Bound by the L2 reads of the two rows (8 ld bytes per pair, 24 ld^-1 flops
 // per byte): eight lanes take a pair, so that every load instruction of the
 // warp covers whole 128-byte lines of four pairs' rows, and four loads of each
@@ -221,7 +297,7 @@ __global__ void k_cp_node_pairs(const float *__restrict__ O32, const double *__r
 // out of L1 and L2) against 36.3 ms for a thread per pair with scalar loads.
 // Requires ld % 32 == 0 (rows padded with zeros).
 __global__ void __launch_bounds__(256)
-k_pair_dist32(const float *__restrict__ X, int ld, PairCand *__restrict__ p, int64_t n)
+k_pair_dist32(const float *__restrict__ X, int ld, PairCand *__restrict__ p, int64_t n, float *__restrict__ dst)
 {
     const int lane = threadIdx.x & 31, grp = lane >> 3, g = lane & 7, nf4 = ld >> 2;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -258,16 +334,19 @@ k_pair_dist32(const float *__restrict__ X, int ld, PairCand *__restrict__ p, int
         acc = __fadd_rn(acc, __shfl_xor_sync(0xffffffffu, acc, 1));
         acc = __fadd_rn(acc, __shfl_xor_sync(0xffffffffu, acc, 2));
         acc = __fadd_rn(acc, __shfl_xor_sync(0xffffffffu, acc, 4));
-        if (e < n && g == 0) p[e].key = acc;
+        if (e < n && g == 0) {
+            if (dst) dst[e] = acc;
+            else p[e].key = acc;
+        }
     }
 }
 
 // Launches k_pair_dist32: four pairs per warp and step, up to eight 256-thread
 // blocks per SM.
-void launch_pair_dist32(const pmlsh_index *ix, PairCand *p, int64_t n, cudaStream_t st)
+void launch_pair_dist32(const pmlsh_index *ix, PairCand *p, int64_t n, cudaStream_t st, float *dst = nullptr)
 {
     const unsigned grid = (unsigned)std::min<int64_t>((n + 31) / 32, 8 * 152);
-    PM_LAUNCH("k_pair_dist32", st, k_pair_dist32<<<grid, 256, 0, st>>>(ix->X, ix->ld, p, n));
+    PM_LAUNCH("k_pair_dist32", st, k_pair_dist32<<<grid, 256, 0, st>>>(ix->X, ix->ld, p, n, dst));
 }
 
 // Histogram of key bits [sh, sh+w) among keys whose bits above sh+w equal
@@ -317,11 +396,68 @@ __global__ void k_pair_collect(const PairCand *__restrict__ p, int64_t n, float 
     out[slot] = x;
 }
 
-__device__ __forceinline__ bool pe_less(const PairExact &x, const PairExact &y)
+__host__ __device__ __forceinline__ bool pe_less(const PairExact &x, const PairExact &y)
 {
     if (x.dist != y.dist) return x.dist < y.dist;
     if (x.i != y.i) return x.i < y.i;
     return x.j < y.j;
+}
+
+// A batch of nodes [from, to) replayed for one value of ub: per node the
+// candidates with FP64 projected distance < Rt (FP32 band as in k_cp_tiles) and
+// the FP64 decisions taken, and, with FP64 distances, those that may enter the
+// top-k (FP32 squared distance <= thr).  Entries of one node are mostly
+// neighbours: lanes with the same node add once.
+struct NodeExact {
+    PairExact x;
+    int32_t node;
+    int32_t pad;
+};
+
+__global__ void __launch_bounds__(256)
+k_cp_replay(const PairCand *__restrict__ cand, const int32_t *__restrict__ node, const float *__restrict__ d32,
+            int64_t n, int from, int to, float loT, float hiT, double Rt, float thr, const float *__restrict__ X, int ld,
+            int d, const double *__restrict__ O64, int m, const int32_t *__restrict__ perm, int *__restrict__ nodeCnt,
+            int *__restrict__ nodeFp, NodeExact *__restrict__ out, unsigned long long *nOut, unsigned long long cap)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    // (the last round is entered by whole warps)
+    for (int64_t e0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); e0 < n; e0 += step) {
+        const int64_t e = e0 + lane;
+        const int nd = e < n ? node[e] : -1;
+        bool in = false, fp = false;
+        PairCand c;
+        if (nd >= from && nd < to) {
+            c = cand[e];
+            in = c.key < loT;
+            if (!in && c.key <= hiT) {
+                fp = true;
+                in = pm_pdist64(O64 + (int64_t)c.a * PM_MP, O64 + (int64_t)c.b * PM_MP, m) < Rt;
+            }
+        }
+        const unsigned peers = __match_any_sync(0xffffffffu, nd);
+        const unsigned ins = __ballot_sync(0xffffffffu, in) & peers, fps = __ballot_sync(0xffffffffu, fp) & peers;
+        if (lane == __ffs(peers) - 1) {
+            if (ins) atomicAdd(&nodeCnt[nd], __popc(ins));
+            if (fps) atomicAdd(&nodeFp[nd], __popc(fps));
+        }
+        if (in && d32[e] <= thr) {
+            const unsigned long long slot = atomicAdd(nOut, 1ull);
+            if (slot < cap) {
+                NodeExact y;
+                y.x.dist = pm_dist64(X + (int64_t)c.a * ld, X + (int64_t)c.b * ld, d);
+                const int64_t ia = perm[c.a], ib = perm[c.b];
+                y.x.i = ia < ib ? ia : ib;
+                y.x.j = ia < ib ? ib : ia;
+                y.x.a = c.a;
+                y.x.b = c.b;
+                y.node = nd;
+                y.pad = 0;
+                out[slot] = y;
+            }
+        }
+    }
 }
 
 // One block: sorts n (<= PAIR_SORT_CAP) entries by (dist, i, j) in place.
@@ -1003,14 +1139,38 @@ pmlsh_status pm_closest_pair(pmlsh_index *ix, const pmlsh_cp_opts *o, int64_t *o
             for (int64_t p = ix->leafOffH[l]; p < ix->leafOffH[l + 1]; p++) lof[p] = (int32_t)l;
         PM_CUDA(cudaMemcpyAsync(dLeafOf, lof.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     }
-    // 3. nodes in ascending radius while count <= T
+    // 3. nodes in ascending radius while count <= T.  A node's filter depends on
+    // ub as the nodes before it leave it, but ub changes at a few nodes only
+    // (tens of thousands of candidates per change), so nodes are taken in
+    // batches: the candidates of every node of a batch are listed for the ub at
+    // its start (a superset for each later, smaller ub) with their distances,
+    // and the nodes are replayed in order from per-node counts and the few
+    // candidates that may enter the top-k; where ub falls, the rest of the batch
+    // is counted again for the new ub.  On 100,000 x 512 (1,265 nodes, 2.2 M
+    // candidates) node by node took 245 ms, most of it 1,265 rounds of five host
+    // synchronisations; two batches and 13 replays take 4 ms.
     int64_t nodesDone = 0, fp64 = 0;
     PairCand *cand = nullptr;
     size_t candCap = 0;
-    for (size_t ai = 0; ai < A.size() && count <= T; ai++) {
-        const int64_t e = A[ai];
-        const int64_t lo = pLo[e], hi = pHi[e];
+    struct Cut { float lo, hi; };
+    auto cut_of = [&](double Rt) -> Cut {
+        Cut c{INFINITY, INFINITY};   // infinite ub: every pair is a candidate
+        if (!std::isinf(Rt)) {
+            const double eps = 0x1.0p-22 * ix->maxNorm + 0x1.0p-19 * Rt + 1e-300;
+            c.lo = Rt - eps > 0 ? (float)((Rt - eps) * (Rt - eps)) : -1.f;
+            if ((double)c.lo > (Rt - eps) * (Rt - eps)) c.lo = nextafterf(c.lo, -INFINITY);
+            c.hi = (float)((Rt + eps) * (Rt + eps));
+            if ((double)c.hi < (Rt + eps) * (Rt + eps)) c.hi = nextafterf(c.hi, INFINITY);
+        }
+        return c;
+    };
+    // one node by itself: a node that crosses count > T, one met while ub is
+    // infinite, or one with more candidates than a batch takes
+    auto single = [&](size_t ai) -> pmlsh_status {
+        const int64_t lo = pLo[A[ai]], hi = pHi[A[ai]];
         const double Rt = t * ub;
+        const Cut c = cut_of(Rt);
+        const int64_t nt = (hi - lo + CT - 1) / CT;
         int64_t ncand = 0;
         for (int attempt = 0; attempt < 2; attempt++) {
             if (!cand) {
@@ -1018,25 +1178,18 @@ pmlsh_status pm_closest_pair(pmlsh_index *ix, const pmlsh_cp_opts *o, int64_t *o
                 PM_TRY(mem.get(&cand, candCap));
             }
             PM_CUDA(cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), st));
-            float loT = -1.f, hiT = INFINITY;
-            if (!std::isinf(Rt)) {
-                const double eps = 0x1.0p-22 * ix->maxNorm + 0x1.0p-19 * Rt + 1e-300;
-                loT = Rt - eps > 0 ? (float)((Rt - eps) * (Rt - eps)) : -1.f;
-                if ((double)loT > (Rt - eps) * (Rt - eps)) loT = nextafterf(loT, -INFINITY);
-                hiT = (float)((Rt + eps) * (Rt + eps));
-                if ((double)hiT < (Rt + eps) * (Rt + eps)) hiT = nextafterf(hiT, INFINITY);
-            } else {
-                loT = INFINITY;   // every pair is a candidate
-                hiT = INFINITY;
-            }
-            PM_LAUNCH("k_cp_node_pairs", st, k_cp_node_pairs<<<(unsigned)((hi - lo + 127) / 128), 128, 0, st>>>(
-                ix->O32, ix->O64, ix->m, dLeafOf, lo, hi, loT, hiT, Rt, cand, cnt, candCap, cnt + 1));
+            PM_LAUNCH("k_cp_tiles", st, k_cp_tiles<<<dim3((unsigned)nt, (unsigned)std::min<int64_t>(nt, 65535)), 256, 0, st>>>(
+                ix->O32, ix->O64, ix->m, dLeafOf, nullptr, lo, hi, 1, c.lo, c.hi, Rt, cand, nullptr, cnt, candCap,
+                cnt + 1));
             PM_CUDA(cudaGetLastError());
             unsigned long long hc[2];
             PM_CUDA(cudaMemcpyAsync(hc, cnt, sizeof(hc), cudaMemcpyDeviceToHost, st));
             PM_CUDA(cudaStreamSynchronize(st));
-            fp64 += (int64_t)hc[1];
-            if (hc[0] <= candCap) { ncand = (int64_t)hc[0]; break; }
+            if (hc[0] <= candCap) {
+                ncand = (int64_t)hc[0];
+                fp64 += (int64_t)hc[1];
+                break;
+            }
             // grow and redo this node
             candCap = (size_t)hc[0];
             cand = nullptr;
@@ -1054,6 +1207,128 @@ pmlsh_status pm_closest_pair(pmlsh_index *ix, const pmlsh_cp_opts *o, int64_t *o
         count += keep;
         ub = (int)top.v.size() >= k ? top.v[k - 1].dist : INFINITY;
         nodesDone++;
+        return PMLSH_OK;
+    };
+    // batches: up to CB_CAND candidates (20 bytes each), CB_TILES tiles
+    constexpr unsigned long long CB_CAND = 1ull << 22;
+    constexpr size_t CB_TILES = (size_t)1 << 16, CB_NODES = (size_t)1 << 14;
+    PairCand *bCand = nullptr;
+    int32_t *bNode = nullptr;
+    float *bD32 = nullptr;
+    PairTile *bTiles = nullptr;
+    int *bCnt = nullptr;          // nodeCnt [CB_NODES], nodeFp [CB_NODES], then two 64-bit counters
+    NodeExact *bEx = nullptr;
+    std::vector<PairTile> tiles;
+    std::vector<int> cntH(2 * CB_NODES + 4);
+    std::vector<NodeExact> exH;
+    const double epsv = (double)(ix->ld + 8) * 0x1.0p-24;
+    size_t tileBudget = 512, grow = 8;   // tiles of a batch: few at first, which lower ub for the rest
+    for (size_t ai = 0; ai < A.size() && count <= T;) {
+        if ((int)top.v.size() < k) {
+            PM_TRY(single(ai++));
+            continue;
+        }
+        tiles.clear();
+        size_t aj = ai;
+        for (; aj < A.size() && aj - ai < CB_NODES; aj++) {
+            const int64_t lo = pLo[A[aj]], hi = pHi[A[aj]], nt = (hi - lo + CT - 1) / CT;
+            const size_t add = (size_t)(nt * (nt + 1) / 2);
+            if (tiles.size() + add > (aj == ai ? CB_TILES : tileBudget)) break;
+            for (int64_t y = 0; y < nt; y++)
+                for (int64_t x = y; x < nt; x++)
+                    tiles.push_back(PairTile{(int32_t)(lo + y * CT), (int32_t)(lo + x * CT), (int32_t)hi, (int32_t)(aj - ai)});
+        }
+        if (aj == ai) {   // one node of more tiles than a batch holds
+            PM_TRY(single(ai++));
+            continue;
+        }
+        if (!bCand) {
+            PM_TRY(mem.get(&bCand, (size_t)CB_CAND));
+            PM_TRY(mem.get(&bNode, (size_t)CB_CAND));
+            PM_TRY(mem.get(&bD32, (size_t)CB_CAND));
+            PM_TRY(mem.get(&bTiles, CB_TILES));
+            PM_TRY(mem.get(&bCnt, 2 * CB_NODES + 4));
+            PM_TRY(mem.get(&bEx, PAIR_SORT_CAP));
+        }
+        const int nb = (int)(aj - ai);
+        unsigned long long *bN = (unsigned long long *)(bCnt + 2 * nb);   // candidates, top-k entrants
+        const Cut c0 = cut_of(t * ub);
+        PM_CUDA(cudaMemcpyAsync(bTiles, tiles.data(), tiles.size() * sizeof(PairTile), cudaMemcpyHostToDevice, st));
+        PM_CUDA(cudaMemsetAsync(bN, 0, sizeof(unsigned long long), st));
+        PM_LAUNCH("k_cp_tiles", st, k_cp_tiles<<<(unsigned)tiles.size(), 256, 0, st>>>(
+            ix->O32, ix->O64, ix->m, dLeafOf, bTiles, 0, 0, 0, c0.lo, c0.hi, 0.0, bCand, bNode, bN, CB_CAND, cnt));
+        PM_CUDA(cudaGetLastError());
+        unsigned long long nC = 0;
+        PM_CUDA(cudaMemcpyAsync(&nC, bN, sizeof(nC), cudaMemcpyDeviceToHost, st));
+        PM_CUDA(cudaStreamSynchronize(st));
+        if (nC > CB_CAND) {
+            if (nb == 1) PM_TRY(single(ai++));
+            tileBudget = std::max<size_t>(1, std::min(tileBudget, tiles.size()) / 4);
+            grow = 2;
+            continue;
+        }
+        if (nC > 0) launch_pair_dist32(ix, bCand, (int64_t)nC, st, bD32);
+        PM_CUDA(cudaGetLastError());
+        const unsigned rgrid = (unsigned)std::max<unsigned long long>(1, std::min<unsigned long long>((nC + 255) / 256, 8 * 152));
+        int to = nb;
+        bool alone = false;   // the node at ai is taken by itself next
+        for (size_t base = ai; ai < aj && !alone;) {
+            // replay nodes [from, to) of the batch for this ub
+            const int from = (int)(ai - base);
+            const double Rt = t * ub, thr = ub * ub * (1.0 + 3.0 * epsv) + 1e-36;
+            const Cut c = cut_of(Rt);
+            float thr32 = (float)thr;
+            if ((double)thr32 < thr) thr32 = nextafterf(thr32, INFINITY);
+            PM_CUDA(cudaMemsetAsync(bCnt, 0, (size_t)(2 * nb + 4) * sizeof(int), st));
+            if (nC > 0)
+                PM_LAUNCH("k_cp_replay", st, k_cp_replay<<<rgrid, 256, 0, st>>>(
+                    bCand, bNode, bD32, (int64_t)nC, from, to, c.lo, c.hi, Rt, thr32, ix->X, ix->ld, ix->d, ix->O64,
+                    ix->m, ix->perm, bCnt, bCnt + nb, bEx, bN + 1, PAIR_SORT_CAP));
+            PM_CUDA(cudaGetLastError());
+            PM_CUDA(cudaMemcpyAsync(cntH.data(), bCnt, (size_t)(2 * nb + 4) * sizeof(int), cudaMemcpyDeviceToHost, st));
+            PM_CUDA(cudaStreamSynchronize(st));
+            unsigned long long nX;
+            std::memcpy(&nX, cntH.data() + 2 * nb + 2, sizeof(nX));
+            if (nX > PAIR_SORT_CAP) {
+                // more than the list holds: fewer nodes, down to one by itself
+                if (to - from == 1) alone = true;
+                else to = from + (to - from) / 2;
+                continue;
+            }
+            exH.resize((size_t)nX);
+            if (nX > 0) {
+                PM_CUDA(cudaMemcpyAsync(exH.data(), bEx, (size_t)nX * sizeof(NodeExact), cudaMemcpyDeviceToHost, st));
+                PM_CUDA(cudaStreamSynchronize(st));
+                std::sort(exH.begin(), exH.end(), [](const NodeExact &x, const NodeExact &y) {
+                    return x.node != y.node ? x.node < y.node : pe_less(x.x, y.x);
+                });
+            }
+            bool moved = false;
+            size_t x0 = 0;
+            for (int i = from; i < to && !moved && !alone; i++) {
+                if (count + cntH[i] > T) {
+                    alone = true;   // the cut inside a node (or, at count > T, the end)
+                    break;
+                }
+                size_t x1 = x0;
+                while (x1 < exH.size() && exH[x1].node == i) x1++;
+                if (x1 > x0) {
+                    for (size_t x = x0; x < x1; x++) top.v.push_back(exH[x].x);
+                    std::sort(top.v.begin(), top.v.end(), pe_less);
+                    top.v.resize(k);
+                    moved = top.v[k - 1].dist < ub;
+                    ub = top.v[k - 1].dist;
+                }
+                x0 = x1;
+                count += cntH[i];
+                fp64 += cntH[nb + i];
+                nodesDone++;
+                ai++;
+            }
+            if (!moved && !alone) to = nb;
+        }
+        if (alone && count <= T) PM_TRY(single(ai++));
+        tileBudget = std::min(CB_TILES, tileBudget * grow);
     }
     // results
     std::vector<int64_t> op((size_t)2 * k, -1);

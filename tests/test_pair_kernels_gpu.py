@@ -35,3 +35,29 @@ def test_pair_distance_row_lengths(d):
     X, _, _, _ = datagen.mixture(700, d, 7, 1.0, seed=d)
     A = oracle.gen_projection(3, 15, d).astype(np.float32)
     _check(X, A, 9, 2.0, 10 ** 9, 16)
+
+
+# nodes of one tile of 64 x 64 positions, at its edges and of several tiles;
+# one cluster makes one large node
+@pytest.mark.parametrize("n,clusters,leaf,k,gamma,T", [
+    (64, 1, 16, 3, math.inf, 10 ** 9),
+    (65, 1, 16, 3, math.inf, 10 ** 9),
+    (129, 1, 16, 3, math.inf, 10 ** 9),
+    (1000, 9, 16, 12, 1.4, 10 ** 9),
+    (1000, 9, 16, 400, 1.4, 10 ** 9),    # ub is infinite at the start: fewer self pairs than k
+    (1000, 9, 32, 12, 3.0, 6000),        # the budget cut inside a node
+    (6000, 40, 16, 1000, 2.5, 10 ** 9),  # many nodes, ub falls often
+])
+def test_node_tiles_and_replay(n, clusters, leaf, k, gamma, T):
+    X, _, _, _ = datagen.mixture(n, 20, clusters, 1.0, seed=n + k)
+    A = oracle.gen_projection(4, 15, 20).astype(np.float32)
+    _check(X, A, k, gamma, T, leaf)
+
+
+def test_more_entrants_than_the_list_holds():
+    # the ten self pairs that set ub are farther apart than most of the pairs
+    # between leaves, so one ub admits more than 4,096 of them
+    rng = np.random.default_rng(3)
+    X = rng.standard_normal((900, 6)).astype(np.float32)
+    A = oracle.gen_projection(4, 6, 6).astype(np.float32)
+    _check(X, A, 1024, math.inf, 10 ** 9, 16)
