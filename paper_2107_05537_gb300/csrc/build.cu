@@ -795,7 +795,7 @@ void DevBuf::release()
 }
 
 pmlsh_status pm_build_index(pmlsh_index *ix, const float *X, bool x_on_device,
-                            const pmlsh_build_opts *o, cudaStream_t st)
+                            const pmlsh_build_opts *o, cudaStream_t st, bool layoutOnly)
 {
     const int64_t n = ix->n;
     const int d = ix->d;
@@ -837,7 +837,7 @@ pmlsh_status pm_build_index(pmlsh_index *ix, const float *X, bool x_on_device,
         PM_CUDA(cudaGetLastError());
     }
     // 4. distance sample for r_min (Sec. 5.2), stream seed+3, original order
-    {
+    if (!layoutOnly) {
         int64_t np = o->rmin_pairs > 0 ? o->rmin_pairs : 10000;
         ix->distSample.clear();
         if (n >= 2) {
@@ -932,9 +932,15 @@ pmlsh_status pm_build_index(pmlsh_index *ix, const float *X, bool x_on_device,
     PM_CUDA(cudaMemcpyAsync(ix->perm, ix->permH.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     PM_TRY(dalloc(&ix->leafOff, L + 1));
     PM_CUDA(cudaMemcpyAsync(ix->leafOff, ix->leafOffH.data(), (L + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, st));
+    PM_TRY(dalloc(&ix->O64, (size_t)n * PM_MP));
+    if (layoutOnly) {
+        PM_LAUNCH("k_gather_rows", st, k_gather_rows<double><<<2048, 256, 0, st>>>(O64o, ix->O64, ix->perm, n, PM_MP));
+        PM_CUDA(cudaGetLastError());
+        PM_CUDA(cudaStreamSynchronize(st));
+        return PMLSH_OK;
+    }
     PM_TRY(dalloc(&ix->X, (size_t)n * ld));
     PM_TRY(dalloc(&ix->O32, (size_t)n * PM_MP));
-    PM_TRY(dalloc(&ix->O64, (size_t)n * PM_MP));
     PM_LAUNCH("k_gather_rows", st, k_gather_rows<float><<<2048, 256, 0, st>>>(Xo, ix->X, ix->perm, n, ld));
     PM_LAUNCH("k_gather_rows", st, k_gather_rows<float><<<2048, 256, 0, st>>>(O32o, ix->O32, ix->perm, n, PM_MP));
     PM_LAUNCH("k_gather_rows", st, k_gather_rows<double><<<2048, 256, 0, st>>>(O64o, ix->O64, ix->perm, n, PM_MP));

@@ -1052,10 +1052,20 @@ pmlsh_status pm_gamma_calibrate(pmlsh_index *ix, double pr, int64_t nsample, uin
     bo.seed = ix->seed;
     bo.proj = ix->A_host.data();
     bo.bf16_shadow = 0;
-    pmlsh_index *sub = nullptr;
-    pmlsh_status s = pmlsh_build(S, nsample, ix->d, &bo, st, &sub);
-    if (s == PMLSH_OK) s = gamma_of_layout(sub, pr, gamma, st);
-    pmlsh_free(sub);
+    // (only its hierarchy and projected points: what queries read of an index,
+    // the principal directions of its leaf centres above all, took 75 of the
+    // 100 ms of a calibration on 100,000 x 512)
+    pmlsh_index sub;
+    sub.n = nsample;
+    sub.d = ix->d;
+    sub.ld = ix->ld;
+    sub.m = bo.m;
+    sub.s = (int)std::min<int64_t>(bo.s, (nsample + bo.leaf_size - 1) / bo.leaf_size);
+    sub.M = bo.leaf_size;
+    sub.seed = bo.seed;
+    pmlsh_status s = pm_build_index(&sub, S, true, &bo, st, true);
+    if (s == PMLSH_OK) s = gamma_of_layout(&sub, pr, gamma, st);
+    pm_free_index(&sub);
     return s;
 }
 

@@ -132,9 +132,10 @@ struct pmlsh_index {
     KnnWork work;
 };
 
-// Build helpers (build.cu)
+// Build helpers (build.cu).  layoutOnly: the leaf hierarchy and the FP64
+// projected points in leaf order only (no structure that queries read).
 pmlsh_status pm_build_index(pmlsh_index *ix, const float *X, bool x_on_device,
-                            const pmlsh_build_opts *o, cudaStream_t st);
+                            const pmlsh_build_opts *o, cudaStream_t st, bool layoutOnly = false);
 void pm_free_index(pmlsh_index *ix);
 
 // FP64 + FP32 projection of rows X [n][ld] (build.cu), original row order;
