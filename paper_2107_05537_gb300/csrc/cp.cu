@@ -2,8 +2,8 @@
 // (Algorithm 5) over the index's leaf hierarchy.
 //
 //   k_cp_selfjoin   every pair inside each leaf: FP32 squared distance
-//   k_node_ball     node balls (Sec. 4.1) in FP64, bounding-box midpoint and
-//                   largest distance, the same arithmetic as the oracle
+//   k_node_box,     node balls (Sec. 4.1) in FP64, bounding-box midpoint and
+//   k_node_radius   largest distance, the same arithmetic as the oracle
 //   [host]          FindLCA: maximal inner nodes with radius < R = gamma t ub,
 //                   sorted by (radius, node id)
 //   k_cp_tiles      cross-leaf pairs of nodes' subtrees with projected distance
@@ -59,59 +59,96 @@ __global__ void k_cp_selfjoin(const float *__restrict__ X, int ld, const int64_t
     }
 }
 
-__device__ __forceinline__ double dmin_warp(double v)
+// Node balls in FP64 (Sec. 4.1): centre = midpoint of the bounding box of the
+// node's projected points, radius = largest FP64 distance to it.  A node is
+// cut into slices of NB_SLICE positions, a warp per slice: k_node_box takes the
+// bounding boxes (minima and maxima of order-preserving integer keys, which
+// leave the FP64 pipe to the distances), k_node_radius the largest distance;
+// the slices of a node meet in integer atomics, so no order matters.  Bound by
+// the FP64 pipe, two operations per SM and clock here: n depth 45 operations,
+// which slices spread evenly; a block per node left the root's 100,000 points
+// to one SM (77,000 nodes: 5.5 ms, in slices 0.3 ms).
+constexpr int NB_SLICE = 256;
+struct NodeSlice {
+    int64_t lo, hi;
+    int32_t node;
+    int32_t pad;
+};
+
+__device__ __forceinline__ long long nb_key(double v)
 {
-    for (int o = 16; o; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
 }
-__device__ __forceinline__ double dmax_warp(double v)
+__device__ __forceinline__ double nb_unkey(long long k)
 {
-    for (int o = 16; o; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffLL));
 }
 
-// Node ball in FP64: centre = midpoint of the bounding box of the node's
-// projected points, radius = largest FP64 distance to it.  One block (256
-// threads) per node.
-__global__ void k_node_ball(const double *__restrict__ O64, const int64_t *__restrict__ posLo,
-                            const int64_t *__restrict__ posHi, int m, double *__restrict__ rad)
+// box [node][2][PM_MP]: keys of the minima and maxima
+__global__ void k_node_box_init(long long *__restrict__ box, unsigned long long *__restrict__ rad, int64_t nodes)
 {
-    __shared__ double smn[8][PM_MP], smx[8][PM_MP], sro[PM_MP], srad[8];
-    const int e = blockIdx.x;
-    const int64_t a = posLo[e], b = posHi[e];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int j = 0; j < PM_MP; j++) {
-        double mn = INFINITY, mx = -INFINITY;
-        for (int64_t p = a + threadIdx.x; p < b; p += blockDim.x) {
-            double v = O64[p * PM_MP + j];
-            mn = fmin(mn, v);
-            mx = fmax(mx, v);
-        }
-        mn = dmin_warp(mn);
-        mx = dmax_warp(mx);
-        if (lane == 0) { smn[warp][j] = mn; smx[warp][j] = mx; }
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < nodes * 2 * PM_MP) box[i] = (i / PM_MP) % 2 == 0 ? 0x7fffffffffffffffLL : (long long)0x8000000000000000ULL;
+    if (i < nodes) rad[i] = 0ull;
+}
+
+__global__ void __launch_bounds__(256)
+k_node_box(const double *__restrict__ O64, const NodeSlice *__restrict__ sl, int64_t ns, long long *__restrict__ box)
+{
+    const int lane = threadIdx.x & 31, j = lane & 7;
+    const int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (i >= ns) return;   // warp-uniform
+    const NodeSlice S = sl[i];
+    // eight lanes per point, two coordinates per lane
+    long long mn0 = 0x7fffffffffffffffLL, mn1 = mn0, mx0 = (long long)0x8000000000000000ULL, mx1 = mx0;
+#pragma unroll 4
+    for (int64_t p = S.lo + (lane >> 3); p < S.hi; p += 4) {
+        const double2 v = __ldg((const double2 *)(O64 + p * PM_MP) + j);
+        const long long k0 = nb_key(v.x), k1 = nb_key(v.y);
+        mn0 = k0 < mn0 ? k0 : mn0;
+        mx0 = k0 > mx0 ? k0 : mx0;
+        mn1 = k1 < mn1 ? k1 : mn1;
+        mx1 = k1 > mx1 ? k1 : mx1;
     }
-    __syncthreads();
-    if (threadIdx.x < PM_MP) {
-        int j = threadIdx.x;
-        double mn = smn[0][j], mx = smx[0][j];
-        for (int w = 1; w < (int)(blockDim.x >> 5); w++) {
-            mn = fmin(mn, smn[w][j]);
-            mx = fmax(mx, smx[w][j]);
-        }
-        sro[j] = j < m ? __dmul_rn(0.5, __dadd_rn(mn, mx)) : 0.0;
+    for (int o = 8; o < 32; o <<= 1) {
+        const long long a = __shfl_xor_sync(0xffffffffu, mn0, o), b = __shfl_xor_sync(0xffffffffu, mn1, o);
+        const long long c = __shfl_xor_sync(0xffffffffu, mx0, o), d = __shfl_xor_sync(0xffffffffu, mx1, o);
+        mn0 = a < mn0 ? a : mn0;
+        mn1 = b < mn1 ? b : mn1;
+        mx0 = c > mx0 ? c : mx0;
+        mx1 = d > mx1 ? d : mx1;
     }
-    __syncthreads();
+    if (lane < 8) {
+        long long *B = box + (int64_t)S.node * 2 * PM_MP;
+        atomicMin(B + 2 * j, mn0);
+        atomicMin(B + 2 * j + 1, mn1);
+        atomicMax(B + PM_MP + 2 * j, mx0);
+        atomicMax(B + PM_MP + 2 * j + 1, mx1);
+    }
+}
+
+__global__ void __launch_bounds__(256)
+k_node_radius(const double *__restrict__ O64, const NodeSlice *__restrict__ sl, int64_t ns,
+              const long long *__restrict__ box, int m, unsigned long long *__restrict__ rad)
+{
+    __shared__ double sC[8][PM_MP];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + w;
+    if (i >= ns) return;   // warp-uniform
+    const NodeSlice S = sl[i];
+    const long long *B = box + (int64_t)S.node * 2 * PM_MP;
+    if (lane < PM_MP) sC[w][lane] = lane < m ? __dmul_rn(0.5, __dadd_rn(nb_unkey(B[lane]), nb_unkey(B[PM_MP + lane]))) : 0.0;
+    __syncwarp();
     double r = 0.0;
-    for (int64_t p = a + threadIdx.x; p < b; p += blockDim.x) r = fmax(r, pm_pdist64(O64 + p * PM_MP, sro, m));
-    r = dmax_warp(r);
-    if (lane == 0) srad[warp] = r;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double rr = srad[0];
-        for (int w = 1; w < (int)(blockDim.x >> 5); w++) rr = fmax(rr, srad[w]);
-        rad[e] = rr;
+    for (int64_t p = S.lo + lane; p < S.hi; p += 32) r = fmax(r, pm_pdist64(O64 + p * PM_MP, sC[w], m));
+    // distances are >= +0: their bits order like them
+    unsigned long long rb = (unsigned long long)__double_as_longlong(r);
+    for (int o = 16; o; o >>= 1) {
+        const unsigned long long x = __shfl_xor_sync(0xffffffffu, rb, o);
+        rb = x > rb ? x : rb;
     }
+    if (lane == 0) atomicMax(rad + S.node, rb);
 }
 
 // Sec. 6.3, setting of gamma: for every pair (a, b), a < b, of the n
@@ -756,6 +793,37 @@ struct DevPtrs {
     }
 };
 
+// FP64 ball radii of the index's nodes into dRad [N] (device); innerOnly: the
+// leaf nodes' entries are left at 0.
+pmlsh_status node_radii(const pmlsh_index *ix, bool innerOnly, DevPtrs &mem, double **dRad, cudaStream_t st)
+{
+    const int64_t N = (int64_t)ix->nodeLo.size();
+    std::vector<NodeSlice> sl;
+    sl.reserve((size_t)N);
+    for (int64_t e = 0; e < N; e++) {
+        if (innerOnly && ix->nodeLeft[e] < 0) continue;
+        const int64_t lo = ix->leafOffH[ix->nodeLo[e]], hi = ix->leafOffH[ix->nodeHi[e]];
+        for (int64_t a = lo; a < hi; a += NB_SLICE) sl.push_back(NodeSlice{a, std::min(hi, a + NB_SLICE), (int32_t)e, 0});
+    }
+    const int64_t ns = (int64_t)sl.size();
+    NodeSlice *dSl;
+    long long *box;
+    PM_TRY(mem.get(&dSl, (size_t)ns));
+    PM_TRY(mem.get(&box, (size_t)N * 2 * PM_MP));
+    PM_TRY(mem.get(dRad, (size_t)N));
+    PM_CUDA(cudaMemcpyAsync(dSl, sl.data(), (size_t)ns * sizeof(NodeSlice), cudaMemcpyHostToDevice, st));
+    PM_LAUNCH("k_node_box_init", st, k_node_box_init<<<(unsigned)((N * 2 * PM_MP + 255) / 256), 256, 0, st>>>(
+        box, (unsigned long long *)*dRad, N));
+    if (ns > 0) {
+        const unsigned g = (unsigned)((ns + 7) / 8);
+        PM_LAUNCH("k_node_box", st, k_node_box<<<g, 256, 0, st>>>(ix->O64, dSl, ns, box));
+        PM_LAUNCH("k_node_radius", st, k_node_radius<<<g, 256, 0, st>>>(ix->O64, dSl, ns, box, ix->m,
+                                                                        (unsigned long long *)*dRad));
+    }
+    PM_CUDA(cudaGetLastError());
+    return PMLSH_OK;
+}
+
 // Radix select over a device pair buffer: the rank-th smallest FP32 key
 // (1-based).  Three passes of 11/11/10 bits.
 pmlsh_status pair_kth(const PairCand *p, int64_t n, int64_t rank, unsigned int *hist, float *out, cudaStream_t st)
@@ -950,10 +1018,8 @@ static pmlsh_status gamma_of_layout(const pmlsh_index *lx, double pr, double *ga
     const int64_t npairs = n * (n - 1) / 2;
     DevPtrs mem;
     // node balls (FP64, the oracle's arithmetic)
-    std::vector<int64_t> pLo(N), pHi(N), nodeH((size_t)N * 4);
+    std::vector<int64_t> nodeH((size_t)N * 4);
     for (int64_t e = 0; e < N; e++) {
-        pLo[e] = lx->leafOffH[lx->nodeLo[e]];
-        pHi[e] = lx->leafOffH[lx->nodeHi[e]];
         nodeH[e * 4] = lx->nodeLeft[e];
         nodeH[e * 4 + 1] = lx->nodeRight[e];
         nodeH[e * 4 + 2] = lx->nodeLo[e];
@@ -962,25 +1028,20 @@ static pmlsh_status gamma_of_layout(const pmlsh_index *lx, double pr, double *ga
     std::vector<int32_t> lof(n);
     for (int64_t l = 0; l < L; l++)
         for (int64_t p = lx->leafOffH[l]; p < lx->leafOffH[l + 1]; p++) lof[p] = (int32_t)l;
-    int64_t *dLo, *dHi, *dNode;
+    int64_t *dNode;
     double *dRad, *ratio;
     int32_t *dLeafOf;
     unsigned int *hist;
     int *err;
-    PM_TRY(mem.get(&dLo, N));
-    PM_TRY(mem.get(&dHi, N));
     PM_TRY(mem.get(&dNode, (size_t)N * 4));
-    PM_TRY(mem.get(&dRad, N));
     PM_TRY(mem.get(&dLeafOf, n));
     PM_TRY(mem.get(&ratio, (size_t)npairs));
     PM_TRY(mem.get(&hist, 256));
     PM_TRY(mem.get(&err, 1));
-    PM_CUDA(cudaMemcpyAsync(dLo, pLo.data(), N * sizeof(int64_t), cudaMemcpyHostToDevice, st));
-    PM_CUDA(cudaMemcpyAsync(dHi, pHi.data(), N * sizeof(int64_t), cudaMemcpyHostToDevice, st));
     PM_CUDA(cudaMemcpyAsync(dNode, nodeH.data(), N * 4 * sizeof(int64_t), cudaMemcpyHostToDevice, st));
     PM_CUDA(cudaMemcpyAsync(dLeafOf, lof.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     PM_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
-    PM_LAUNCH("k_node_ball", st, k_node_ball<<<(unsigned)N, 256, 0, st>>>(lx->O64, dLo, dHi, lx->m, dRad));
+    PM_TRY(node_radii(lx, false, mem, &dRad, st));
     PM_LAUNCH("k_gamma_ratio", st, k_gamma_ratio<<<(unsigned)(n - 1), 256, 0, st>>>(lx->O64, n, lx->m, dLeafOf, dNode,
                                                                                      dRad, ratio, err));
     PM_CUDA(cudaGetLastError());
@@ -1115,15 +1176,8 @@ pmlsh_status pm_closest_pair(pmlsh_index *ix, const pmlsh_cp_opts *o, int64_t *o
         pLo[e] = ix->leafOffH[ix->nodeLo[e]];
         pHi[e] = ix->leafOffH[ix->nodeHi[e]];
     }
-    int64_t *dLo, *dHi;
     double *dRad;
-    PM_TRY(mem.get(&dLo, N));
-    PM_TRY(mem.get(&dHi, N));
-    PM_TRY(mem.get(&dRad, N));
-    PM_CUDA(cudaMemcpyAsync(dLo, pLo.data(), N * sizeof(int64_t), cudaMemcpyHostToDevice, st));
-    PM_CUDA(cudaMemcpyAsync(dHi, pHi.data(), N * sizeof(int64_t), cudaMemcpyHostToDevice, st));
-    PM_LAUNCH("k_node_ball", st, k_node_ball<<<(unsigned)N, 256, 0, st>>>(ix->O64, dLo, dHi, ix->m, dRad));
-    PM_CUDA(cudaGetLastError());
+    PM_TRY(node_radii(ix, true, mem, &dRad, st));
     std::vector<double> rad(N);
     PM_CUDA(cudaMemcpyAsync(rad.data(), dRad, N * sizeof(double), cudaMemcpyDeviceToHost, st));
     PM_CUDA(cudaStreamSynchronize(st));
