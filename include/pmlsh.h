@@ -252,7 +252,9 @@ typedef struct {
                          upper bound are reranked from the FP32 rows, then
                          FP64 where FP32 cannot decide; a query whose bounds
                          cannot settle that set is verified again without
-                         the first pass.  PMLSH_FP32_PLAIN (0): neither.
+                         the first pass; batches small enough for a block
+                         per query read the FP32 rows at once.
+                         PMLSH_FP32_PLAIN (0): neither.
                          Every mode returns the same ids, distances and
                          statistics |C|, rounds, stop rule (n_verified and
                          leaves_visited describe the work done).  Both BF16

@@ -14,7 +14,8 @@
 //   [host]         |S_i| per query -> which queries reach the budget B
 //   k_collect,     for budget queries: the B nearest in projected space
 //   k_select       (radix select, FP64 resolution of the band at the cut)
-//   k_verify       one warp per query: exact FP32 distances of the candidates
+//   k_verify       one warp per query (k_verify_block: one block per query, for
+//                  smaller batches): exact FP32 distances of the candidates
 //                  that can reach the top-k (leaves visited best first by an
 //                  original-space lower bound, chunks of <= 32 points skipped
 //                  by their own), guard set, FP64 distances, exact top-k and
@@ -831,50 +832,6 @@ k_select(const int32_t *__restrict__ sel, const int32_t *__restrict__ act, Thr *
 
 constexpr int VW_MAXWARPS = 8;                // queries in flight per block (one per warp)
 constexpr int VW_MINBLOCKS = 4;               // blocks per SM the register budget allows
-struct VwArgs {
-    const int32_t *act;
-    int na;
-    const Thr *thr;
-    const float *qp32, *qpiv;
-    int s;
-    const float *meta;
-    int64_t L;
-    const float *O32, *X, *Qd;
-    int ld, d;
-    const float *leafMu, *leafRx;
-    const int64_t *chunkOff;
-    const int32_t *leafChunk;
-    const float *chunkMu, *chunkRx;
-    int KP, k;
-    const int *inN, *inPos;
-    const int32_t *perm;
-    int64_t *outIds;
-    float *outD, *outErr;
-    double *dk;
-    int *fp64cnt, *nverOut, *nleafOut, *errFlag;
-    int *workCtr;   // next entry of `order` to take (persistent warps)
-    const int *order;   // [na] active queries, the costliest first
-    int *dbg;       // [3]: site, value, query of the first failed index check
-    int64_t n;      // points
-    int2 *lists;    // [warps][L]: per-warp candidate leaves {leaf, lower bound bits}
-    const uint32_t *leafBits;   // [na][W32]: leaves Eq. 5 does not exclude (k_class)
-    const uint32_t *fullBits;   // [na][W32]: leaves k_class calls full (all members within the radius)
-    int W32;
-    const double *O64, *qp64;   // FP64 projected points and queries
-    const float *leafPmu;       // [L][PM_PCA] leaf centres along the principal directions
-    const float *qpca, *qnx;    // [nq][PM_PCA] queries along them, [nq] ||q|| (rounded up)
-    float muMax;                // max ||mu_l|| (rounded up)
-    int m;
-    int inlineBand;             // 1: decide FP32 band points in FP64 here (no exact count ran)
-    int nwork;                  // entries of `order` to take
-    // BF16 first pass (bf16 != 0): residual rows and their rounding bounds;
-    // a query whose first-pass bounds cannot settle its rerank set is
-    // marked in redo[a] and verified again without the first pass
-    int bf16;
-    const uint16_t *Xr;
-    const float *rowErr;
-    int *redo;
-};
 
 constexpr int VW_WIN = 64;                    // leaves per window of the best-first walk
 constexpr uint32_t VW_TAKEN = 0xFFFFFFFFu;    // list key of a leaf already windowed
@@ -963,12 +920,6 @@ __device__ __forceinline__ void warp_sort_win(uint32_t *key, int32_t *val, int l
         }
 }
 
-#define VW_CHECK(cond, site, val)                                              \
-    (((cond)) ? true                                                           \
-              : (atomicCAS(&A.dbg[0], 0, (site)) == 0 ? (A.dbg[1] = (int)(val), A.dbg[2] = a, \
-                                                         atomicOr(A.errFlag, 1024), false)    \
-                                                      : (atomicOr(A.errFlag, 1024), false)))
-
 // Exact top-k of the candidate set, one warp per query (persistent warps
 // take active queries from a counter).  The candidates are the points with
 // FP32 d'^2 <= lov plus the FP64-resolved band-in points: listed by the
@@ -988,18 +939,16 @@ __device__ __forceinline__ void warp_sort_win(uint32_t *key, int32_t *val, int l
 //     value provably contain the exact k nearest; they are recomputed in
 //     FP64 and ranked by (FP64 distance, id).
 // The result equals verifying every candidate.
-template <bool WIDE, bool BF>
-__global__ void __launch_bounds__(32 * VW_MAXWARPS, WIDE ? 2 : VW_MINBLOCKS)
+__global__ void __launch_bounds__(32 * VW_MAXWARPS, VW_MINBLOCKS)
 k_verify(VwArgs A)
 {
     extern __shared__ __align__(16) unsigned char vsm[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int ld = A.ld, KP = A.KP, KPW = A.KP >> 5, k = A.k, s = A.s, nf4 = A.ld >> 2;
     const int64_t L = A.L;
-    // BF = false compiles the first pass out (the register-rich form without
-    // it has registers to spare); the 64-register form keeps one copy for
-    // both modes, measured faster than its FP32-only copy (1.74 vs 1.98 ms)
-    const bool bfAll = BF && A.bf16 != 0;
+    // one copy for both precisions: a copy without the first pass measured slower
+    // at 64 registers (1.98 vs 1.74 ms)
+    const bool bfAll = A.bf16 != 0;
     unsigned char *wbase = vsm + (size_t)wib * verify_smem_warp(ld, KP, A.bf16);
     double *gd = (double *)wbase;
     long long *gid = (long long *)(gd + KP);
@@ -1060,7 +1009,7 @@ k_verify(VwArgs A)
         }
         __syncwarp();
         auto D2 = [&](const float *p) -> float {
-            return WIDE ? warp_d2x4w(q4, p, nf4, lane) : warp_d2x4(q4, p, nf4, lane);
+            return warp_d2x4(q4, p, nf4, lane);
         };
         // top-KP state: lane owns slots lane, lane + 32, ...; cmax is the
         // largest entry (the KP-th smallest so far), cslot its slot
@@ -1503,37 +1452,8 @@ k_verify(VwArgs A)
             if (e2 < G && !VW_CHECK(p2 >= 0 && p2 < A.n, 5, p2)) p2 = -1;
             double s1 = 0.0, s2 = 0.0;
             const float *x1 = A.X + (int64_t)max(p, 0) * ld, *x2 = A.X + (int64_t)max(p2, 0) * ld;
-            // the same sequential sum over i = 0 .. d - 1, four coordinates per
-            // 16-byte load in the register-rich form (rows and the query are
-            // 16-byte aligned, zero-padded to ld; the tail past d is not summed)
             const bool two = p2 >= 0;
             int i = 0;
-            // (the 64-register form keeps scalar loads: its register budget
-            // is better spent elsewhere)
-            for (; WIDE && i + 4 <= A.d; i += 4) {
-                const float4 qv = *(const float4 *)(qs + i);
-                const float4 a1 = __ldg((const float4 *)(x1 + i));
-                const float4 a2 = two ? __ldg((const float4 *)(x2 + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                const double q0 = f2d_exact(qv.x), q1 = f2d_exact(qv.y), q2 = f2d_exact(qv.z), q3 = f2d_exact(qv.w);
-                double t = __dsub_rn(f2d_exact(a1.x), q0);
-                s1 = __dadd_rn(s1, __dmul_rn(t, t));
-                t = __dsub_rn(f2d_exact(a1.y), q1);
-                s1 = __dadd_rn(s1, __dmul_rn(t, t));
-                t = __dsub_rn(f2d_exact(a1.z), q2);
-                s1 = __dadd_rn(s1, __dmul_rn(t, t));
-                t = __dsub_rn(f2d_exact(a1.w), q3);
-                s1 = __dadd_rn(s1, __dmul_rn(t, t));
-                if (two) {
-                    t = __dsub_rn(f2d_exact(a2.x), q0);
-                    s2 = __dadd_rn(s2, __dmul_rn(t, t));
-                    t = __dsub_rn(f2d_exact(a2.y), q1);
-                    s2 = __dadd_rn(s2, __dmul_rn(t, t));
-                    t = __dsub_rn(f2d_exact(a2.z), q2);
-                    s2 = __dadd_rn(s2, __dmul_rn(t, t));
-                    t = __dsub_rn(f2d_exact(a2.w), q3);
-                    s2 = __dadd_rn(s2, __dmul_rn(t, t));
-                }
-            }
             for (; i < A.d; i++) {
                 const double qd = f2d_exact(qs[i]);
                 const double t1 = __dsub_rn(f2d_exact(x1[i]), qd);
@@ -2206,9 +2126,9 @@ namespace {
 // single-query kernel otherwise.
 struct VerifyPlan {
     int nsm = 148;
-    int vWarps = 0, vPerSM = 1;   // single-query kernel
-    int vPerSMw = 1;              // its register-rich form (for batches that fit one wave of it)
+    int vWarps = 0, vPerSM = 1;   // a warp per query (k_verify)
     size_t vsmem = 0;
+    int64_t blockMax = 0;         // batches up to this size take a block per query (k_verify_block)
     int gvTR = 0, gvPerSM = 0;    // grouped kernel
     size_t gvSmem = 0;
     bool grouped = false;
@@ -2225,20 +2145,27 @@ pmlsh_status verify_plan(int ld, int KP, VerifyPlan &vp, bool bf16 = false)
     vp.vWarps = (int)std::min<size_t>(VW_MAXWARPS, (size_t)(227 * 1024) / vwarp);
     if (vp.vWarps < 1) return PMLSH_OK;
     vp.vsmem = (size_t)vp.vWarps * vwarp;
-    const void *kn = (const void *)k_verify<false, true>;
-    const void *kw = bf16 ? (const void *)k_verify<true, true> : (const void *)k_verify<true, false>;
+    const void *kn = (const void *)k_verify;
     PM_TRY(pm_allow_max_dyn_smem(kn));
-    PM_TRY(pm_allow_max_dyn_smem(kw));
     PM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&vp.vPerSM, kn, 32 * vp.vWarps, vp.vsmem));
-    PM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&vp.vPerSMw, kw, 32 * vp.vWarps, vp.vsmem));
     vp.vPerSM = std::max(1, vp.vPerSM);
-    vp.vPerSMw = std::max(1, vp.vPerSMw);
+    // A block per query up to the batch size where a warp per query keeps the GPU
+    // as busy: the longer the rows, the later, and never below the sixteen warps
+    // per SM that a block per query fills.  Measured, block against warp (us per
+    // launch, k = 10): 64 coordinates 209 / 247 at 2,500 queries, 396 / 332 at
+    // 5,000; 128 coordinates 597 / 739 at 5,000, 1,195 / 1,095 at 10,000; 256
+    // coordinates 1,507 / 1,745 at 10,000.  It reads FP32 rows in every precision
+    // mode (1,000 queries, d = 960: 568 us against 1,394 with the BF16 first pass of
+    // a warp per query).
+    if (vb_smem_bytes(ld, KP) <= (size_t)pm_max_smem_optin())
+        vp.blockMax = std::max<int64_t>(16 * vp.nsm, (int64_t)vp.nsm * ld * 2 / 5);
     vp.gvTR = gv_tile_rows(ld);
     vp.gvSmem = vp.gvTR > 0 ? gv_smem_bytes(ld, KP, vp.gvTR) : 0;
     if (vp.gvTR > 0 && vp.gvSmem <= (size_t)pm_max_smem_optin()) PM_TRY(gv_ctas_per_sm(vp.gvSmem, &vp.gvPerSM));
     const char *vsel = std::getenv("PMLSH_VERIFY");
     // (the grouped kernel has no BF16 first pass)
     vp.grouped = !bf16 && vp.gvPerSM > 0 && vsel && std::strcmp(vsel, "group") == 0;
+    if (vp.grouped) vp.blockMax = 0;
     return PMLSH_OK;
 }
 
@@ -2269,7 +2196,7 @@ void knn_work_needs(const pmlsh_index *ix, int64_t nq, int k, int precision,
     } else {
         const int64_t vw = std::max(1, vp.vWarps);
         const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((nq + vw - 1) / vw, (int64_t)vp.vPerSM * vp.nsm));
-        vscratch = grid * vw * L * 8;
+        vscratch = std::max<int64_t>(grid * vw, std::min<int64_t>(nq, VB_MAXGRID * vp.nsm)) * L * 8;
     }
     out = {
         {&KnnWork::Qd, nq * ld * 4}, {&KnnWork::qp64, nq * PM_MP * 8}, {&KnnWork::qp32, nq * PM_MP * 4},
@@ -2463,7 +2390,6 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
         return PMLSH_EINVAL;
     }
     const int nsm = vp.nsm, vWarps = vp.vWarps, vPerSM = vp.vPerSM, gvTR = vp.gvTR, gvPerSM = vp.gvPerSM;
-    const int vPerSMw = vp.vPerSMw;
     const size_t vsmem = vp.vsmem, gvSmem = vp.gvSmem;
     const bool grouped = vp.grouped;
 
@@ -2792,17 +2718,19 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
             ga.TR = gvTR;
             PM_TRY(gv_launch(ga, gGrid, gvSmem, st));
         } else {
-            // a batch that one wave of the register-rich form holds takes it
-            // (more loads in flight per lane; resident warps do not limit it)
-            const bool wide = na <= vPerSMw * nsm * vWarps;
-            const int vGrid = std::max(1, std::min((na + vWarps - 1) / vWarps, (wide ? vPerSMw : vPerSM) * nsm));
-            int2 *vLists = grow<int2>(w.partD, (size_t)vGrid * vWarps * L, s);
+            // a block per query (eight warps while one wave of two blocks per SM
+            // holds the batch, else four), or a warp per query
+            const bool vblock = na <= vp.blockMax;
+            const int vbW = na <= 2 * nsm ? 8 : 4;
+            const int vGrid = vblock ? std::min(na, 16 / vbW * nsm)
+                                     : std::max(1, std::min((na + vWarps - 1) / vWarps, vPerSM * nsm));
+            int2 *vLists = grow<int2>(w.partD, (size_t)vGrid * (vblock ? 1 : vWarps) * L, s);
             if (s != PMLSH_OK) return s;
             VwArgs va;
             va.act = act; va.na = na; va.thr = thr; va.qp32 = qp32; va.qpiv = qpiv; va.s = ix->s;
             va.meta = ix->leafMeta; va.L = L; va.O32 = ix->O32; va.X = ix->X; va.Qd = Qd;
             va.ld = ld; va.d = d; va.leafMu = ix->leafMu; va.leafRx = ix->leafRx; va.chunkOff = ix->chunkOff;
-            va.leafChunk = ix->leafChunk; va.chunkMu = ix->chunkMu; va.chunkRx = ix->chunkRx; va.KP = KP; va.k = k;
+            va.leafOff = ix->leafOff; va.leafChunk = ix->leafChunk; va.chunkMu = ix->chunkMu; va.chunkRx = ix->chunkRx; va.KP = KP; va.k = k;
             va.inN = inN; va.inPos = inPos; va.perm = ix->perm; va.outIds = oIds; va.outD = oD; va.outErr = oE;
             va.dk = dk; va.fp64cnt = fpc; va.nverOut = nverD; va.nleafOut = nverD + na; va.errFlag = errFlag;
             va.workCtr = nverD + 2 * na; va.dbg = nverD + 2 * na + 1; va.n = n; va.lists = vLists;
@@ -2817,12 +2745,10 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
             va.rowErr = ix->rowErr;
             va.redo = redoD;
             if (bf16v) PM_CUDA(cudaMemsetAsync(redoD, 0, na * sizeof(int), st));
-            if (wide && bf16v)
-                PM_LAUNCH("k_verify", st, k_verify<true, true><<<vGrid, 32 * vWarps, vsmem, st>>>(va));
-            else if (wide)
-                PM_LAUNCH("k_verify", st, k_verify<true, false><<<vGrid, 32 * vWarps, vsmem, st>>>(va));
+            if (vblock)
+                PM_TRY(vb_launch(va, vbW, vGrid, st));
             else
-                PM_LAUNCH("k_verify", st, k_verify<false, true><<<vGrid, 32 * vWarps, vsmem, st>>>(va));
+                PM_LAUNCH("k_verify", st, k_verify<<<vGrid, 32 * vWarps, vsmem, st>>>(va));
         }
         PM_CUDA(cudaGetLastError());
         if (stats) {

@@ -248,62 +248,6 @@ __device__ __forceinline__ float warp_d2x4(const float4 *__restrict__ q4, const 
     return __shfl_sync(VW_FULL, keep, ((lane & 7) << 2) | (lane >> 3));
 }
 
-// warp_d2x4 with two of its eight-row groups in flight at once (for kernels
-// with registers to spare): sixteen 16-byte loads per lane are issued
-// together, halving the dependent load rounds again; the same sums per row.
-__device__ __forceinline__ float warp_d2x4w(const float4 *__restrict__ q4, const float *p, int nf4, int lane)
-{
-    const int grp = lane >> 2, g = lane & 3;
-    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    float keep = 0.f;
-#pragma unroll 1
-    for (int j = 0; j < 4; j += 2) {
-        const float4 *xa = (const float4 *)__shfl_sync(VW_FULL, (unsigned long long)p, grp + 8 * j);
-        const float4 *xb = (const float4 *)__shfl_sync(VW_FULL, (unsigned long long)p, grp + 8 * (j + 1));
-        unsigned long long accA = 0ull, accB = 0ull;
-        if (xa != nullptr || xb != nullptr) {
-            int t = g;
-            for (; t + 28 < nf4; t += 32) {
-                float4 a[8], b[8];
-#pragma unroll
-                for (int u = 0; u < 8; u++) {
-                    a[u] = xa != nullptr ? __ldg(xa + t + 4 * u) : zero;
-                    b[u] = xb != nullptr ? __ldg(xb + t + 4 * u) : zero;
-                }
-#pragma unroll
-                for (int u = 0; u < 8; u++) {
-                    const float4 qv = q4[t + 4 * u];
-                    const unsigned long long q0 = f32x2_pack(qv.x, qv.y), q1 = f32x2_pack(qv.z, qv.w);
-                    f32x2_sqdiff_acc(accA, q0, f32x2_pack(a[u].x, a[u].y));
-                    f32x2_sqdiff_acc(accA, q1, f32x2_pack(a[u].z, a[u].w));
-                    f32x2_sqdiff_acc(accB, q0, f32x2_pack(b[u].x, b[u].y));
-                    f32x2_sqdiff_acc(accB, q1, f32x2_pack(b[u].z, b[u].w));
-                }
-            }
-            for (; t < nf4; t += 4) {
-                const float4 a = xa != nullptr ? __ldg(xa + t) : zero;
-                const float4 b = xb != nullptr ? __ldg(xb + t) : zero;
-                const float4 qv = q4[t];
-                const unsigned long long q0 = f32x2_pack(qv.x, qv.y), q1 = f32x2_pack(qv.z, qv.w);
-                f32x2_sqdiff_acc(accA, q0, f32x2_pack(a.x, a.y));
-                f32x2_sqdiff_acc(accA, q1, f32x2_pack(a.z, a.w));
-                f32x2_sqdiff_acc(accB, q0, f32x2_pack(b.x, b.y));
-                f32x2_sqdiff_acc(accB, q1, f32x2_pack(b.z, b.w));
-            }
-        }
-        float sa = __fadd_rn(__uint_as_float((unsigned)accA), __uint_as_float((unsigned)(accA >> 32)));
-        float sb = __fadd_rn(__uint_as_float((unsigned)accB), __uint_as_float((unsigned)(accB >> 32)));
-        sa = __fadd_rn(sa, __shfl_xor_sync(VW_FULL, sa, 1));
-        sb = __fadd_rn(sb, __shfl_xor_sync(VW_FULL, sb, 1));
-        sa = __fadd_rn(sa, __shfl_xor_sync(VW_FULL, sa, 2));
-        sb = __fadd_rn(sb, __shfl_xor_sync(VW_FULL, sb, 2));
-        if (g == j) keep = sa;
-        if (g == j + 1) keep = sb;
-    }
-    // lane (grp, g) holds row grp + 8 g; row v sits at lane 4 (v % 8) + v / 8
-    return __shfl_sync(VW_FULL, keep, ((lane & 7) << 2) | (lane >> 3));
-}
-
 // ||u - r~_v||^2 in FP32 of up to 32 BF16 rows r~_v (one per lane, length
 // ld; nullptr: none, the lane then gets 0) against the FP32 vector u in
 // shared memory: eight lanes share a row (16-byte loads of 8 BF16 values),
@@ -427,6 +371,70 @@ __device__ __forceinline__ float pd2_row(const float *__restrict__ o, const floa
     return s;
 }
 
+
+// ------------------------------------------------ verification (arguments)
+
+// Arguments of the verification kernels (k_verify in knn.cu, k_verify_block in
+// verify_block.cu).
+struct VwArgs {
+    const int32_t *act;
+    int na;
+    const Thr *thr;
+    const float *qp32, *qpiv;
+    int s;
+    const float *meta;
+    int64_t L;
+    const float *O32, *X, *Qd;
+    int ld, d;
+    const float *leafMu, *leafRx;
+    const int64_t *leafOff;     // [L+1]
+    const int64_t *chunkOff;
+    const int32_t *leafChunk;
+    const float *chunkMu, *chunkRx;
+    int KP, k;
+    const int *inN, *inPos;
+    const int32_t *perm;
+    int64_t *outIds;
+    float *outD, *outErr;
+    double *dk;
+    int *fp64cnt, *nverOut, *nleafOut, *errFlag;
+    int *workCtr;   // next entry of `order` to take (persistent warps)
+    const int *order;   // [na] active queries, the costliest first
+    int *dbg;       // [3]: site, value, query of the first failed index check
+    int64_t n;      // points
+    int2 *lists;    // [warps][L]: per-warp candidate leaves {leaf, lower bound bits}
+    const uint32_t *leafBits;   // [na][W32]: leaves Eq. 5 does not exclude (k_class)
+    const uint32_t *fullBits;   // [na][W32]: leaves k_class calls full (all members within the radius)
+    int W32;
+    const double *O64, *qp64;   // FP64 projected points and queries
+    const float *leafPmu;       // [L][PM_PCA] leaf centres along the principal directions
+    const float *qpca, *qnx;    // [nq][PM_PCA] queries along them, [nq] ||q|| (rounded up)
+    float muMax;                // max ||mu_l|| (rounded up)
+    int m;
+    int inlineBand;             // 1: decide FP32 band points in FP64 here (no exact count ran)
+    int nwork;                  // entries of `order` to take
+    // BF16 first pass (bf16 != 0): residual rows and their rounding bounds;
+    // a query whose first-pass bounds cannot settle its rerank set is
+    // marked in redo[a] and verified again without the first pass
+    int bf16;
+    const uint16_t *Xr;
+    const float *rowErr;
+    int *redo;
+};
+
+// Records the first failed index check (site, value, query) and the error flag;
+// false if the check fails.  Uses the kernel's A and a.
+#define VW_CHECK(cond, site, val)                                              \
+    (((cond)) ? true                                                           \
+              : (atomicCAS(&A.dbg[0], 0, (site)) == 0 ? (A.dbg[1] = (int)(val), A.dbg[2] = a, \
+                                                         atomicOr(A.errFlag, 1024), false)    \
+                                                      : (atomicOr(A.errFlag, 1024), false)))
+
+// Block verification (verify_block.cu): shared memory of one block of W warps,
+// and the launch on `grid` persistent blocks; W is 4 or 8, 16 / W blocks per SM.
+constexpr int VB_MAXGRID = 4;   // blocks per SM at most
+size_t vb_smem_bytes(int ld, int KP);
+pmlsh_status vb_launch(const VwArgs &A, int W, int grid, cudaStream_t st);
 
 // --------------------------------------------- grouped verification (host)
 
