@@ -37,85 +37,238 @@ using namespace pmk;
 
 // ------------------------------------------------------------ prep kernels
 
-// Routes each query down the bisection hierarchy to a leaf (locality key).
-__global__ void k_leaf_key(const float *__restrict__ qp32, int64_t nq, const int32_t *__restrict__ T,
-                           const float *__restrict__ V, unsigned int *__restrict__ key)
+// FP32 thresholds of the range test at projected radius R (FP64).
+__device__ __forceinline__ Thr make_thr(double R, double maxNorm, double qnorm)
 {
-    int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= nq) return;
-    int e = 0;
-    for (int guard = 0; guard < 4096; guard++) {
-        int l = T[e * 4 + 0];
-        if (l < 0) break;
-        const float *w = V + (int64_t)e * (PM_MP + 1);
-        float s = 0.f;
-        for (int j = 0; j < PM_MP; j++) s = fmaf(w[j], qp32[q * PM_MP + j], s);
-        e = s < w[PM_MP] ? l : T[e * 4 + 1];
-    }
-    key[q] = (unsigned int)T[e * 4 + 3];
+    const double eps = band_eps(R, maxNorm, qnorm);
+    Thr T;
+    T.R = R;
+    T.lo = R - eps > 0.0 ? __double2float_rd((R - eps) * (R - eps)) : -1.f;
+    T.hi = __double2float_ru((R + eps) * (R + eps));
+    T.lov = T.lo;
+    T.pad = 0.f;
+    return T;
 }
 
-// q norms (FP64 coordinates) and FP32 distances to the pivots.
-__global__ void k_query_aux(const double *__restrict__ qp64, const float *__restrict__ qp32,
-                            int64_t nq, const float *__restrict__ piv, int s,
-                            double *__restrict__ qnorm, float *__restrict__ qpiv)
-{
-    int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= nq) return;
-    double nn = 0.0;
-    for (int j = 0; j < PM_MP; j++) nn = fma(qp64[q * PM_MP + j], qp64[q * PM_MP + j], nn);
-    qnorm[q] = sqrt(nn);
-    for (int i = 0; i < PM_MAX_PIVOTS; i++)
-        qpiv[q * PM_MAX_PIVOTS + i] = i < s ? sqrtf(pm_pd2_32(qp32 + q * PM_MP, piv + i * PM_MP)) : 0.f;
-}
-
-// Query coordinates along the leaf centres' principal directions in FP32
-// (P rounded to FP32, sequential fma over the row; each coordinate within
-// (ld + 2) 2^-24 ||q|| of the exact one, which the verification's slack
-// covers) and ||q|| (FP64, rounded up to FP32).  One thread per query.
-__global__ void k_query_pca(const float *__restrict__ Qd, int64_t nq, int ld, const float *__restrict__ P,
-                            float *__restrict__ qpca, float *__restrict__ qnx)
-{
-    // one warp per query: lanes over the coordinates (16-byte loads), one
-    // partial sum per direction and lane, then a butterfly (any summation
-    // order is within the slack of the bound that uses P q)
-    const int lane = threadIdx.x & 31;
-    const int64_t q = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (q >= nq) return;   // warp-uniform
-    const float4 *x4 = (const float4 *)(Qd + q * ld);
-    const int nf4 = ld >> 2;
-    float acc[PM_PCA];
-#pragma unroll
-    for (int r = 0; r < PM_PCA; r++) acc[r] = 0.f;
-    double nn = 0.0;
-    for (int j4 = lane; j4 < nf4; j4 += 32) {
-        const float4 xv = x4[j4];
-        nn = fma((double)xv.x, (double)xv.x, nn);
-        nn = fma((double)xv.y, (double)xv.y, nn);
-        nn = fma((double)xv.z, (double)xv.z, nn);
-        nn = fma((double)xv.w, (double)xv.w, nn);
-#pragma unroll
-        for (int r = 0; r < PM_PCA; r++) {
-            const float4 pv = ((const float4 *)(P + (int64_t)r * ld))[j4];
-            acc[r] = __fmaf_rn(pv.x, xv.x, acc[r]);
-            acc[r] = __fmaf_rn(pv.y, xv.y, acc[r]);
-            acc[r] = __fmaf_rn(pv.z, xv.z, acc[r]);
-            acc[r] = __fmaf_rn(pv.w, xv.w, acc[r]);
+// Zeroes up to ZL_MAX int arrays (grid-stride over each).
+constexpr int ZL_MAX = 12;
+struct ZeroList {
+    int *p[ZL_MAX];
+    int64_t n[ZL_MAX];
+    int cnt = 0;
+    void add(int *ptr, int64_t count)
+    {
+        if (ptr && count > 0 && cnt < ZL_MAX) {
+            p[cnt] = ptr;
+            n[cnt] = count;
+            cnt++;
         }
     }
+};
+__device__ __forceinline__ void zero_arrays(const ZeroList &z)
+{
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int i = 0; i < z.cnt; i++)
+        for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < z.n[i]; e += stride) z.p[i][e] = 0;
+}
+
+__global__ void k_zero(ZeroList z) { zero_arrays(z); }
+
+// Everything a call computes once per query, eight queries per block, sixteen
+// lanes each: the padded row (Qd), q' = A q (lane j: the sequential FP64 fma over
+// the columns that k_project64 takes, so the coordinates are bit-identical), its
+// FP32 rounding and norm, the distances to the pivots, P q along the leaf centres'
+// principal directions (FP32; any order is within the (ld + 2) 2^-24 ||q|| that
+// the verification's slack covers), ||q|| rounded up, the first round's thresholds
+// (radius t r), the locality key (the hierarchy node met `depth` levels down), and
+// the zeros that the round's counters start from.
+// Bound by the FP64 chain of the projection, 64 cycles per column: A and the rows
+// are widened once per block and chunk into shared memory (a thread per row and
+// direction widened both operands of every fma), and the next chunk is fetched
+// while one is summed.  It stands for seven launches and two copies (1 query of 128
+// columns 20 us for 51, 1,000 of 960 79 us for 255, 10,000 of 128 80 us for 223).
+constexpr int QP_Q = 8, QP_CH = 64;
+struct PrepArgs {
+    const float *Q;         // rows, stride qs (device); may be Qd itself (then only the padding is written)
+    int64_t qs;
+    int64_t nq;
+    int ld, d, m, s;
+    const float *A, *P;     // [16][ld]
+    const float *piv;       // [PM_MAX_PIVOTS][16]
+    const int32_t *T;       // hierarchy
+    const float *V;
+    int depth;
+    double tr, maxNorm;     // t r of the first round
+    float *Qd;
+    double *qp64, *qnorm;
+    float *qp32, *qpiv, *qpca, *qnx;
+    unsigned int *key;
+    Thr *thr;               // by query
+    int32_t *order;         // or null: the identity order
+    ZeroList z;
+};
+
+__global__ void __launch_bounds__(16 * QP_Q)
+k_query_prep(PrepArgs a)
+{
+    __shared__ double sA[QP_CH][16], sX[QP_Q][QP_CH];
+    __shared__ float sP[QP_CH][16], sXf[QP_Q][QP_CH], sQ[QP_Q][16];
+    const int t = threadIdx.x, j = t & 15, qq = t >> 4;
+    const int64_t q0 = blockIdx.x * (int64_t)QP_Q, q = q0 + qq;
+    const unsigned half = 0xFFFFu << (t & 16);   // the query's sixteen lanes
+    const bool own = a.Q == a.Qd;
+    zero_arrays(a.z);
+    // this thread's share of a chunk: A and P rows j, columns 4 (t / 16) and 32 on;
+    // four row values
+    float4 fa[2], fp[2];
+    float fx[4];
+    auto fetch = [&](int c0) {
 #pragma unroll
-    for (int r = 0; r < PM_PCA; r++)
-        for (int o = 16; o; o >>= 1) acc[r] = __fadd_rn(acc[r], __shfl_xor_sync(0xffffffffu, acc[r], o));
-    for (int o = 16; o; o >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, o);
-    if (lane < PM_PCA) {
-        float v = acc[0];
+        for (int u = 0; u < 2; u++) {
+            const int c = c0 + 4 * (t >> 4) + 32 * u;
+            fa[u] = c < a.ld ? __ldg((const float4 *)(a.A + (int64_t)j * a.ld + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            fp[u] = c < a.ld ? __ldg((const float4 *)(a.P + (int64_t)j * a.ld + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
 #pragma unroll
-        for (int r = 1; r < PM_PCA; r++) v = lane == r ? acc[r] : v;
-        qpca[q * PM_PCA + lane] = v;
+        for (int u = 0; u < 4; u++) {
+            const int e = t + 16 * QP_Q * u, c = c0 + (e & (QP_CH - 1));
+            const int64_t r = q0 + e / QP_CH;
+            fx[u] = r < a.nq && c < a.d ? a.Q[r * a.qs + c] : 0.f;
+        }
+    };
+    double acc = 0.0, nn = 0.0;
+    float pca = 0.f;
+    fetch(0);
+    for (int c0 = 0; c0 < a.ld; c0 += QP_CH) {
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const int c = 4 * (t >> 4) + 32 * u;
+            sA[c][j] = pm_f2d_exact(fa[u].x);
+            sA[c + 1][j] = pm_f2d_exact(fa[u].y);
+            sA[c + 2][j] = pm_f2d_exact(fa[u].z);
+            sA[c + 3][j] = pm_f2d_exact(fa[u].w);
+            sP[c][j] = fp[u].x;
+            sP[c + 1][j] = fp[u].y;
+            sP[c + 2][j] = fp[u].z;
+            sP[c + 3][j] = fp[u].w;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int e = t + 16 * QP_Q * u, cc = e & (QP_CH - 1), c = c0 + cc;
+            const int64_t r = q0 + e / QP_CH;
+            sX[e / QP_CH][cc] = pm_f2d_exact(fx[u]);
+            sXf[e / QP_CH][cc] = fx[u];
+            if (r < a.nq && c < a.ld && (!own || c >= a.d)) a.Qd[r * a.ld + c] = fx[u];
+        }
+        __syncthreads();
+        if (c0 + QP_CH < a.ld) fetch(c0 + QP_CH);
+        const int nc = min(QP_CH, a.d - c0);
+        int c = 0;
+        for (; c + 8 <= nc; c += 8) {
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                acc = __fma_rn(sA[c + u][j], sX[qq][c + u], acc);
+                pca = __fmaf_rn(sP[c + u][j], sXf[qq][c + u], pca);
+            }
+        }
+        for (; c < nc; c++) {
+            acc = __fma_rn(sA[c][j], sX[qq][c], acc);
+            pca = __fmaf_rn(sP[c][j], sXf[qq][c], pca);
+        }
+        for (int x = j; x < nc; x += 16) nn = __fma_rn(sX[qq][x], sX[qq][x], nn);
     }
-    // ||q|| for the slack: the FP64 sum (any order, within 2^-45 relative of
-    // exact) rounded up to FP32 with a relative margin
-    if (lane == 0) qnx[q] = __double2float_ru(sqrt(nn) * (1.0 + 0x1.0p-40));
+    if (j >= a.m) acc = 0.0;
+    const float q32 = __double2float_rn(acc);
+    sQ[qq][j] = q32;
+    double n2 = acc * acc;
+    for (int o = 8; o; o >>= 1) {
+        nn += __shfl_xor_sync(half, nn, o);
+        n2 += __shfl_xor_sync(half, n2, o);
+    }
+    __syncwarp(half);
+    if (q >= a.nq) return;
+    a.qp64[q * PM_MP + j] = acc;
+    a.qp32[q * PM_MP + j] = q32;
+    a.qpca[q * PM_PCA + j] = pca;
+    if (j < PM_MAX_PIVOTS)
+        a.qpiv[q * PM_MAX_PIVOTS + j] = j < a.s ? sqrtf(pm_pd2_32(sQ[qq], a.piv + j * PM_MP)) : 0.f;
+    // ||q'|| (lane 0) and ||q|| (lane 1; the FP64 sum, within 2^-45 relative of
+    // exact, rounded up to FP32 with a relative margin)
+    const double root = sqrt(j == 0 ? n2 : nn);
+    if (j == 1) a.qnx[q] = __double2float_ru(root * (1.0 + 0x1.0p-40));
+    if (j == 0) {
+        a.qnorm[q] = root;
+        a.thr[q] = make_thr(a.tr, a.maxNorm, root);
+        if (a.order) a.order[q] = (int32_t)q;
+    }
+    // locality key: down the bisection hierarchy, the sixteen lanes taking a
+    // node's hyperplane together
+    int e = 0;
+    for (int lv = 0; lv < a.depth; lv++) {
+        const int4 nd = __ldg((const int4 *)a.T + e);   // left, right, -, first leaf
+        if (nd.x < 0) break;
+        const float *w = a.V + (int64_t)e * (PM_MP + 1);
+        const float th = __ldg(w + PM_MP);
+        float sum = __ldg(w + j) * q32;
+        for (int o = 8; o; o >>= 1) sum += __shfl_xor_sync(half, sum, o);
+        e = sum < th ? nd.x : nd.y;
+    }
+    if (j == 0 && a.depth > 0) a.key[q] = (unsigned int)a.T[e * 4 + 3];
+}
+
+// Locality order by one block: counting sort of the queries by their key (a leaf
+// number; mul: 2^32 OB_BINS / L where there are more leaves than bins, else 0),
+// with the first round's thresholds moved along.  10,000 queries over 15,096 leaves: 31 us for a memset and three kernels of
+// 38 us together; 200 queries 6 us.
+constexpr int OB_BINS = 4096;
+__global__ void __launch_bounds__(1024)
+k_order(const unsigned int *__restrict__ key, int64_t nq, unsigned int mul, const Thr *__restrict__ thrQ,
+        int32_t *__restrict__ order, Thr *__restrict__ thr)
+{
+    __shared__ int h[OB_BINS];
+    __shared__ int ws[32];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    constexpr int PER = OB_BINS / 1024;
+    for (int i = t; i < OB_BINS; i += 1024) h[i] = 0;
+    __syncthreads();
+    auto bin = [&](int64_t q) { return min(mul ? (int)__umulhi(key[q], mul) : (int)key[q], OB_BINS - 1); };
+    for (int64_t q = t; q < nq; q += 1024) atomicAdd(&h[bin(q)], 1);
+    __syncthreads();
+    int v[PER], sum = 0;
+#pragma unroll
+    for (int i = 0; i < PER; i++) {
+        v[i] = h[t * PER + i];
+        sum += v[i];
+    }
+    int incl = sum;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += x;
+    }
+    if (lane == 31) ws[w] = incl;
+    __syncthreads();
+    if (w == 0) {
+        int x = ws[lane], xi = x;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, xi, o);
+            if (lane >= o) xi += y;
+        }
+        ws[lane] = xi - x;
+    }
+    __syncthreads();
+    int run = ws[w] + incl - sum;
+#pragma unroll
+    for (int i = 0; i < PER; i++) {
+        h[t * PER + i] = run;
+        run += v[i];
+    }
+    __syncthreads();
+    for (int64_t q = t; q < nq; q += 1024) {
+        const int at = atomicAdd(&h[bin(q)], 1);
+        order[at] = (int32_t)q;
+        thr[at] = thrQ[q];
+    }
 }
 
 __global__ void k_thresholds(const int32_t *__restrict__ act, int na, const double *__restrict__ r,
@@ -125,15 +278,7 @@ __global__ void k_thresholds(const int32_t *__restrict__ act, int na, const doub
     int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= na) return;
     int q = act[a];
-    double R = t * r[q];
-    double eps = band_eps(R, maxNorm, qnorm[q]);
-    Thr T;
-    T.R = R;
-    T.lo = R - eps > 0.0 ? __double2float_rd((R - eps) * (R - eps)) : -1.f;
-    T.hi = __double2float_ru((R + eps) * (R + eps));
-    T.lov = T.lo;
-    T.pad = 0.f;
-    thr[a] = T;
+    thr[a] = make_thr(t * r[q], maxNorm, qnorm[q]);
 }
 
 // ------------------------------------------------------------ range round
@@ -597,29 +742,6 @@ __global__ void k_band64(const int *__restrict__ bandN, int bandCap, const int *
             else atomicOr(errFlag, 2);
         }
     }
-}
-
-// Zeroes up to ZL_MAX int arrays in one launch (grid-stride over each).
-constexpr int ZL_MAX = 12;
-struct ZeroList {
-    int *p[ZL_MAX];
-    int64_t n[ZL_MAX];
-    int cnt = 0;
-    void add(int *ptr, int64_t count)
-    {
-        if (ptr && count > 0 && cnt < ZL_MAX) {
-            p[cnt] = ptr;
-            n[cnt] = count;
-            cnt++;
-        }
-    }
-};
-
-__global__ void k_zero(ZeroList z)
-{
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int i = 0; i < z.cnt; i++)
-        for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < z.n[i]; e += stride) z.p[i][e] = 0;
 }
 
 // --------------------------------------------------------- budget (rule 2)
@@ -2071,45 +2193,6 @@ __global__ void k_gather_sub(const int *__restrict__ idx, int n2, const int32_t 
     thr2[i] = thr[idx[i]];
 }
 
-// Locality order: counting sort of queries by leaf key.
-__global__ void k_hist(const unsigned int *__restrict__ key, int64_t nq, int *__restrict__ h)
-{
-    int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q < nq) atomicAdd(&h[key[q]], 1);
-}
-
-__global__ void k_scan_single(int *__restrict__ h, int64_t L)
-{
-    // one block: exclusive scan of L counters, 1024 at a time
-    __shared__ int carry;
-    __shared__ int buf[1024];
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    for (int64_t b0 = 0; b0 < L; b0 += 1024) {
-        int64_t i = b0 + threadIdx.x;
-        int v = i < L ? h[i] : 0;
-        buf[threadIdx.x] = v;
-        __syncthreads();
-        for (int o = 1; o < 1024; o <<= 1) {
-            int t = threadIdx.x >= o ? buf[threadIdx.x - o] : 0;
-            __syncthreads();
-            buf[threadIdx.x] += t;
-            __syncthreads();
-        }
-        if (i < L) h[i] = carry + buf[threadIdx.x] - v;
-        __syncthreads();
-        if (threadIdx.x == 1023) carry += buf[1023];
-        __syncthreads();
-    }
-}
-
-__global__ void k_scatter_order(const unsigned int *__restrict__ key, int64_t nq, int *__restrict__ h,
-                                int32_t *__restrict__ order)
-{
-    int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q < nq) order[atomicAdd(&h[key[q]], 1)] = (int32_t)q;
-}
-
 template <class T> T *grow(DevBuf &b, size_t count, pmlsh_status &st)
 {
     if (st != PMLSH_OK) return nullptr;
@@ -2201,7 +2284,7 @@ void knn_work_needs(const pmlsh_index *ix, int64_t nq, int k, int precision,
     out = {
         {&KnnWork::Qd, nq * ld * 4}, {&KnnWork::qp64, nq * PM_MP * 8}, {&KnnWork::qp32, nq * PM_MP * 4},
         {&KnnWork::qnorm, nq * 8}, {&KnnWork::qpiv, nq * PM_MAX_PIVOTS * 4}, {&KnnWork::keys, nq * 4},
-        {&KnnWork::order, nq * 4}, {&KnnWork::qpca, nq * (PM_PCA + 1) * 4}, {&KnnWork::keys2, (L + 1) * 4},
+        {&KnnWork::order, nq * 4}, {&KnnWork::qpca, nq * (PM_PCA + 1) * 4},
         {&KnnWork::qstate, nq * 8}, {&KnnWork::outIds, nq * k * 8}, {&KnnWork::outD64, nq * k * 4},
         {&KnnWork::outErr, nq * k * 4}, {&KnnWork::active, nq * 4}, {&KnnWork::thr, nq * (int64_t)sizeof(Thr)},
         {&KnnWork::cntSure, nq * 4}, {&KnnWork::cntBand, nq * 4}, {&KnnWork::cntPart, nq * 4},
@@ -2316,7 +2399,6 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
     int32_t *order = grow<int32_t>(w.order, nq, s);
     float *qpca = grow<float>(w.qpca, (size_t)nq * (PM_PCA + 1), s);
     float *qnx = qpca + (size_t)nq * PM_PCA;
-    int *hist = grow<int>(w.keys2, L + 1, s);
     double *rq = grow<double>(w.qstate, nq, s);
     // results go straight to the caller's arrays when those are in device
     // memory, else to scratch copied out at the end
@@ -2326,16 +2408,6 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
     float *oD = ddev ? dists : grow<float>(w.outD64, (size_t)nq * k, s);
     float *oE = edev ? err : grow<float>(w.outErr, (size_t)nq * k, s);
     if (s != PMLSH_OK) return s;
-    PM_TRY(pm_project_rows(ix, Q, nq, Qd, qp64, qp32, PM_MP, st));
-    const unsigned gq = (unsigned)((nq + 255) / 256);
-    PM_LAUNCH("k_query_aux", st, k_query_aux<<<gq, 256, 0, st>>>(qp64, qp32, nq, ix->piv32, ix->s, qnorm, qpiv));
-    PM_LAUNCH("k_query_pca", st, k_query_pca<<<(unsigned)((nq + 7) / 8), 256, 0, st>>>(Qd, nq, ld, ix->pcaP32, qpca, qnx));
-    PM_LAUNCH("k_leaf_key", st, k_leaf_key<<<gq, 256, 0, st>>>(qp32, nq, ix->treeI, ix->treeV, key));
-    PM_CUDA(cudaMemsetAsync(hist, 0, (L + 1) * sizeof(int), st));
-    PM_LAUNCH("k_hist", st, k_hist<<<gq, 256, 0, st>>>(key, nq, hist));
-    PM_LAUNCH("k_scan_single", st, k_scan_single<<<1, 1024, 0, st>>>(hist, L + 1));
-    PM_LAUNCH("k_scatter_order", st, k_scatter_order<<<gq, 256, 0, st>>>(key, nq, hist, order));
-    PM_CUDA(cudaGetLastError());
     // pinned staging of the per-round decisions: order [nq], bounds [2 nq],
     // verification outputs (k-th distance [nq] f64, fp64/verified/leaves
     // counts [3 nq], error flag)
@@ -2348,7 +2420,6 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
     int32_t *stOrder = (int32_t *)(stTight + nq);
     int *stHs = stOrder + nq, *stHp = stHs + nq, *stFp = stHp + nq, *stNv = stFp + nq, *stNl = stNv + nq,
         *stVo = stNl + nq, *stRedo = stVo + nq, *stList = stRedo + nq, *stErr = stList + nq;
-    PM_CUDA(cudaMemcpyAsync(stOrder, order, nq * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     std::vector<int32_t> orderH;   // host copy, read after the first round's sync
 
     // host round state
@@ -2357,8 +2428,6 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
     std::vector<int64_t> ncand(nq, 0), nver(nq, 0);
     std::vector<int32_t> nleaf(nq, 0), fallback(nq, 0);
     std::vector<char> done(nq, 0);
-    std::memcpy(stR, r.data(), nq * sizeof(double));
-    PM_CUDA(cudaMemcpyAsync(rq, stR, nq * sizeof(double), cudaMemcpyHostToDevice, st));
 
     const int bandCap = 1 << 20;
     int *actBuf = grow<int32_t>(w.active, nq, s);
@@ -2402,6 +2471,53 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
     int2 *recheck = tensor ? grow<int2>(w.recheck, recheckCap, s) : nullptr;
     if (s != PMLSH_OK) return s;
 
+    // one block's queries need no locality order; a deeper key than the blocks can
+    // use would only cost its levels
+    const int qbt = tensor ? TC_QN : QB;
+    const int64_t nblk = (nq + qbt - 1) / qbt;
+    const bool sorted = nblk > 1;
+    {
+        int *blkCnt = grow<int>(w.blkCnt, nblk, s);
+        Thr *thrQ = sorted ? grow<Thr>(w.subThr, nq, s) : thr;   // by query, until the order is known
+        if (s != PMLSH_OK) return s;
+        const bool qdev = pm_is_device_ptr(Q);
+        if (!qdev)
+            PM_CUDA(cudaMemcpy2DAsync(Qd, ld * sizeof(float), Q, d * sizeof(float), d * sizeof(float), nq,
+                                      cudaMemcpyHostToDevice, st));
+        PrepArgs pa;
+        pa.Q = qdev ? Q : Qd;
+        pa.qs = qdev ? d : ld;
+        pa.nq = nq; pa.ld = ld; pa.d = d; pa.m = m; pa.s = ix->s;
+        pa.A = ix->A32; pa.P = ix->pcaP32; pa.piv = ix->piv32; pa.T = ix->treeI; pa.V = ix->treeV;
+        pa.depth = 0;
+        if (sorted) {
+            pa.depth = 6;
+            while (((int64_t)1 << (pa.depth - 6)) < nblk) pa.depth++;
+        }
+        pa.tr = t * rmin; pa.maxNorm = ix->maxNorm;
+        pa.Qd = Qd; pa.qp64 = qp64; pa.qnorm = qnorm; pa.qp32 = qp32; pa.qpiv = qpiv; pa.qpca = qpca; pa.qnx = qnx;
+        pa.key = key; pa.thr = thrQ; pa.order = sorted ? nullptr : order;
+        // the round's counters start at zero (class_phase's list, and the error and
+        // list counters after fpc's per-query part)
+        pa.z.add(blkCnt, nblk);
+        pa.z.add(cntSure, nq);
+        pa.z.add(cntPart, nq);
+        pa.z.add(cntBand, nq);
+        pa.z.add(inTrue, nq);
+        pa.z.add(inN, nq);
+        pa.z.add(fpc, nq + 8);
+        if (stats == nullptr) pa.z.add((int *)cntTight, 2 * nq);
+        PM_LAUNCH("k_query_prep", st, k_query_prep<<<(unsigned)((nq + QP_Q - 1) / QP_Q), 16 * QP_Q, 0, st>>>(pa));
+        if (sorted) {
+            const unsigned int mul = L > OB_BINS ? (unsigned int)(((uint64_t)OB_BINS << 32) / (uint64_t)L) : 0u;
+            PM_LAUNCH("k_order", st, k_order<<<1, 1024, 0, st>>>(key, nq, mul, thrQ, order, thr));
+            PM_CUDA(cudaMemcpyAsync(stOrder, order, nq * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+        } else {
+            for (int64_t q = 0; q < nq; q++) stOrder[q] = (int32_t)q;
+        }
+        PM_CUDA(cudaGetLastError());
+    }
+
     std::vector<int32_t> actH;
     actH.reserve(nq);
     for (int round = 0; round < 100000; round++) {
@@ -2417,8 +2533,8 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
             if (na == 0) break;
             std::memcpy(stList, actH.data(), na * sizeof(int32_t));
             PM_CUDA(cudaMemcpyAsync(act, stList, na * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+            PM_LAUNCH("k_thresholds", st, k_thresholds<<<(na + 255) / 256, 256, 0, st>>>(act, na, rq, t, ix->maxNorm, qnorm, thr));
         }
-        PM_LAUNCH("k_thresholds", st, k_thresholds<<<(na + 255) / 256, 256, 0, st>>>(act, na, rq, t, ix->maxNorm, qnorm, thr));
         // leaf classification (Eq. 5): bounds of |S_i|, leaf lists with the
         // masks of partially covering queries, per-query leaf bit sets.  The
         // phases run on the active batch or on a gathered sub-batch (io).
@@ -2433,7 +2549,7 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
             const int32_t *amb;   // a gathered sub-batch: its rows in the batch (lists from the batch's bits)
         };
         const int64_t Tdec = std::min<int64_t>(B, n);
-        auto class_phase = [&](bool tc, const CountIO &io, ZeroList z) -> pmlsh_status {
+        auto class_phase = [&](bool tc, const CountIO &io, ZeroList z, bool zeroed) -> pmlsh_status {
             const int nlist = tc ? (io.na + TC_QN - 1) / TC_QN : (io.na + QB - 1) / QB;
             const int mwords = tc ? TC_MW : QB / 32;
             pmlsh_status s2 = PMLSH_OK;
@@ -2452,7 +2568,8 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
             z.add(bandN, 1);
             z.add(recheckN, 1);
             z.add((int *)io.cntTight, io.cntTight ? 2 * io.na : 0);
-            PM_LAUNCH("k_zero", st, k_zero<<<2 * nsm, 256, 0, st>>>(z));
+            // (round 0's were zeroed beside the queries' preparation)
+            if (!zeroed) PM_LAUNCH("k_zero", st, k_zero<<<2 * nsm, 256, 0, st>>>(z));
             if (io.amb) {
                 // a sub-batch: its block lists from the batch's leaf bits
                 const int64_t nch = (W32 + 7) / 8;
@@ -2534,20 +2651,22 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
             int hN[3] = {0, 0, 0};   // bandN, errFlag, recheckN
             for (int pass = 0; pass < 2; pass++) {
                 const bool tcp = tensor && pass == 0;
-                if (pass == 1) PM_TRY(class_phase(false, io, ZeroList()));
+                if (pass == 1) PM_TRY(class_phase(false, io, ZeroList(), false));
                 PM_TRY(point_count(tcp, io));
                 PM_LAUNCH("k_band64", st, k_band64<<<2 * nsm, 256, 0, st>>>(bandN, bandCap, bandA, bandPos, io.act,
                                                        io.thr, ix->O64, qp64, m, io.inTrue, io.inN, io.inPos,
                                                        io.fpc, errFlag));
                 PM_CUDA(cudaGetLastError());
-                es.resize(io.na);
-                eb.resize(io.na);
-                ein.resize(io.na);
-                PM_CUDA(cudaMemcpyAsync(hN, bandN, 3 * sizeof(int), cudaMemcpyDeviceToHost, st));
-                PM_CUDA(cudaMemcpyAsync(es.data(), io.cntSure, io.na * sizeof(int), cudaMemcpyDeviceToHost, st));
-                PM_CUDA(cudaMemcpyAsync(eb.data(), io.cntBand, io.na * sizeof(int), cudaMemcpyDeviceToHost, st));
-                PM_CUDA(cudaMemcpyAsync(ein.data(), io.inTrue, io.na * sizeof(int), cudaMemcpyDeviceToHost, st));
+                // (pinned staging: copies to pageable memory would each wait)
+                PM_CUDA(cudaMemcpyAsync(stErr, bandN, 3 * sizeof(int), cudaMemcpyDeviceToHost, st));
+                PM_CUDA(cudaMemcpyAsync(stHs, io.cntSure, io.na * sizeof(int), cudaMemcpyDeviceToHost, st));
+                PM_CUDA(cudaMemcpyAsync(stHp, io.cntBand, io.na * sizeof(int), cudaMemcpyDeviceToHost, st));
+                PM_CUDA(cudaMemcpyAsync(stNl, io.inTrue, io.na * sizeof(int), cudaMemcpyDeviceToHost, st));
                 PM_CUDA(cudaStreamSynchronize(st));
+                es.assign(stHs, stHs + io.na);
+                eb.assign(stHp, stHp + io.na);
+                ein.assign(stNl, stNl + io.na);
+                for (int i = 0; i < 3; i++) hN[i] = stErr[i];
                 if (!(tcp && hN[2] > recheckCap)) break;
             }
             if (hN[0] > bandCap) {
@@ -2563,20 +2682,21 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
             // after them (fpc [nq + 8]) start at zero
             ZeroList z;
             z.add(fpc, nq + 8);
-            PM_TRY(class_phase(tensor, full, z));
+            PM_TRY(class_phase(tensor, full, z, round == 0));
         }
-        std::vector<int> hs(na), hp(na), hb(na, 0), hin(na, 0);
+        std::vector<int> hs, hp, hb, hin;
         std::vector<int2> ht;
-        PM_CUDA(cudaMemcpyAsync(stHs, cntSure, na * sizeof(int), cudaMemcpyDeviceToHost, st));
-        PM_CUDA(cudaMemcpyAsync(stHp, cntPart, na * sizeof(int), cudaMemcpyDeviceToHost, st));
-        if (full.cntTight) PM_CUDA(cudaMemcpyAsync(stTight, cntTight, na * sizeof(int2), cudaMemcpyDeviceToHost, st));
-        PM_CUDA(cudaStreamSynchronize(st));
-        std::memcpy(hs.data(), stHs, na * sizeof(int));
-        std::memcpy(hp.data(), stHp, na * sizeof(int));
-        if (full.cntTight) ht.assign(stTight, stTight + na);
-        if (round == 0) {
-            orderH.assign(stOrder, stOrder + nq);
-            actH.assign(stOrder, stOrder + nq);
+        const bool needExact = stats != nullptr;
+        if (!needExact) {
+            PM_CUDA(cudaMemcpyAsync(stHs, cntSure, na * sizeof(int), cudaMemcpyDeviceToHost, st));
+            PM_CUDA(cudaMemcpyAsync(stHp, cntPart, na * sizeof(int), cudaMemcpyDeviceToHost, st));
+            if (full.cntTight) PM_CUDA(cudaMemcpyAsync(stTight, cntTight, na * sizeof(int2), cudaMemcpyDeviceToHost, st));
+            PM_CUDA(cudaStreamSynchronize(st));
+            hs.assign(stHs, stHs + na);
+            hp.assign(stHp, stHp + na);
+            hb.assign(na, 0);
+            hin.assign(na, 0);
+            if (full.cntTight) ht.assign(stTight, stTight + na);
         }
         // The decisions of Algorithm 2 compare |S_i| only with min(B, n)
         // (rule 2: |S_i| >= B; rule 3: |S_i| = n).  Whole-leaf counts bound
@@ -2585,13 +2705,17 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
         // (|C| is one of them), else only for the queries whose bounds
         // straddle min(B, n); for the rest the verification decides the FP32
         // band points it meets in FP64 itself.
-        const bool needExact = stats != nullptr;
         // hb: points with FP32 d'^2 <= hi beyond the sure ones (the budget
         // selection's capacity); without the exact count, the partial leaves
         std::vector<int32_t> ambH;
         if (needExact) {
             PM_TRY(exact_count(full, hs, hb, hin));
-        } else {
+        }
+        if (round == 0) {   // (the order is on the host since the wait above)
+            orderH.assign(stOrder, stOrder + nq);
+            actH.assign(stOrder, stOrder + nq);
+        }
+        if (!needExact) {
             // the bounds of |S_i| from whole leaves, tightened by the partial
             // leaves' radial profiles; a query whose lower bound reaches
             // min(B, n) counts as min(B, n) (rule 2, or rule 3 when n < B)
@@ -2645,7 +2769,7 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
             PM_LAUNCH("k_gather_sub", st, k_gather_sub<<<(na2 + 255) / 256, 256, 0, st>>>(amb, na2, act, thr, act2, thr2));
             const CountIO subIO{act2, na2, thr2, s2Sure, s2Part, s2Band, s2In, s2InN, s2InPos, s2Fp, bits2, nullptr,
                                 nullptr, amb};
-            PM_TRY(class_phase(tensor, subIO, ZeroList()));   // zeroes inTrue, inN, fp64 of the sub-batch
+            PM_TRY(class_phase(tensor, subIO, ZeroList(), false));   // zeroes inTrue, inN, fp64 of the sub-batch
             std::vector<int> es, eb, ein;
             PM_TRY(exact_count(subIO, es, eb, ein));
             for (int i = 0; i < na2; i++) {
