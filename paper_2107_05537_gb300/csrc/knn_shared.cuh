@@ -332,10 +332,6 @@ __device__ __forceinline__ float warp_d2_bf16x4(const float *__restrict__ us, co
     return __shfl_sync(VW_FULL, keep, ((lane & 7) << 2) | (lane >> 3));
 }
 
-// FP32 -> FP64 re-encoded with integer operations (exact, equal to the
-// conversion instruction), so that the widening does not occupy the FP64
-// pipe; zeros are re-encoded too, subnormals, infinities and NaNs use the
-// conversion instruction.
 __device__ __forceinline__ double f2d_exact(float f) { return pm_f2d_exact(f); }
 
 // pm_dist64 (FP64 sequential sum of (x_i - y_i)^2, separate multiply and
