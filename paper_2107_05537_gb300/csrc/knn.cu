@@ -305,8 +305,11 @@ constexpr float CL_INV_HI = 1.0f / (1.f + SLACK) * (1.f - 1e-7f);   // <= 1 / (1
 // calls full, fullBits): thread qq of the CTA
 // holds query qq of the block (coordinates as packed pairs and its pivot
 // thresholds in registers) and the CTA walks its share of the leaves in tiles
-// of CQ_LT, reading each leaf record with loads that every lane of a warp
-// shares.  A thread keeps its whole-leaf and partial sizes and its leaf
+// of 32 NWD.  The leaf records come through shared memory, 32 at a time, the next
+// 32 copied (cp.async) while one set is tested: read directly, each record's load
+// latency stood in every warp's path (200 queries, 517 leaves: 130 us, 22 in tiles
+// of 32 leaves; 10,000 queries, 15,096 leaves: 514, 450).
+// A thread keeps its whole-leaf and partial sizes and its leaf
 // bit-set words in registers.  The centre test is the only work for a
 // (query, leaf) pair that it excludes; the pivot rings, the full-leaf test,
 // the counts and the ballot of the partial-leaf mask run only for a leaf
@@ -314,11 +317,24 @@ constexpr float CL_INV_HI = 1.0f / (1.f + SLACK) * (1.f - 1e-7f);   // <= 1 / (1
 // shared memory (double-buffered, one barrier per tile), where the tile's
 // partially covered leaves are listed.  Queries beyond the batch sit at
 // +1e18 on every coordinate, so the centre test excludes them.
-constexpr int CQ_LT = 256;   // leaves per tile: eight bit-set words (one 32-byte sector) per query
-// words per query in a leaf bit set: L bits padded to whole tiles
+// NWD = 8 writes a query's bits as whole 32-byte sectors; NWD = 1 cuts the leaves
+// into eight times as many tiles, for batches whose larger tiles leave SMs idle.
+constexpr int CQ_LT = 256;   // leaf bit sets are padded to whole tiles of 256 leaves (32-byte sectors)
+// words per query in a leaf bit set
 static inline int64_t pm_leaf_words(int64_t L) { return (L + CQ_LT - 1) / CQ_LT * (CQ_LT / 32); }
 
-template <int QBT>
+__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async8(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
+template <int QBT, int NWD>
 __global__ void __launch_bounds__(QBT, QBT == 256 ? 4 : 16)
 k_class(const int32_t *__restrict__ act, int na, const Thr *__restrict__ thr,
         const float *__restrict__ qp32, const float *__restrict__ qpiv, int s,
@@ -328,15 +344,28 @@ k_class(const int32_t *__restrict__ act, int na, const Thr *__restrict__ thr,
         uint32_t *__restrict__ fullBits)
 {
     constexpr int W = QBT / 32;   // warps = mask words per list entry
-    constexpr int NWD = CQ_LT / 32;   // bit-set words per query and tile
-    __shared__ uint32_t sM[2][CQ_LT][W];
+    constexpr int LT = 32 * NWD;  // leaves per tile
+    constexpr int NM = NWD == 1 ? 1 : 2;   // mask buffers
+    __shared__ __align__(16) float sMeta[2][32][PM_LEAF_STRIDE];
+    __shared__ int64_t sOff[2][33];
+    __shared__ uint32_t sM[NM][LT][W];
     __shared__ uint32_t sW[NWD][QBT];   // the thread's words of the tile, written out as whole sectors
     __shared__ uint32_t sF[NWD][QBT];   // the same for the whole-leaf bits
     const int b = blockIdx.y;
     const int a0 = b * QBT;
     const int nb = min(QBT, na - a0);
     const int t = threadIdx.x, lane = t & 31, wp = t >> 5;
-    for (int e = t; e < 2 * CQ_LT * W; e += QBT) (&sM[0][0][0])[e] = 0u;
+    for (int e = t; e < NM * LT * W; e += QBT) (&sM[0][0][0])[e] = 0u;
+    const int64_t nTiles = W32 / NWD;   // (the tiles past L write empty words)
+    // records [l0, l0 + 32) of the leaves into buffer v, by all threads
+    auto stage = [&](int v, int64_t l0) {
+        const int n = L - l0 < 32 ? (int)max((int64_t)0, L - l0) : 32;
+        const float4 *src = (const float4 *)(meta + l0 * PM_LEAF_STRIDE);
+        for (int e = t; e < n * (PM_LEAF_STRIDE / 4); e += QBT) cp_async16((float4 *)&sMeta[v][0][0] + e, src + e);
+        if (t <= n && n > 0) cp_async8(&sOff[v][t], off + l0 + t);
+        cp_async_commit();
+    };
+    if (blockIdx.x < nTiles) stage(0, (int64_t)blockIdx.x * LT);
 
     unsigned long long qv[PM_MP / 2];
     // per pivot: out if HR.max < lowT or HR.min > highT
@@ -373,35 +402,39 @@ k_class(const int32_t *__restrict__ act, int na, const Thr *__restrict__ thr,
             highT[i] = INFINITY;
         }
     }
-    __syncthreads();
     int sure = 0, part = 0;
-    const int64_t nTiles = (L + CQ_LT - 1) / CQ_LT;
-    int buf = 0;
-    for (int64_t tile = blockIdx.x; tile < nTiles; tile += gridDim.x, buf ^= 1) {
-        const int64_t l0 = tile * CQ_LT;
-        const int nl = L - l0 < CQ_LT ? (int)(L - l0) : CQ_LT;
+    int buf = 0, v = 0;
+    for (int64_t tile = blockIdx.x; tile < nTiles; tile += gridDim.x, buf ^= NM - 1) {
+        const int64_t l0 = tile * LT;
+        const int nl = L - l0 < LT ? (int)max((int64_t)0, L - l0) : LT;
 #pragma unroll 1
-        for (int w4 = 0; w4 < NWD; w4++) {
+        for (int w4 = 0; w4 < NWD; w4++, v ^= 1) {
             uint32_t bits = 0u, fbits = 0u;
             const int jn = min(32, nl - w4 * 32);
+            // this set of records is here; the next one (of this tile or of the
+            // CTA's next) is copied meanwhile
+            cp_async_wait_all();
+            __syncthreads();
+            if (w4 + 1 < NWD) stage(v ^ 1, l0 + 32 * (w4 + 1));
+            else if (tile + gridDim.x < nTiles) stage(v ^ 1, (tile + gridDim.x) * LT);
 #pragma unroll 2
             for (int jj = 0; jj < jn; jj++) {
                 const int j = w4 * 32 + jj;
-                const float *M = meta + (l0 + j) * PM_LEAF_STRIDE;
+                const float *M = sMeta[v][jj];
                 const float4 *c4 = (const float4 *)M;
                 unsigned long long acc0 = 0ull, acc1 = 0ull;
 #pragma unroll
                 for (int j4 = 0; j4 < PM_MP / 4; j4 += 2) {
-                    const float4 v = __ldg(c4 + j4), u = __ldg(c4 + j4 + 1);
-                    f32x2_sqdiff_acc(acc0, qv[2 * j4], f32x2_pack(v.x, v.y));
-                    f32x2_sqdiff_acc(acc1, qv[2 * j4 + 1], f32x2_pack(v.z, v.w));
+                    const float4 x = c4[j4], u = c4[j4 + 1];
+                    f32x2_sqdiff_acc(acc0, qv[2 * j4], f32x2_pack(x.x, x.y));
+                    f32x2_sqdiff_acc(acc1, qv[2 * j4 + 1], f32x2_pack(x.z, x.w));
                     f32x2_sqdiff_acc(acc0, qv[2 * j4 + 2], f32x2_pack(u.x, u.y));
                     f32x2_sqdiff_acc(acc1, qv[2 * j4 + 3], f32x2_pack(u.z, u.w));
                 }
                 unsigned long long acc;
                 asm("add.rn.f32x2 %0, %1, %2;" : "=l"(acc) : "l"(acc0), "l"(acc1));
                 // out: sqrt(d^2) (1 - SLACK) - r > ro, i.e. d^2 > ((ro + r) / (1 - SLACK))^2
-                const float rr = __ldg(M + 16);
+                const float rr = M[16];
                 const float lo = __fadd_rd(__uint_as_float((unsigned)acc), __uint_as_float((unsigned)(acc >> 32)));
                 const float tb = __fadd_ru(roL, __fmul_ru(rr, CL_INV_LO));
                 const bool in = !(lo > __fmul_ru(tb, tb));
@@ -410,7 +443,7 @@ k_class(const int32_t *__restrict__ act, int na, const Thr *__restrict__ thr,
                     unsigned char c = CL_OUT;
                     if (in) {
                         const float4 *h4 = (const float4 *)(M + 24);   // HR.min [8], HR.max [8]
-                        const float4 n0 = __ldg(h4), n1 = __ldg(h4 + 1), x0 = __ldg(h4 + 2), x1 = __ldg(h4 + 3);
+                        const float4 n0 = h4[0], n1 = h4[1], x0 = h4[2], x1 = h4[3];
                         const bool out = x0.x < lowT[0] || x0.y < lowT[1] || x0.z < lowT[2] || x0.w < lowT[3] ||
                                          x1.x < lowT[4] || x1.y < lowT[5] || x1.z < lowT[6] || x1.w < lowT[7] ||
                                          n0.x > highT[0] || n0.y > highT[1] || n0.z > highT[2] || n0.w > highT[3] ||
@@ -421,7 +454,7 @@ k_class(const int32_t *__restrict__ act, int na, const Thr *__restrict__ thr,
                             const float hi = __fadd_ru(__uint_as_float((unsigned)acc), __uint_as_float((unsigned)(acc >> 32)));
                             const float f = __fmul_rd(__fsub_rd(rinLo, rr), CL_INV_HI);
                             if (rinLo > 0.f && f > 0.f && hi <= __fmul_rd(f, f)) c = CL_FULL;
-                            const int n = (int)(__ldg(off + l0 + j + 1) - __ldg(off + l0 + j));
+                            const int n = (int)(sOff[v][jj + 1] - sOff[v][jj]);
                             if (c == CL_FULL) {
                                 sure += n;
                                 fbits |= 1u << jj;
@@ -439,16 +472,20 @@ k_class(const int32_t *__restrict__ act, int na, const Thr *__restrict__ thr,
             sF[w4][t] = fbits;
         }
         // the tile's words of this query's leaf bit set: one 32-byte sector
-        // (rows are W32 words, a multiple of 8, so the sector is aligned)
-        if (qv_ok) {
+        // (rows are W32 words, a multiple of 8, so the sector is aligned), or
+        // the one word
+        if (qv_ok && NWD == 8) {
             uint4 *dst = (uint4 *)(leafBits + (int64_t)(a0 + t) * W32 + l0 / 32);
-            dst[0] = make_uint4(sW[0][t], sW[1][t], sW[2][t], sW[3][t]);
-            dst[1] = make_uint4(sW[4][t], sW[5][t], sW[6][t], sW[7][t]);
+            dst[0] = make_uint4(sW[0][t], sW[1 % NWD][t], sW[2 % NWD][t], sW[3 % NWD][t]);
+            dst[1] = make_uint4(sW[4 % NWD][t], sW[5 % NWD][t], sW[6 % NWD][t], sW[7 % NWD][t]);
             if (fullBits) {
                 uint4 *fd = (uint4 *)(fullBits + (int64_t)(a0 + t) * W32 + l0 / 32);
-                fd[0] = make_uint4(sF[0][t], sF[1][t], sF[2][t], sF[3][t]);
-                fd[1] = make_uint4(sF[4][t], sF[5][t], sF[6][t], sF[7][t]);
+                fd[0] = make_uint4(sF[0][t], sF[1 % NWD][t], sF[2 % NWD][t], sF[3 % NWD][t]);
+                fd[1] = make_uint4(sF[4 % NWD][t], sF[5 % NWD][t], sF[6 % NWD][t], sF[7 % NWD][t]);
             }
+        } else if (qv_ok) {
+            leafBits[(int64_t)(a0 + t) * W32 + l0 / 32] = sW[0][t];
+            if (fullBits) fullBits[(int64_t)(a0 + t) * W32 + l0 / 32] = sF[0][t];
         }
         __syncthreads();
         // the tile's leaves that some query of the block covers partially;
@@ -2584,20 +2621,21 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
                                                      cntSure, io.cntSure, blkCnt, blkEnt, blkMask));
             } else {
                 // query-stationary test: leaf tiles split evenly over enough
-                // CTAs per query block to fill the GPU once
-                const int64_t nTiles = (L + CQ_LT - 1) / CQ_LT;
+                // CTAs per query block to fill the GPU once; tiles of 32 leaves
+                // where tiles of 256 would leave part of it idle
                 const int perSm = tc ? 4 : 16;
+                const bool fine = (int64_t)(W32 / 8) * nlist < (int64_t)nsm * perSm;
+                const int64_t nTiles = fine ? W32 : W32 / 8;
                 int64_t gx = std::max<int64_t>(1, std::min<int64_t>(nTiles, ((int64_t)nsm * perSm + nlist - 1) / nlist));
                 gx = (nTiles + (nTiles + gx - 1) / gx - 1) / ((nTiles + gx - 1) / gx);
                 dim3 gq((unsigned)gx, (unsigned)nlist);
-                if (!tc)
-                    PM_LAUNCH("k_class", st, k_class<QB><<<gq, QB, 0, st>>>(io.act, io.na, io.thr, qp32, qpiv,
-                                                ix->s, ix->leafMeta, ix->leafOff, nullptr, L, io.cntSure, blkCnt,
-                                                blkEnt, blkMask, io.leafBits, W32, io.cntPart, io.fullBits));
-                else
-                    PM_LAUNCH("k_class", st, k_class<TC_QN><<<gq, TC_QN, 0, st>>>(io.act, io.na, io.thr, qp32,
-                                                qpiv, ix->s, ix->leafMeta, ix->leafOff, ix->bOff, L, io.cntSure,
-                                                blkCnt, blkEnt, blkMask, io.leafBits, W32, io.cntPart, io.fullBits));
+                auto launch = [&](auto kern, int threads, const int64_t *bOff) {
+                    PM_LAUNCH("k_class", st, kern<<<gq, threads, 0, st>>>(io.act, io.na, io.thr, qp32, qpiv, ix->s,
+                                                ix->leafMeta, ix->leafOff, bOff, L, io.cntSure, blkCnt, blkEnt,
+                                                blkMask, io.leafBits, W32, io.cntPart, io.fullBits));
+                };
+                if (!tc) fine ? launch(k_class<QB, 1>, QB, nullptr) : launch(k_class<QB, 8>, QB, nullptr);
+                else fine ? launch(k_class<TC_QN, 1>, TC_QN, ix->bOff) : launch(k_class<TC_QN, 8>, TC_QN, ix->bOff);
             }
             if (io.cntTight)
                 PM_LAUNCH("k_tight", st, k_tight<<<(unsigned)io.na, 256, 0, st>>>(io.act, io.na, io.thr,
