@@ -25,6 +25,7 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <type_traits>
 
 #include <cuda_bf16.h>
 
@@ -685,8 +686,16 @@ k_sublists(const int32_t *__restrict__ amb, int na2, const uint32_t *__restrict_
 }
 
 // Per-point test in partially covered leaves (the queries of the block's
-// list mask).  Grid (block, split).
-__global__ void __launch_bounds__(256)
+// list mask).  Grid (block, split); a warp per listed leaf, up to four of its
+// points per lane in registers, so that a leaf of any size fills its lanes (a block
+// per leaf ran eight warps over leaves of 92 points on average).  Points go in
+// pairs through the packed arithmetic: each half is pm_pd2_32's sequence of
+// operations on that point, bit for bit.  Bound by FP32 issue, 32 operations per
+// pair of a query and a point; a query's coordinates are read once per 128 points
+// and its two counts leave the warp in one reduction.  5,000 queries on 300,000
+// points: 0.76 ms, 1.67 with a block per leaf and a point per thread.
+constexpr int CT_PTS = 4;   // points per lane
+__global__ void __launch_bounds__(256, 2)
 k_count(const int32_t *__restrict__ act, int na, const Thr *__restrict__ thr,
         const float *__restrict__ qp32, const float *__restrict__ O32,
         const int *__restrict__ blkCnt, const int4 *__restrict__ blkEnt,
@@ -694,60 +703,99 @@ k_count(const int32_t *__restrict__ act, int na, const Thr *__restrict__ thr,
         int *__restrict__ cntSure, int *__restrict__ cntBand,
         int *__restrict__ bandN, int bandCap, int *__restrict__ bandA, int *__restrict__ bandPos)
 {
-    __shared__ float sq[QB][PM_MP];
-    __shared__ float sLo[QB], sHi[QB];
+    __shared__ __align__(16) unsigned long long sq[QB][PM_MP];   // (q_j, q_j)
+    __shared__ float2 sT[QB];                                    // lo, hi
     __shared__ int sSure[QB], sBand[QB];
     const int b = blockIdx.x;
     const int a0 = b * QB;
     const int nb = min(QB, na - a0);
+    const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
     for (int e = threadIdx.x; e < QB * PM_MP; e += blockDim.x) {
-        int qq = e / PM_MP, j = e % PM_MP;
-        sq[qq][j] = qq < nb ? qp32[(int64_t)act[a0 + qq] * PM_MP + j] : 0.f;
+        const int qq = e / PM_MP, j = e % PM_MP;
+        const float v = qq < nb ? qp32[(int64_t)act[a0 + qq] * PM_MP + j] : 0.f;
+        sq[qq][j] = f32x2_pack(v, v);
     }
     for (int qq = threadIdx.x; qq < QB; qq += blockDim.x) {
         if (qq < nb) {
-            Thr T = thr[a0 + qq];
-            sLo[qq] = T.lo;
-            sHi[qq] = T.hi;
+            const Thr T = thr[a0 + qq];
+            sT[qq] = make_float2(T.lo, T.hi);
         }
         sSure[qq] = 0;
         sBand[qq] = 0;
     }
     __syncthreads();
     const int nl = blkCnt[b];
-    for (int li = blockIdx.y; li < nl; li += gridDim.y) {
+    for (int li = blockIdx.y * wpb + (threadIdx.x >> 5); li < nl; li += gridDim.y * wpb) {
         const int64_t e = (int64_t)b * L + li;
         const int4 ent = blkEnt[e];
         const unsigned long long part =
             ((unsigned long long)blkMask[e * 2 + 1] << 32) | (unsigned long long)blkMask[e * 2];
-        const int64_t p0 = ent.y, p1 = (int64_t)ent.y + ent.z;
-        for (int64_t base = p0; base < p1; base += blockDim.x) {
-            const int64_t pos = base + threadIdx.x;
-            const bool valid = pos < p1;
-            float o[PM_MP];
+        // NP pairs of points per lane: positions base + 32 u + lane
+        auto run = [&](auto np, int64_t base, int64_t p1) {
+            constexpr int NP = decltype(np)::value;
+            unsigned long long o[NP][PM_MP];
 #pragma unroll
-            for (int j = 0; j < PM_MP; j++) o[j] = valid ? O32[pos * PM_MP + j] : 0.f;
+            for (int u = 0; u < NP; u++) {
+                const int64_t pa = base + 64 * u + lane, pb = pa + 32;
+                // positions past the leaf: NaN, which no comparison takes
+                const float nan = __int_as_float(0x7fffffff);
+#pragma unroll
+                for (int j4 = 0; j4 < PM_MP / 4; j4++) {
+                    const float4 x = pa < p1 ? __ldg((const float4 *)(O32 + pa * PM_MP) + j4) : make_float4(nan, nan, nan, nan);
+                    const float4 y = pb < p1 ? __ldg((const float4 *)(O32 + pb * PM_MP) + j4) : make_float4(nan, nan, nan, nan);
+                    o[u][4 * j4] = f32x2_pack(x.x, y.x);
+                    o[u][4 * j4 + 1] = f32x2_pack(x.y, y.y);
+                    o[u][4 * j4 + 2] = f32x2_pack(x.z, y.z);
+                    o[u][4 * j4 + 3] = f32x2_pack(x.w, y.w);
+                }
+            }
             unsigned long long bits = part;
             while (bits) {
                 const int qq = __ffsll(bits) - 1;
                 bits &= bits - 1;
-                float v = pm_pd2_32(o, sq[qq]);
-                bool sure = valid && v <= sLo[qq];
-                bool band = valid && !sure && v <= sHi[qq];
-                unsigned bs = __ballot_sync(0xffffffffu, sure);
-                unsigned bb = __ballot_sync(0xffffffffu, band);
-                if ((threadIdx.x & 31) == 0) {
-                    if (bs) atomicAdd(&sSure[qq], __popc(bs));
-                    if (bb) atomicAdd(&sBand[qq], __popc(bb));
+                const ulonglong2 *qv = (const ulonglong2 *)sq[qq];
+                unsigned long long acc[NP];
+#pragma unroll
+                for (int u = 0; u < NP; u++) acc[u] = 0ull;
+#pragma unroll
+                for (int j2 = 0; j2 < PM_MP / 2; j2++) {
+                    const ulonglong2 x = qv[j2];
+#pragma unroll
+                    for (int u = 0; u < NP; u++) {
+                        f32x2_sqdiff_acc(acc[u], o[u][2 * j2], x.x);
+                        f32x2_sqdiff_acc(acc[u], o[u][2 * j2 + 1], x.y);
+                    }
                 }
-                if (band) {
-                    int e2 = atomicAdd(bandN, 1);
-                    if (e2 < bandCap) {
-                        bandA[e2] = a0 + qq;
-                        bandPos[e2] = (int)pos;
+                const float2 T = sT[qq];
+                int c = 0;   // points <= lo, points <= hi (upper half)
+#pragma unroll
+                for (int u = 0; u < NP; u++) {
+                    const float v0 = __uint_as_float((unsigned)acc[u]), v1 = __uint_as_float((unsigned)(acc[u] >> 32));
+                    c += (v0 <= T.x ? 1 : 0) + (v1 <= T.x ? 1 : 0) + (v0 <= T.y ? 0x10000 : 0) + (v1 <= T.y ? 0x10000 : 0);
+                }
+                c = __reduce_add_sync(0xffffffffu, c);
+                const int sure = c & 0xFFFF, band = (c >> 16) - sure;
+                if (lane == 0 && sure) atomicAdd(&sSure[qq], sure);
+                if (band) {   // (warp-uniform)
+                    if (lane == 0) atomicAdd(&sBand[qq], band);
+#pragma unroll
+                    for (int u = 0; u < 2 * NP; u++) {
+                        const float v = __uint_as_float((unsigned)(u & 1 ? acc[u >> 1] >> 32 : acc[u >> 1]));
+                        if (v > T.x && v <= T.y) {
+                            const int e2 = atomicAdd(bandN, 1);
+                            if (e2 < bandCap) {
+                                bandA[e2] = a0 + qq;
+                                bandPos[e2] = (int)(base + 32 * u + lane);
+                            }
+                        }
                     }
                 }
             }
+        };
+        const int64_t p1 = (int64_t)ent.y + ent.z;
+        for (int64_t base = ent.y; base < p1; base += 32 * CT_PTS) {
+            if (p1 - base > 64) run(std::integral_constant<int, 2>(), base, p1);
+            else run(std::integral_constant<int, 1>(), base, p1);
         }
     }
     __syncthreads();
@@ -2652,7 +2700,9 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
             const int4 *blkEnt = w.blkLeaves.as<int4>();
             const uint32_t *blkMask = w.blkMask.as<uint32_t>();
             if (!tc) {
-                int splitC = std::max(1, std::min(64, (4 * nsm + nlist - 1) / nlist));
+                // about sixteen blocks per SM: the query blocks' lists differ, and
+                // blocks that are short against the launch even them out
+                const int splitC = std::max(1, std::min(256, 16 * nsm / nlist));
                 PM_LAUNCH("k_count", st, k_count<<<dim3(nlist, splitC), 256, 0, st>>>(io.act, io.na, io.thr, qp32,
                                             ix->O32, blkCnt, blkEnt, blkMask, L, io.cntSure, io.cntBand, bandN,
                                             bandCap, bandA, bandPos));

@@ -1,0 +1,33 @@
+"""Per-point range count on the CUDA cores (a warp per leaf, points in packed pairs)
+at the sizes where it can go wrong, against the FP64 oracle: |C|, rounds and stop
+rule equal for every query."""
+import math
+
+import numpy as np
+import pytest
+
+import datagen
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_2107_05537_gb300 as pm  # noqa: E402
+
+
+# leaves below, at and past 32, 64 and 128 points; one query, a block of 64, and one
+# more than several blocks; radii that cut through the leaves
+@pytest.mark.parametrize("leaf", [16, 32, 64, 129, 1024])
+@pytest.mark.parametrize("nq", [1, 64, 193])
+def test_counts_by_leaf_size(leaf, nq):
+    X, Q, _, _ = datagen.mixture(2600, 24, 2, 4.0, seed=leaf, nq=nq)
+    A = oracle.gen_projection(2, 13, 24).astype(np.float32)
+    t, _, _ = oracle.params(13, 1.5, 1 / math.e)
+    ix = pm.Index(torch.from_numpy(X).cuda(), m=13, leaf_size=leaf, proj=A)
+    for r in (3.0, 12.0, 25.0):
+        got = ix.knn(torch.from_numpy(Q).cuda(), k=3, beta=0.9, r_min=r, t=t)
+        ref = oracle.knn(X, A, Q, 3, 1.5, t, oracle.budget(len(X), 0.9, 3), r, 0)
+        assert np.array_equal(got["ids"].cpu().numpy(), ref["ids"])
+        for f in ("ncand", "rounds", "rule"):
+            assert np.array_equal(got["stats"][f], ref[f])
+    ix.close()
