@@ -2,10 +2,16 @@
 // the PM-tree of Sec. 4.1), leaf balls and pivot rings, distance sample for
 // the r_min rule of Sec. 5.2.
 #include <algorithm>
+#include <atomic>
 #include <cstdlib>
 #include <cmath>
 #include <cstring>
+#include <deque>
+#include <functional>
+#include <mutex>
+#include <new>
 #include <numeric>
+#include <thread>
 
 #include <cuda_bf16.h>
 
@@ -393,6 +399,72 @@ namespace {
 
 // ------------------------------------------------------------ host layout
 
+// Threads of one build's host layout: run(f) calls f(t) for t < threads(), on this
+// thread and the helpers; helpers wait spinning (a layout's passes are tens of
+// microseconds apart) and leave with the object.  A helper that cannot be started
+// is done without.
+class HostTeam {
+public:
+    explicit HostTeam(int want)
+    {
+        helpers_.reserve(std::max(0, want - 1));
+        for (int t = 1; t < want; t++) {
+            try {
+                helpers_.emplace_back([this, t] { loop(t); });
+            } catch (...) {
+                break;
+            }
+        }
+    }
+    ~HostTeam()
+    {
+        stop_.store(true);
+        epoch_.fetch_add(1, std::memory_order_release);
+        for (std::thread &h : helpers_) h.join();
+    }
+    int threads() const { return (int)helpers_.size() + 1; }
+    void run(const std::function<void(int)> &f)
+    {
+        job_ = &f;
+        left_.store((int)helpers_.size(), std::memory_order_relaxed);
+        epoch_.fetch_add(1, std::memory_order_release);
+        call(0);
+        for (int spin = 0; left_.load(std::memory_order_acquire) > 0; spin++)
+            if (spin > 4096) std::this_thread::yield();
+        if (failed_.exchange(false)) throw std::bad_alloc();
+    }
+    bool failed() const { return failed_.load(std::memory_order_relaxed); }
+
+private:
+    // the only exception a layout meets is a failed allocation; it is thrown again
+    // on the calling thread once every thread is back
+    void call(int t)
+    {
+        try {
+            (*job_)(t);
+        } catch (...) {
+            failed_.store(true);
+        }
+    }
+    void loop(int t)
+    {
+        unsigned seen = 0;
+        for (;;) {
+            for (int spin = 0; epoch_.load(std::memory_order_acquire) == seen; spin++)
+                if (spin > 4096) std::this_thread::yield();
+            seen++;
+            if (stop_.load()) return;
+            call(t);
+            left_.fetch_sub(1, std::memory_order_release);
+        }
+    }
+    std::vector<std::thread> helpers_;
+    const std::function<void(int)> *job_ = nullptr;
+    std::atomic<unsigned> epoch_{0};
+    std::atomic<int> left_{0};
+    std::atomic<bool> stop_{false}, failed_{false};
+};
+
 struct Bisect {
     const float *O;   // [n][16] FP32 coordinates, original order
     int m, M;
@@ -405,6 +477,7 @@ struct Bisect {
     std::vector<int32_t> pre;   // [N] index of the node's segment for the refinement, -1 if inner
     std::vector<int64_t> preLo, preHi;
     std::vector<double> key;
+    std::vector<unsigned char> side;   // by position: the 2-means side of a segment the team splits
     // the final layout (assemble): leaf-index ranges of the nodes, leaves, chunks
     std::vector<int64_t> nlo, nhi;
     std::vector<int64_t> leafOff{0};
@@ -440,33 +513,90 @@ struct Bisect {
         return std::sqrt(r);
     }
 
+    // A segment's passes over its points run on the whole team (`team` set: the
+    // large segments at the top of the hierarchy) or on the calling thread.
+    // f(part, a, b): a contiguous part of [lo, hi).
+    template <class F> static void parts(HostTeam *team, int64_t lo, int64_t hi, F f)
+    {
+        if (!team) {
+            f(0, lo, hi);
+            return;
+        }
+        const int64_t n = team->threads(), len = (hi - lo + n - 1) / n;
+        team->run([&](int t) {
+            const int64_t a = std::min(hi, lo + t * len), b = std::min(hi, a + len);
+            if (a < b) f(t, a, b);
+        });
+    }
+
+    // The first point of perm[lo, hi) farthest from c.
+    int64_t farthest(HostTeam *team, const double *c, int64_t lo, int64_t hi) const
+    {
+        const int n = team ? team->threads() : 1;
+        std::vector<double> best(n, -1.0);
+        std::vector<int64_t> at(n, lo);
+        parts(team, lo, hi, [&](int t, int64_t a, int64_t b) {
+            double v0 = -1.0;
+            int64_t i0 = a;
+            for (int64_t e = a; e < b; e++) {
+                const double v = d2(c, pt(perm[e]));
+                if (v > v0) { v0 = v; i0 = e; }
+            }
+            best[t] = v0;
+            at[t] = i0;
+        });
+        int k = 0;
+        for (int t = 1; t < n; t++)
+            if (best[t] > best[k]) k = t;
+        return at[k];
+    }
+
     // 2-means of perm[lo, hi) started from a farthest pair; returns the
-    // hyperplane (w, t) separating the two means.
-    void two_means(int64_t lo, int64_t hi, double *w, double &t)
+    // hyperplane (w, t) separating the two means.  The sums run in the order of
+    // the points whatever the threads: the team divides the distances by points
+    // and the sums by coordinates.
+    void two_means(HostTeam *team, int64_t lo, int64_t hi, double *w, double &t)
     {
         double c0[PM_MP], a[PM_MP], b[PM_MP];
         for (int j = 0; j < PM_MP; j++) c0[j] = pt(perm[lo])[j];
-        int64_t ia = lo;
-        double best = -1.0;
-        for (int64_t e = lo; e < hi; e++) {
-            double v = d2(c0, pt(perm[e]));
-            if (v > best) { best = v; ia = e; }
-        }
+        const int64_t ia = farthest(team, c0, lo, hi);
         for (int j = 0; j < PM_MP; j++) a[j] = pt(perm[ia])[j];
-        int64_t ib = lo;
-        best = -1.0;
-        for (int64_t e = lo; e < hi; e++) {
-            double v = d2(a, pt(perm[e]));
-            if (v > best) { best = v; ib = e; }
-        }
+        const int64_t ib = farthest(team, a, lo, hi);
         for (int j = 0; j < PM_MP; j++) b[j] = pt(perm[ib])[j];
         for (int it = 0; it < 6; it++) {
             double sa[PM_MP] = {0}, sb[PM_MP] = {0};
             int64_t na = 0, nb = 0;
-            for (int64_t e = lo; e < hi; e++) {
-                const float *p = pt(perm[e]);
-                if (d2(b, p) < d2(a, p)) { nb++; for (int j = 0; j < PM_MP; j++) sb[j] += p[j]; }
-                else { na++; for (int j = 0; j < PM_MP; j++) sa[j] += p[j]; }
+            if (!team) {
+                for (int64_t e = lo; e < hi; e++) {
+                    const float *p = pt(perm[e]);
+                    if (d2(b, p) < d2(a, p)) { nb++; for (int j = 0; j < PM_MP; j++) sb[j] += p[j]; }
+                    else { na++; for (int j = 0; j < PM_MP; j++) sa[j] += p[j]; }
+                }
+            } else {
+                std::vector<int64_t> cb(team->threads(), 0);
+                parts(team, lo, hi, [&](int part, int64_t x, int64_t y) {
+                    int64_t c = 0;
+                    for (int64_t e = x; e < y; e++) {
+                        const float *p = pt(perm[e]);
+                        side[e] = d2(b, p) < d2(a, p);
+                        c += side[e];
+                    }
+                    cb[part] = c;
+                });
+                for (int64_t c : cb) nb += c;
+                na = hi - lo - nb;
+                parts(team, 0, PM_MP, [&](int, int64_t x, int64_t y) {
+                    double u[PM_MP] = {0}, v[PM_MP] = {0};
+                    for (int64_t e = lo; e < hi; e++) {
+                        const float *p = pt(perm[e]);
+                        double *acc = side[e] ? v : u;
+                        for (int64_t j = x; j < y; j++) acc[j] += p[j];
+                    }
+                    for (int64_t j = x; j < y; j++) {
+                        sa[j] = u[j];
+                        sb[j] = v[j];
+                    }
+                });
             }
             if (na == 0 || nb == 0) break;
             bool moved = false;
@@ -511,31 +641,44 @@ struct Bisect {
         return id;
     }
 
-    // Splits perm[lo, hi) by 2-means in the projected space (Sec. 4.1 builds
+    // One node of the bisection as it is found; numbered in preorder afterwards.
+    struct Cut {
+        int64_t lo, hi;
+        int64_t mid = -1;        // -1: not split
+        double w[PM_MP], t;
+        Cut *left = nullptr, *right = nullptr;
+    };
+
+    // Splits one segment by 2-means in the projected space (Sec. 4.1 builds
     // the PM-tree so that node balls are tight; the m_RAD promotion of
     // Sec. 6.3 minimises covering radii).  Segments above M points are always
     // split; smaller ones only when both halves' balls shrink below 0.85 of
     // the parent's (a segment holding separate groups of points), so that a
-    // leaf does not straddle groups.  A degenerate 2-means split of a large
-    // segment falls back to the median along the same direction.
-    int32_t split(int64_t lo, int64_t hi)
+    // leaf does not straddle groups (c.mid stays -1 where it is not split).  A
+    // degenerate 2-means split of a large segment falls back to the median along
+    // the same direction.
+    void cut(HostTeam *team, Cut &c)
     {
-        const int32_t id = new_node(lo, hi);
-        const int64_t size = hi - lo;
-        if (size <= 8) return pre_leaf(id, lo, hi);
+        const int64_t lo = c.lo, hi = c.hi, size = hi - lo;
+        if (size <= 8) return;
         double w[PM_MP], t;
-        two_means(lo, hi, w, t);
-        for (int64_t e = lo; e < hi; e++) {
-            const float *p = pt(perm[e]);
-            double s = 0.0;
-            for (int j = 0; j < PM_MP; j++) s += w[j] * (double)p[j];
-            key[perm[e]] = s;
-        }
+        two_means(team, lo, hi, w, t);
+        std::vector<int64_t> right(team ? team->threads() : 1, 0);
+        parts(team, lo, hi, [&](int part, int64_t a, int64_t b) {
+            int64_t r = 0;
+            for (int64_t e = a; e < b; e++) {
+                const float *p = pt(perm[e]);
+                double s = 0.0;
+                for (int j = 0; j < PM_MP; j++) s += w[j] * (double)p[j];
+                key[perm[e]] = s;
+                r += s >= t;
+            }
+            right[part] = r;
+        });
         const double *K = key.data();
         auto less = [K](int32_t a, int32_t b) { return K[a] < K[b] || (K[a] == K[b] && a < b); };
-        int64_t nright = 0;
-        for (int64_t e = lo; e < hi; e++) nright += K[perm[e]] >= t;
-        int64_t left = size - nright;
+        int64_t left = size;
+        for (int64_t r : right) left -= r;
         if (size > M) {
             if (left < size / 16 || left > size - size / 16) {
                 left = size / 2;
@@ -545,22 +688,109 @@ struct Bisect {
                 std::partition(perm.begin() + lo, perm.begin() + hi, [K, t](int32_t a) { return K[a] < t; });
             }
         } else {
-            if (left == 0 || left == size) return pre_leaf(id, lo, hi);
+            if (left == 0 || left == size) return;
             std::vector<int32_t> saved(perm.begin() + lo, perm.begin() + hi);
             std::partition(perm.begin() + lo, perm.begin() + hi, [K, t](int32_t a) { return K[a] < t; });
             double rp = radius(lo, hi), rl = radius(lo, lo + left), rr = radius(lo + left, hi);
             if (!(std::max(rl, rr) < 0.85 * rp)) {
                 std::copy(saved.begin(), saved.end(), perm.begin() + lo);
-                return pre_leaf(id, lo, hi);
+                return;
             }
         }
-        for (int j = 0; j < PM_MP; j++) nw[(size_t)id * PM_MP + j] = (float)w[j];
-        nt[id] = (float)t;
-        int32_t L = split(lo, lo + left);
-        int32_t R = split(lo + left, hi);
-        nl[id] = L;
-        nr[id] = R;
-        return id;
+        std::copy(w, w + PM_MP, c.w);
+        c.t = t;
+        c.mid = lo + left;
+    }
+
+    // The whole bisection of perm[0, n).  Segments share no point, so their
+    // splits are independent: the largest ones are split by the team together, the
+    // rest by its threads from a common list (a thread takes a small segment with
+    // everything below it).  Positions, keys and sums are those of splitting one
+    // segment after another, and the nodes are numbered in that order.
+    void split_all(int64_t n)
+    {
+        const int64_t hw = std::max(1u, std::thread::hardware_concurrency());
+        HostTeam team((int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(hw, 16), n / 512)));
+        const int64_t big = std::max<int64_t>(2048, n / team.threads()), small = 512;
+        std::deque<Cut> pool;    // (stable addresses)
+        auto make = [&pool](int64_t lo, int64_t hi) {
+            pool.emplace_back();
+            pool.back().lo = lo;
+            pool.back().hi = hi;
+            return &pool.back();
+        };
+        Cut *root = make(0, n);
+        std::vector<Cut *> todo, large{root};
+        while (!large.empty()) {
+            Cut *c = large.back();
+            large.pop_back();
+            if (c->hi - c->lo < big || team.threads() == 1) {
+                todo.push_back(c);
+                continue;
+            }
+            cut(&team, *c);
+            if (c->mid < 0) continue;
+            c->left = make(c->lo, c->mid);
+            c->right = make(c->mid, c->hi);
+            large.push_back(c->left);
+            large.push_back(c->right);
+        }
+        std::sort(todo.begin(), todo.end(), [](const Cut *x, const Cut *y) { return x->hi - x->lo < y->hi - y->lo; });
+        std::mutex mu;
+        std::atomic<int64_t> open{(int64_t)todo.size()};   // segments listed or in work
+        team.run([&](int) {
+            std::vector<Cut *> own;
+            for (;;) {
+                Cut *c = nullptr;
+                if (!own.empty()) {
+                    c = own.back();
+                    own.pop_back();
+                } else {
+                    if (open.load(std::memory_order_acquire) == 0 || team.failed()) return;
+                    std::lock_guard<std::mutex> lk(mu);
+                    if (!todo.empty()) {
+                        c = todo.back();
+                        todo.pop_back();
+                    }
+                }
+                if (!c) {
+                    std::this_thread::yield();
+                    continue;
+                }
+                cut(nullptr, *c);
+                const bool mine = c->hi - c->lo <= small;   // (its children stay with this thread)
+                if (c->mid >= 0) {
+                    {
+                        std::lock_guard<std::mutex> lk(mu);
+                        c->left = make(c->lo, c->mid);
+                        c->right = make(c->mid, c->hi);
+                        if (!mine) todo.push_back(c->left);
+                    }
+                    open.fetch_add(2, std::memory_order_relaxed);
+                    if (mine) own.push_back(c->left);
+                    own.push_back(c->right);
+                }
+                open.fetch_sub(1, std::memory_order_release);
+            }
+        });
+        // preorder numbers
+        std::vector<std::pair<Cut *, int32_t>> stack;   // node, and its parent's right slot (-1: none)
+        stack.emplace_back(root, -1);
+        while (!stack.empty()) {
+            const auto [c, parent] = stack.back();
+            stack.pop_back();
+            const int32_t id = new_node(c->lo, c->hi);
+            if (parent >= 0) nr[parent] = id;
+            if (c->mid < 0) {
+                pre_leaf(id, c->lo, c->hi);
+                continue;
+            }
+            for (int j = 0; j < PM_MP; j++) nw[(size_t)id * PM_MP + j] = (float)c->w[j];
+            nt[id] = (float)c->t;
+            nl[id] = id + 1;   // the left child follows
+            stack.emplace_back(c->right, id);
+            stack.emplace_back(c->left, -1);
+        }
     }
 
     // The hierarchy after the original-space refinement: the refined
@@ -884,8 +1114,9 @@ pmlsh_status pm_build_index(pmlsh_index *ix, const float *X, bool x_on_device,
     bs.M = ix->M;
     bs.perm.resize(n);
     bs.key.resize(n);
+    bs.side.resize(n);
     std::iota(bs.perm.begin(), bs.perm.end(), 0);
-    bs.split(0, n);
+    bs.split_all(n);
     // original-space refinement of the segments on the device, over the
     // device copy of X (original order)
     {
