@@ -91,8 +91,9 @@ k_refine_leaves(const float *__restrict__ X, int ld, int d, int32_t *__restrict_
     int32_t *P = perm + S.lo;   // this segment's ids
     int32_t *T = tmp + S.lo;
     // centres: mu, a, b, a2, b2 (FP64 [ld] each, this CTA's scratch)
-    double *mu = scratch + (size_t)blockIdx.x * 5 * ld;
+    double *mu = scratch + (size_t)blockIdx.x * 6 * ld;
     double *ca = mu + ld, *cb = ca + ld, *ca2 = cb + ld, *cb2 = ca2 + ld;
+    float *cf0 = (float *)(cb2 + ld), *cf1 = cf0 + ld;   // FP32 roundings of the Lloyd centres
     int4 *onode = out.node + S.nodeBase;
     int4 *oleaf = out.leaf + S.leafBase;
     int32_t *ochunk = out.chunkEnd + S.chunkBase;
@@ -101,17 +102,41 @@ k_refine_leaves(const float *__restrict__ X, int ld, int d, int32_t *__restrict_
         return;
     }
 
-    // ||x_P[i] - c||^2 for i in [a, b) into sDist (a warp per point, FP64 sums)
+    // cSlack >= ||c - FP32(c)|| for every centre: 2^-24 of the largest row norm
+    // (centres are means of rows), with a margin for the FP32 norms
+    float xn = 0.f;
+    for (int i = w; i < s; i += nw) {
+        const float *x = X + (int64_t)P[i] * ld;
+        float v = 0.f;
+        for (int j = lane; j < d; j += 32) v = fmaf(x[j], x[j], v);
+        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        xn = fmaxf(xn, v);
+    }
+    if (lane == 0) sDist[w] = xn;
+    __syncthreads();
+    for (int v = 0; v < nw; v++) xn = fmaxf(xn, sDist[v]);
+    const float cSlack = 0x1.0p-24f * 1.01f * (1.f + (float)(d + 16) * 0x1.0p-24f) * sqrtf(xn) + 1e-30f;
+    __syncthreads();
+
+    // The kernel is bound by the FP64 pipe (64 cycles per warp instruction): the
+    // inputs are widened by integer operations, divisions and last sums are taken by
+    // one thread, and the Lloyd steps compare FP32 distances with a proven bound,
+    // FP64 ones only where that cannot decide.  100,000 points of 128 coordinates:
+    // 6.7 ms, 17.5 with every distance in FP64; the same layout.
+    // ||x - c||^2 of one row by a warp (FP64 sums, rounded to FP32), in every lane
+    auto row_dist = [&](const float *x, const double *c) -> float {
+        double acc = 0.0;
+        for (int j = lane; j < d; j += 32) {
+            const double t = pm_f2d_exact(x[j]) - c[j];
+            acc += t * t;
+        }
+        return (float)lr_warp_sum(acc);
+    };
+    // ||x_P[i] - c||^2 for i in [a, b) into sDist (a warp per point)
     auto dist_to = [&](const double *c, int a, int b) {
         for (int i = a + w; i < b; i += nw) {
-            const float *x = X + (int64_t)P[i] * ld;
-            double acc = 0.0;
-            for (int j = lane; j < d; j += 32) {
-                const double t = (double)x[j] - c[j];
-                acc += t * t;
-            }
-            acc = lr_warp_sum(acc);
-            if (lane == 0) sDist[i] = (float)acc;
+            const float v = row_dist(X + (int64_t)P[i] * ld, c);
+            if (lane == 0) sDist[i] = v;
         }
         __syncthreads();
     };
@@ -127,18 +152,20 @@ k_refine_leaves(const float *__restrict__ X, int ld, int d, int32_t *__restrict_
     // FP64 mean of the points i in [a, b) with sSide[i] == side (side < 0: all)
     auto mean_of = [&](double *c, int a, int b, int side) {
         const int cnt = count_if(a, b, [&](int i) { return side < 0 || sSide[i] == side; });
-        const double inv = cnt > 0 ? 1.0 / (double)cnt : 0.0;
+        if (tid == 0) sRed[0] = cnt > 0 ? 1.0 / (double)cnt : 0.0;
+        __syncthreads();
+        const double inv = sRed[0];
         for (int j = tid; j < d; j += LR_THREADS) {
             double acc = 0.0;
             for (int i = a; i < b; i++)
-                if (side < 0 || sSide[i] == side) acc += (double)X[(int64_t)P[i] * ld + j];
+                if (side < 0 || sSide[i] == side) acc += pm_f2d_exact(X[(int64_t)P[i] * ld + j]);
             c[j] = acc * inv;
         }
         __syncthreads();
         return cnt;
     };
     auto copy_point = [&](double *c, int i) {
-        for (int j = tid; j < d; j += LR_THREADS) c[j] = (double)X[(int64_t)P[i] * ld + j];
+        for (int j = tid; j < d; j += LR_THREADS) c[j] = pm_f2d_exact(X[(int64_t)P[i] * ld + j]);
         __syncthreads();
     };
     // index of the largest sDist[i] in [a, b) (first on ties)
@@ -168,43 +195,69 @@ k_refine_leaves(const float *__restrict__ X, int ld, int d, int32_t *__restrict_
     auto sum_dist = [&](int a, int b, int side) -> double {
         double acc = 0.0;
         for (int i = a + tid; i < b; i += LR_THREADS)
-            if (side < 0 || sSide[i] == side) acc += (double)sDist[i];
+            if (side < 0 || sSide[i] == side) acc += pm_f2d_exact(sDist[i]);
         acc = lr_warp_sum(acc);
         if (lane == 0) sRed[w] = acc;
         __syncthreads();
-        double all = 0.0;
-        for (int v = 0; v < nw; v++) all += sRed[v];
+        if (tid == 0) {
+            double all = 0.0;
+            for (int v = 0; v < nw; v++) all += sRed[v];
+            sRed[0] = all;
+        }
+        __syncthreads();
+        const double all = sRed[0];
         __syncthreads();
         return all;
     };
     // Lloyd steps from centres (c0, c1) over [a, b): sides in sSide (1 =
-    // nearer c1); returns the side-0 count, the two sums of squared
-    // deviations in *s0, *s1
+    // nearer c1, by the FP32 roundings of the FP64 distances); returns the side-0
+    // count, the two sums of squared deviations in *s0, *s1
     auto lloyd = [&](double *c0, double *c1, int a, int b, double *s0, double *s1) -> int {
         const int size = b - a;
         int n0 = 0;
+        for (int j = tid; j < d; j += LR_THREADS) {
+            cf0[j] = (float)c0[j];
+            cf1[j] = (float)c1[j];
+        }
+        __syncthreads();
         for (int it = 0; it < 6; it++) {
-            dist_to(c0, a, b);
-            for (int i = a + tid; i < b; i += LR_THREADS) sSort[i] = sDist[i];
-            __syncthreads();
-            dist_to(c1, a, b);
-            for (int i = a + tid; i < b; i += LR_THREADS) sSide[i] = sDist[i] < sSort[i] ? 1 : 0;
+            for (int i = a + w; i < b; i += nw) {
+                const float *x = X + (int64_t)P[i] * ld;
+                float D0 = 0.f, D1 = 0.f;
+                for (int j = lane; j < d; j += 32) {
+                    const float v = x[j], u0 = v - cf0[j], u1 = v - cf1[j];
+                    D0 = fmaf(u0, u0, D0);
+                    D1 = fmaf(u1, u1, D1);
+                }
+                for (int o = 16; o; o >>= 1) {
+                    D0 += __shfl_xor_sync(0xffffffffu, D0, o);
+                    D1 += __shfl_xor_sync(0xffffffffu, D1, o);
+                }
+                // D_i within a relative (d + 16) 2^-24 of the distance^2 to the
+                // FP32 centre, which lies within cSlack of the FP64 one: twice
+                // the sum of both errors, and more than the rounding to FP32
+                const float err = 4.f * (float)(d + 16) * 0x1.0p-24f * (D0 + D1) +
+                                  4.f * cSlack * (sqrtf(D0) + sqrtf(D1)) + 8.f * cSlack * cSlack;
+                bool one = D1 < D0;
+                if (!(fabsf(D0 - D1) > err)) one = row_dist(x, c1) < row_dist(x, c0);   // (warp-uniform)
+                if (lane == 0) sSide[i] = one ? 1 : 0;
+            }
             __syncthreads();
             n0 = count_if(a, b, [&](int i) { return sSide[i] == 0; });
             if (n0 == 0 || n0 == size) break;
-            // new centres (kept if they moved)
+            // new centres (kept if they moved): a thread per side and column
             if (tid == 0) sInt[1] = 0;
             __syncthreads();
-            for (int j = tid; j < d; j += LR_THREADS) {
-                double acc0 = 0.0, acc1 = 0.0;
-                for (int i = a; i < b; i++) {
-                    const double x = (double)X[(int64_t)P[i] * ld + j];
-                    if (sSide[i]) acc1 += x; else acc0 += x;
-                }
-                const double v0 = acc0 / (double)n0, v1 = acc1 / (double)(size - n0);
-                if (v0 != c0[j] || v1 != c1[j]) sInt[1] = 1;
-                c0[j] = v0;
-                c1[j] = v1;
+            for (int e = tid; e < 2 * d; e += LR_THREADS) {
+                const int side = e >= d ? 1 : 0, j = e - side * d;
+                double acc = 0.0;
+                for (int i = a; i < b; i++)
+                    if (sSide[i] == side) acc += pm_f2d_exact(X[(int64_t)P[i] * ld + j]);
+                const double v = acc / (double)(side ? size - n0 : n0);
+                double *c = side ? c1 : c0;
+                if (v != c[j]) sInt[1] = 1;
+                c[j] = v;
+                (side ? cf1 : cf0)[j] = (float)v;
             }
             __syncthreads();
             if (!sInt[1]) break;
@@ -293,11 +346,13 @@ k_refine_leaves(const float *__restrict__ X, int ld, int d, int32_t *__restrict_
             // 1. outliers beyond twice the median distance to the mean
             mean_of(mu, a, b, -1);
             dist_to(mu, a, b);
-            for (int i = tid; i < LR_MAXS; i += LR_THREADS) sSort[i] = i < size ? sDist[a + i] : INFINITY;
+            int np = 2;   // (the sort's length: the next power of two)
+            while (np < size) np <<= 1;
+            for (int i = tid; i < np; i += LR_THREADS) sSort[i] = i < size ? sDist[a + i] : INFINITY;
             __syncthreads();
-            for (int k2 = 2; k2 <= LR_MAXS; k2 <<= 1)
+            for (int k2 = 2; k2 <= np; k2 <<= 1)
                 for (int j2 = k2 >> 1; j2 > 0; j2 >>= 1) {
-                    for (int i = tid; i < LR_MAXS; i += LR_THREADS) {
+                    for (int i = tid; i < np; i += LR_THREADS) {
                         const int l2 = i ^ j2;
                         if (l2 > i) {
                             const float x = sSort[i], y = sSort[l2];
@@ -461,7 +516,7 @@ pmlsh_status pm_refine_leaves(const float *Xo, int ld, int d, int32_t *permD, co
     PM_TRY(lr_alloc(&dLeaf, lb)); mem.p.push_back(dLeaf);
     PM_TRY(lr_alloc(&dChunk, cb)); mem.p.push_back(dChunk);
     PM_TRY(lr_alloc(&dCount, ns * 3)); mem.p.push_back(dCount);
-    PM_TRY(lr_alloc(&dScratch, (size_t)grid * 5 * ld)); mem.p.push_back(dScratch);
+    PM_TRY(lr_alloc(&dScratch, (size_t)grid * 6 * ld)); mem.p.push_back(dScratch);
     PM_TRY(lr_alloc(&dErr, 1)); mem.p.push_back(dErr);
     PM_CUDA(cudaMemcpyAsync(dSeg, segs.data(), ns * sizeof(LrSeg), cudaMemcpyHostToDevice, st));
     PM_CUDA(cudaMemsetAsync(dErr, 0, sizeof(int), st));
