@@ -414,10 +414,10 @@ pmlsh_status pmlsh_gamma_calibrate(pmlsh_index *index, double pr, int64_t nsampl
  * not depend on the bands.  From `opts` the call uses k, T and alpha2 (c,
  * alpha1, t and gamma are not used).  Outputs as pmlsh_closest_pair; stats:
  * count = pairs verified (T), lca_nodes = leaf pairs listed, nodes_done =
- * leaf pairs examined, self_pairs, fp64_checks.  Memory grows with T (12 bytes per kept
- * pair plus a batch of up to 2^24 pairs) and with the leaf count L: a listing
- * buffer of 12 bytes per leaf pair, L(L-1)/2, and 16 bytes per listed leaf
- * pair while a band is ordered (on the device by a radix sort for up to
+ * leaf pairs examined, self_pairs, fp64_checks.  Memory grows with T (two
+ * buffers of 12 bytes per kept pair and per pair of a batch of up to 2^24)
+ * and with the leaf pairs that a band lists (36 bytes each; the list holds at
+ * least 2^23 or all L(L-1)/2; ordered on the device by a radix sort for up to
  * 92,682 leaves, on the host beyond).  Errors: EINVAL, ENOMEM,
  * ECUDA, EINTERNAL (more than 4096 pairs tied inside one FP32 error band; a
  * device ordering that fails its check). */

@@ -109,7 +109,7 @@ template <class T> struct DevTmp {
 }  // namespace
 
 pmlsh_status pm_distance_sample(const pmlsh_index *ix, int64_t npairs, uint64_t seed, std::vector<double> &out,
-                                cudaStream_t st)
+                                cudaStream_t st, bool sorted)
 {
     const int64_t n = ix->n;
     DevTmp<int32_t> inv;
@@ -131,7 +131,7 @@ pmlsh_status pm_distance_sample(const pmlsh_index *ix, int64_t npairs, uint64_t 
             return PMLSH_EINTERNAL;
         }
     }
-    std::sort(out.begin(), out.end());
+    if (sorted) std::sort(out.begin(), out.end());
     return PMLSH_OK;
 }
 

@@ -411,26 +411,36 @@ struct PairExact {
     int32_t a, b;   // positions
 };
 
-__global__ void k_pair_collect(const PairCand *__restrict__ p, int64_t n, float thr, const float *__restrict__ X,
-                               int ld, int d, const double *__restrict__ O64, int m, int useProj,
-                               const int32_t *__restrict__ perm, PairExact *__restrict__ out,
-                               unsigned long long *cnt, unsigned long long cap)
+// (the entries' positions first, so that their FP64 sums fill whole warps: a warp's
+// FP64 instruction takes as long for one entry as for 32)
+__global__ void __launch_bounds__(256)
+k_pair_pick(const PairCand *__restrict__ p, int64_t n, float thr, PairExact *__restrict__ out, unsigned long long *cnt,
+            unsigned long long cap)
 {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+        const PairCand c = p[e];
+        if (!(c.key <= thr)) continue;
+        const unsigned long long slot = atomicAdd(cnt, 1ull);
+        if (slot >= cap) continue;
+        out[slot].a = c.a;
+        out[slot].b = c.b;
+    }
+}
+
+__global__ void __launch_bounds__(32)
+k_pair_exact(const float *__restrict__ X, int ld, int d, const double *__restrict__ O64, int m, int useProj,
+             const int32_t *__restrict__ perm, PairExact *__restrict__ v, const unsigned long long *cnt,
+             unsigned long long cap)
+{
+    const unsigned long long n = *cnt < cap ? *cnt : cap, e = blockIdx.x * 32ull + threadIdx.x;
     if (e >= n) return;
-    const PairCand c = p[e];
-    if (!(c.key <= thr)) return;
-    unsigned long long slot = atomicAdd(cnt, 1ull);
-    if (slot >= cap) return;
-    PairExact x;
-    x.dist = useProj ? pm_pdist64(O64 + (int64_t)c.a * PM_MP, O64 + (int64_t)c.b * PM_MP, m)
-                     : pm_dist64(X + (int64_t)c.a * ld, X + (int64_t)c.b * ld, d);
-    int64_t ia = perm[c.a], ib = perm[c.b];
+    PairExact x = v[e];
+    x.dist = useProj ? pm_pdist64(O64 + (int64_t)x.a * PM_MP, O64 + (int64_t)x.b * PM_MP, m)
+                     : pm_dist64(X + (int64_t)x.a * ld, X + (int64_t)x.b * ld, d);
+    const int64_t ia = perm[x.a], ib = perm[x.b];
     x.i = ia < ib ? ia : ib;
     x.j = ia < ib ? ib : ia;
-    x.a = c.a;
-    x.b = c.b;
-    out[slot] = x;
+    v[e] = x;
 }
 
 __host__ __device__ __forceinline__ bool pe_less(const PairExact &x, const PairExact &y)
@@ -555,32 +565,66 @@ struct LeafPair {
 
 // Mindist of Sec. 6.1 for leaf pairs (l1, l2), l1 < l2: the larger of
 // ||RO1, RO2|| - r1 - r2 and the gaps between the pivot rings, from the leaf
-// entries (FP32, rounded so that it stays a lower bound).  Pairs with
-// Mindist <= dT are listed.  Block per l1, threads over l2.
-__global__ void k_bnb_mindist(const float *__restrict__ meta, int s, int64_t L, float dLo, float dT,
-                              LeafPair *__restrict__ out, unsigned long long *cnt, unsigned long long cap)
+// entries (FP32, rounded so that it stays a lower bound).  Pairs with Mindist in
+// (dLo, dT] are listed, up to cap, and counted.  Bound by FP32 issue,
+// about 70 instructions per pair: a block takes 128 leaves l1, a record per thread
+// in registers, and reads its share of the l2 records (grid.y slices) through shared
+// memory, 32 at a time, instead of each thread reading every 160-byte record from
+// L2; the listed pairs of a warp take one atomic.  22,125 leaves (245 M pairs):
+// 1.2 ms, 9.1 before.
+constexpr int BM_T = 128;
+__global__ void __launch_bounds__(BM_T)
+k_bnb_mindist(const float *__restrict__ meta, int s, int64_t L, float dLo, float dT, LeafPair *__restrict__ out,
+              unsigned long long *cnt, unsigned long long cap)
 {
-    const int64_t l1 = blockIdx.x;
-    const float *M1 = meta + l1 * PM_LEAF_STRIDE;
-    for (int64_t l2 = l1 + 1 + threadIdx.x; l2 < L; l2 += blockDim.x) {
-        const float *M2 = meta + l2 * PM_LEAF_STRIDE;
-        const float dc = __fsqrt_rn(pm_pd2_32(M1, M2));
-        float md = __fsub_rn(__fsub_rn(__fmul_rn(dc, 1.f - 1e-5f), M1[16]), M2[16]);
-        for (int i = 0; i < PM_MAX_PIVOTS; i++) {
-            if (i < s) {
-                // rings [min, max] of the two leaves (already widened outwards)
-                md = fmaxf(md, __fsub_rn(M2[24 + i], M1[32 + i]));
-                md = fmaxf(md, __fsub_rn(M1[24 + i], M2[32 + i]));
+    __shared__ __align__(16) float sM[32][PM_LEAF_STRIDE];
+    const int t = threadIdx.x, lane = t & 31;
+    const int64_t a0 = (int64_t)blockIdx.x * BM_T, l1 = a0 + t;
+    const bool v1 = l1 < L;
+    float o[PM_MP], hn[PM_MAX_PIVOTS], hx[PM_MAX_PIVOTS];
+    const float *M1 = meta + (v1 ? l1 : 0) * PM_LEAF_STRIDE;
+#pragma unroll
+    for (int j = 0; j < PM_MP; j++) o[j] = M1[j];
+    const float r1 = M1[16];
+#pragma unroll
+    for (int i = 0; i < PM_MAX_PIVOTS; i++) {
+        // pivots beyond s give no gap
+        hn[i] = i < s ? M1[24 + i] : -INFINITY;
+        hx[i] = i < s ? M1[32 + i] : INFINITY;
+    }
+    // l2 tiles of 32 from the block's first possible one
+    const int64_t t0 = (a0 + 1) / 32, nT = (L + 31) / 32;
+    for (int64_t tile = t0 + blockIdx.y; tile < nT; tile += gridDim.y) {
+        const int64_t b0 = tile * 32;
+        const int nb = L - b0 < 32 ? (int)(L - b0) : 32;
+        __syncthreads();
+        for (int e = t; e < nb * (PM_LEAF_STRIDE / 4); e += BM_T)
+            ((float4 *)&sM[0][0])[e] = __ldg((const float4 *)(meta + b0 * PM_LEAF_STRIDE) + e);
+        __syncthreads();
+        for (int c = 0; c < nb; c++) {
+            const float *M2 = sM[c];
+            const float dc = __fsqrt_rn(pm_pd2_32(o, M2));
+            float md = __fsub_rn(__fsub_rn(__fmul_rn(dc, 1.f - 1e-5f), r1), M2[16]);
+#pragma unroll
+            for (int i = 0; i < PM_MAX_PIVOTS; i++) {
+                if (i < s) {
+                    // rings [min, max] of the two leaves (already widened outwards)
+                    md = fmaxf(md, __fsub_rn(M2[24 + i], hx[i]));
+                    md = fmaxf(md, __fsub_rn(hn[i], M2[32 + i]));
+                }
             }
-        }
-        if (md > dLo && md <= dT) {
-            const unsigned long long slot = atomicAdd(cnt, 1ull);
-            if (slot < cap) {
+            const bool in = v1 && b0 + c > l1 && md > dLo && md <= dT;
+            const unsigned m = __ballot_sync(0xffffffffu, in);
+            if (m == 0u) continue;
+            unsigned long long base = 0;
+            if (lane == 0) base = atomicAdd(cnt, (unsigned long long)__popc(m));
+            base = __shfl_sync(0xffffffffu, base, 0) + __popc(m & ((1u << lane) - 1u));
+            if (in && base < cap) {
                 LeafPair lp;
                 lp.md = md;
                 lp.l1 = (int32_t)l1;
-                lp.l2 = (int32_t)l2;
-                out[slot] = lp;
+                lp.l2 = (int32_t)(b0 + c);
+                out[base] = lp;
             }
         }
     }
@@ -621,37 +665,33 @@ k_rs_hist(const unsigned long long *__restrict__ key, int64_t n, int shift, unsi
     hist[(int64_t)threadIdx.x * nb + blockIdx.x] = h[threadIdx.x];
 }
 
-// exclusive prefix sum of h[0, N) in place, one block of 1024 threads
-__global__ void __launch_bounds__(1024) k_rs_scan(unsigned int *__restrict__ h, int64_t N)
+// exclusive prefix sums of each digit's row h[d nb, (d + 1) nb) in place, a block
+// per digit, and the rows' totals
+__global__ void __launch_bounds__(256) k_rs_scan(unsigned int *__restrict__ h, int nb, unsigned int *__restrict__ total)
 {
-    __shared__ unsigned int ws[32];
-    const int64_t seg = (N + 1023) / 1024;
-    const int64_t t0 = threadIdx.x * seg, t1 = t0 + seg < N ? t0 + seg : N;
-    unsigned int sum = 0u;
-    for (int64_t i = t0; i < t1; i++) sum += h[i];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    unsigned int incl = sum;
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    if (lane == 31) ws[w] = incl;
-    __syncthreads();
-    if (w == 0) {
-        unsigned int x = ws[lane], xi = x;
+    __shared__ unsigned int ws[8];
+    unsigned int *row = h + (int64_t)blockIdx.x * nb;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    unsigned int carry = 0u;
+    for (int i0 = 0; i0 < nb; i0 += 256) {
+        const unsigned int v = i0 + t < nb ? row[i0 + t] : 0u;
+        unsigned int incl = v;
         for (int o = 1; o < 32; o <<= 1) {
-            const unsigned int v = __shfl_up_sync(0xffffffffu, xi, o);
-            if (lane >= o) xi += v;
+            const unsigned int x = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += x;
         }
-        ws[lane] = xi - x;
+        if (lane == 31) ws[w] = incl;
+        __syncthreads();
+        unsigned int before = 0u, all = 0u;
+        for (int i = 0; i < 8; i++) {
+            before += i < w ? ws[i] : 0u;
+            all += ws[i];
+        }
+        if (i0 + t < nb) row[i0 + t] = carry + before + incl - v;
+        carry += all;
+        __syncthreads();
     }
-    __syncthreads();
-    unsigned int run = ws[w] + incl - sum;
-    for (int64_t i = t0; i < t1; i++) {
-        const unsigned int v = h[i];
-        h[i] = run;
-        run += v;
-    }
+    if (t == 0) total[blockIdx.x] = carry;
 }
 
 // stable scatter by one digit: each block walks its keys in order, 256 per
@@ -659,13 +699,27 @@ __global__ void __launch_bounds__(1024) k_rs_scan(unsigned int *__restrict__ h, 
 // digit before it in the round (earlier warps, then earlier lanes)
 __global__ void __launch_bounds__(RS_THREADS)
 k_rs_scatter(const unsigned long long *__restrict__ in, unsigned long long *__restrict__ out, int64_t n, int shift,
-             const unsigned int *__restrict__ off, int nb)
+             const unsigned int *__restrict__ off, const unsigned int *__restrict__ total, int nb)
 {
     constexpr int NW = RS_THREADS / 32;
     __shared__ unsigned int base[256];
     __shared__ unsigned int wc[NW][256];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    base[t] = off[(int64_t)t * nb + blockIdx.x];
+    {
+        // a digit's first place: the totals of the digits before it
+        const unsigned int v = total[t];
+        unsigned int incl = v;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned int x = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += x;
+        }
+        if (lane == 31) wc[0][w] = incl;
+        __syncthreads();
+        unsigned int before = 0u;
+        for (int i = 0; i < w; i++) before += wc[0][i];
+        __syncthreads();
+        base[t] = off[(int64_t)t * nb + blockIdx.x] + before + incl - v;
+    }
     const int64_t b0 = (int64_t)blockIdx.x * RS_THREADS * RS_ITEMS;
     for (int r = 0; r < RS_ITEMS; r++) {
         for (int j = 0; j < NW; j++) wc[j][t] = 0u;
@@ -724,56 +778,343 @@ __global__ void k_lp_decode(const unsigned long long *__restrict__ key, int64_t 
     out[e] = x;
 }
 
-// Every cross pair of the listed leaf pairs, keyed by the FP32 projected
-// squared distance, at the listed offsets.  Block per leaf pair.
-__global__ void k_bnb_cross(const float *__restrict__ O32, const int64_t *__restrict__ off,
-                            const int2 *__restrict__ lp, const int64_t *__restrict__ lpOff,
-                            PairCand *__restrict__ out)
+// State of the T-cut on the device: the selection's progress, the band of its last
+// key, and the bound dT of the T-th projected distance that the search stops at.
+struct CutState {
+    unsigned long long need;      // rank left inside the selected prefix
+    unsigned long long nBelow, nBand;   // counters of the last split
+    unsigned long long fp64;      // band entries of all cuts
+    unsigned int prefix;          // bits of the T-th key found so far
+    int err;                      // 1: a band did not fit or did not hold the cut
+    float lo, hi;                 // FP32 band of the T-th key
+    int below;                    // keys below lo exist (its distance is above the error)
+    int pad;
+    double dT;                    // upper bound of the T-th projected distance
+};
+// What the next batch of listed leaf pairs takes.
+struct BatchPlan {
+    long long end, tot;           // leaf pairs [next, end), their cross pairs
+    unsigned long long fp64;
+    double dT;
+    int err, stop;                // stop: the first pair's Mindist exceeds dT
+};
+
+// Sizes na nb of the listed leaf pairs, and per block of 1,024 their sum.
+__global__ void __launch_bounds__(1024)
+k_lp_size(const LeafPair *__restrict__ lp, int64_t n, const int64_t *__restrict__ off, int64_t *__restrict__ pre,
+          int64_t *__restrict__ blk)
 {
-    const int2 pr = lp[blockIdx.x];
-    const int64_t a0 = off[pr.x], na = off[pr.x + 1] - a0;
-    const int64_t b0 = off[pr.y], nb = off[pr.y + 1] - b0;
-    const int64_t base = lpOff[blockIdx.x];
-    for (int64_t e = threadIdx.x; e < na * nb; e += blockDim.x) {
-        const int64_t ia = e / nb, ib = e % nb;
-        PairCand pc;
-        pc.key = pm_pd2_32(O32 + (a0 + ia) * PM_MP, O32 + (b0 + ib) * PM_MP);
-        pc.a = (int32_t)(a0 + ia);
-        pc.b = (int32_t)(b0 + ib);
-        out[base + e] = pc;
+    __shared__ int64_t ws[32];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int64_t e = blockIdx.x * 1024ll + t;
+    int64_t v = 0;
+    if (e < n) {
+        const LeafPair x = lp[e];
+        v = (off[x.l1 + 1] - off[x.l1]) * (off[x.l2 + 1] - off[x.l2]);
+    }
+    int64_t incl = v;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t x = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += x;
+    }
+    if (lane == 31) ws[w] = incl;
+    __syncthreads();
+    if (w == 0) {
+        int64_t x = ws[lane], xi = x;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t y = __shfl_up_sync(0xffffffffu, xi, o);
+            if (lane >= o) xi += y;
+        }
+        ws[lane] = xi - x;
+        if (lane == 31) blk[blockIdx.x] = xi;
+    }
+    __syncthreads();
+    if (e < n) pre[e] = ws[w] + incl - v;   // exclusive, inside the block
+}
+// exclusive prefix sums of blk [nb] in place, one block
+__global__ void __launch_bounds__(1024) k_lp_scan(int64_t *__restrict__ blk, int nb)
+{
+    __shared__ int64_t ws[32];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    int64_t carry = 0;
+    for (int i0 = 0; i0 < nb; i0 += 1024) {
+        const int64_t v = i0 + t < nb ? blk[i0 + t] : 0;
+        int64_t incl = v;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t x = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += x;
+        }
+        if (lane == 31) ws[w] = incl;
+        __syncthreads();
+        int64_t before = 0, all = 0;
+        for (int i = 0; i < 32; i++) {
+            before += i < w ? ws[i] : 0;
+            all += ws[i];
+        }
+        if (i0 + t < nb) blk[i0 + t] = carry + before + incl - v;
+        carry += all;
+        __syncthreads();
     }
 }
 
-// Entries with key < lo moved to out (order kept only per block).
-__global__ void k_pair_below(const PairCand *__restrict__ p, int64_t n, float lo, PairCand *__restrict__ out,
-                             unsigned long long *cnt)
+// The batch that starts at listed pair `next`: at most maxPairs leaf pairs, Mindist
+// <= dT, and (beyond the first) at most cap cross pairs.  One warp: 32-way searches.
+__global__ void __launch_bounds__(32)
+k_bnb_plan(const LeafPair *__restrict__ lp, const int64_t *__restrict__ pre, const int64_t *__restrict__ blk,
+           const int64_t *__restrict__ off, int64_t n, int64_t next, int64_t maxPairs, int64_t cap,
+           const CutState *__restrict__ st, BatchPlan *__restrict__ out)
 {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    const PairCand c = p[e];
-    if (c.key < lo) out[atomicAdd(cnt, 1ull)] = c;
+    const int lane = threadIdx.x;
+    const double dT = st->dT;
+    auto at = [&](int64_t e) { return pre[e] + blk[e >> 10]; };
+    auto size = [&](int64_t e) {
+        const LeafPair x = lp[e];
+        return (off[x.l1 + 1] - off[x.l1]) * (off[x.l2 + 1] - off[x.l2]);
+    };
+    const int64_t base = at(next);
+    // first index in [next, hi) that a batch may not hold (ok is true, then false)
+    int64_t lo = next, hi = next + maxPairs < n ? next + maxPairs : n;
+    while (lo < hi) {
+        const int64_t step = (hi - lo + 31) / 32, e = lo + lane * step;
+        bool ok = false;
+        if (e < hi) ok = (double)lp[e].md <= dT && (e == next || at(e) - base + size(e) <= cap);
+        const unsigned m = __ballot_sync(0xffffffffu, ok);
+        const int k = m == 0xffffffffu ? 32 : __ffs(~m) - 1;   // probes 0 .. k - 1 hold
+        if (k == 0) {
+            hi = lo;
+        } else {
+            const int64_t nlo = lo + (k - 1) * step + 1, nhi = k < 32 ? lo + k * step : hi;
+            lo = nlo;
+            hi = nhi < hi ? nhi : hi;
+        }
+    }
+    if (lane == 0) {
+        BatchPlan p;
+        p.end = lo;
+        p.tot = lo > next ? at(lo - 1) - base + size(lo - 1) : 0;
+        p.fp64 = st->fp64;
+        p.dT = dT;
+        p.err = st->err;
+        p.stop = !((double)lp[next].md <= dT);
+        *out = p;
+    }
 }
 
-
-// Entries with lo <= key <= hi, appended with their FP64 projected distance.
-__global__ void k_pair_band(const PairCand *__restrict__ p, int64_t n, float lo, float hi,
-                            const double *__restrict__ O64, int m, const int32_t *__restrict__ perm,
-                            PairExact *__restrict__ out, unsigned long long *cnt, unsigned long long cap)
+// Every cross pair of the listed leaf pairs [first, end), keyed by the FP32 projected
+// squared distance, appended behind cnt.  A warp per leaf pair.  cut: after a first
+// cut, pairs beyond the last one's band (key > hi) cannot be among the T nearest.
+__global__ void __launch_bounds__(256)
+k_bnb_cross(const float *__restrict__ O32, const int64_t *__restrict__ off, const LeafPair *__restrict__ lp,
+            int64_t first, int64_t end, int cut, const CutState *__restrict__ st, PairCand *__restrict__ out,
+            unsigned long long *cnt)
 {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    const int64_t l = first + blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (l >= end) return;   // warp-uniform
+    const float hi = cut ? st->hi : INFINITY;
+    const LeafPair pr = lp[l];
+    const int64_t a0 = off[pr.l1], na = off[pr.l1 + 1] - a0;
+    const int64_t b0 = off[pr.l2], nb = off[pr.l2 + 1] - b0;
+    for (int64_t e0 = 0; e0 < na * nb; e0 += 32) {
+        const int64_t e = e0 + lane;
+        PairCand pc;
+        pc.key = INFINITY;
+        bool in = e < na * nb;
+        if (in) {
+            const int64_t ia = e / nb, ib = e - ia * nb;
+            pc.key = pm_pd2_32(O32 + (a0 + ia) * PM_MP, O32 + (b0 + ib) * PM_MP);
+            pc.a = (int32_t)(a0 + ia);
+            pc.b = (int32_t)(b0 + ib);
+            in = !cut || pc.key <= hi;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        if (m == 0u) continue;
+        unsigned long long base = 0;
+        if (lane == 0) base = atomicAdd(cnt, (unsigned long long)__popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0) + __popc(m & ((1u << lane) - 1u));
+        if (in) out[base] = pc;
+    }
+}
+
+// The T-th smallest FP32 key of p[0, *n) by three histogram passes of 11, 11 and 10
+// bits, on the device: k_cut_hist counts the keys that share the prefix, k_cut_bin
+// extends it (and, after the last pass, forms the FP32 band that the FP64 distance
+// of the T-th pair can lie in).
+__global__ void __launch_bounds__(256)
+k_cut_hist(const PairCand *__restrict__ p, const unsigned long long *__restrict__ np, int pass,
+           const CutState *__restrict__ st, unsigned int *__restrict__ hist)
+{
+    __shared__ unsigned int h[2048];
+    const int sh = pass == 0 ? 21 : (pass == 1 ? 10 : 0), w = pass == 2 ? 10 : 11;
+    const unsigned int hiMask = pass == 0 ? 0u : (0xffffffffu << (sh + w)), prefix = pass == 0 ? 0u : st->prefix;
+    for (int i = threadIdx.x; i < (1 << w); i += blockDim.x) h[i] = 0;
+    __syncthreads();
+    const int64_t n = (int64_t)*np;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+        const unsigned int k = __float_as_uint(p[e].key);
+        if ((k & hiMask) == (prefix & hiMask)) atomicAdd(&h[(k >> sh) & ((1u << w) - 1)], 1u);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < (1 << w); i += blockDim.x)
+        if (h[i]) atomicAdd(&hist[i], h[i]);
+}
+
+__global__ void __launch_bounds__(1024)
+k_cut_bin(unsigned int *__restrict__ hist, int pass, unsigned long long T, double maxNorm, CutState *__restrict__ st)
+{
+    __shared__ unsigned long long ws[32];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int sh = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
+    const unsigned long long need = pass == 0 ? T : st->need;
+    const unsigned int prefix = pass == 0 ? 0u : st->prefix;
+    const unsigned int h0 = hist[2 * t], h1 = hist[2 * t + 1];   // (the last pass's upper half is zero)
+    unsigned long long incl = (unsigned long long)h0 + h1;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long x = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += x;
+    }
+    if (lane == 31) ws[w] = incl;
+    hist[2 * t] = 0u;   // for the next pass
+    hist[2 * t + 1] = 0u;
+    __syncthreads();
+    unsigned long long before = 0;
+    for (int i = 0; i < w; i++) before += ws[i];
+    const unsigned long long ex = before + incl - h0 - h1;
+    if (ex < need && need <= ex + h0 + h1) {
+        const bool first = need <= ex + h0;
+        const unsigned int pf = prefix | ((unsigned int)(first ? 2 * t : 2 * t + 1) << sh);
+        st->prefix = pf;
+        st->need = need - ex - (first ? 0u : h0);
+        if (pass == 2) {
+            const double tau = __dsqrt_rn((double)__uint_as_float(pf));
+            const double eps = __dadd_rn(__dadd_rn(__dmul_rn(0x1.0p-22, maxNorm), __dmul_rn(0x1.0p-19, tau)), 1e-300);
+            const double loD = __dsub_rn(tau, __dmul_rn(2.0, eps)), hiD = __dadd_rn(tau, __dmul_rn(2.0, eps));
+            st->below = loD > 0.0;
+            st->lo = loD > 0.0 ? __double2float_rd(__dmul_rn(loD, loD)) : 0.f;
+            st->hi = __double2float_ru(__dmul_rn(hiD, hiD));
+            st->nBelow = 0;
+            st->nBand = 0;
+            st->dT = fmin(st->dT, __dadd_rn(tau, eps));
+        }
+    }
+}
+
+// Keys below the band go to out in order, 2,048 pairs per block and step with one
+// atomic; keys inside it to the band list (their FP64 distances follow packed, in
+// k_cut_band).  Bound by HBM, 24 bytes per kept pair: 8.6 M pairs 35 us; one atomic
+// per kept pair and a copy back took 235.
+__global__ void __launch_bounds__(256)
+k_cut_split(const PairCand *__restrict__ p, const unsigned long long *__restrict__ np, PairCand *__restrict__ out,
+            PairExact *__restrict__ band, unsigned long long cap, CutState *__restrict__ st)
+{
+    constexpr int PER = 8;
+    __shared__ unsigned int cw[PER * 8];   // kept pairs per step of 256 and warp, then their places
+    __shared__ unsigned long long sBase;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const float lo = st->lo, hi = st->hi;
+    const bool below = st->below != 0;
+    const int64_t n = (int64_t)*np;
+    for (int64_t b0 = blockIdx.x * (int64_t)(256 * PER); b0 < n; b0 += (int64_t)gridDim.x * 256 * PER) {
+        PairCand c[PER];
+        unsigned int m[PER];
+#pragma unroll
+        for (int u = 0; u < PER; u++) {
+            const int64_t e = b0 + u * 256 + t;
+            c[u].key = INFINITY;
+            if (e < n) c[u] = p[e];
+        }
+#pragma unroll
+        for (int u = 0; u < PER; u++) {
+            const bool v = b0 + u * 256 + t < n;
+            m[u] = __ballot_sync(0xffffffffu, v && below && c[u].key < lo);
+            if (lane == 0) cw[u * 8 + w] = __popc(m[u]);
+            if (v && (!below || c[u].key >= lo) && c[u].key <= hi) {
+                const unsigned long long slot = atomicAdd(&st->nBand, 1ull);
+                if (slot < cap) {
+                    band[slot].a = c[u].a;
+                    band[slot].b = c[u].b;
+                }
+            }
+        }
+        __syncthreads();
+        if (w == 0) {
+            const unsigned int x = cw[lane], y = cw[32 + lane];
+            unsigned int ix = x, iy = y;
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned int p0 = __shfl_up_sync(0xffffffffu, ix, o), p1 = __shfl_up_sync(0xffffffffu, iy, o);
+                if (lane >= o) {
+                    ix += p0;
+                    iy += p1;
+                }
+            }
+            const unsigned int half = __shfl_sync(0xffffffffu, ix, 31), all = half + __shfl_sync(0xffffffffu, iy, 31);
+            cw[lane] = ix - x;
+            cw[32 + lane] = half + iy - y;
+            if (lane == 0) sBase = all ? atomicAdd(&st->nBelow, (unsigned long long)all) : 0ull;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < PER; u++)
+            if ((m[u] >> lane) & 1u) out[sBase + cw[u * 8 + w] + __popc(m[u] & ((1u << lane) - 1u))] = c[u];
+        __syncthreads();
+    }
+}
+
+// FP64 projected distances and ids of the band's pairs, 32 per warp.
+__global__ void __launch_bounds__(32)
+k_cut_band(PairExact *__restrict__ band, unsigned long long cap, const double *__restrict__ O64, int m,
+           const int32_t *__restrict__ perm, const CutState *__restrict__ st)
+{
+    const unsigned long long n = st->nBand < cap ? st->nBand : cap, e = blockIdx.x * 32ull + threadIdx.x;
     if (e >= n) return;
-    const PairCand c = p[e];
-    if (!(c.key >= lo && c.key <= hi)) return;
-    const unsigned long long slot = atomicAdd(cnt, 1ull);
-    if (slot >= cap) return;
-    PairExact x;
-    x.dist = pm_pdist64(O64 + (int64_t)c.a * PM_MP, O64 + (int64_t)c.b * PM_MP, m);
-    const int64_t ia = perm[c.a], ib = perm[c.b];
+    PairExact x = band[e];
+    x.dist = pm_pdist64(O64 + (int64_t)x.a * PM_MP, O64 + (int64_t)x.b * PM_MP, m);
+    const int64_t ia = perm[x.a], ib = perm[x.b];
     x.i = ia < ib ? ia : ib;
     x.j = ia < ib ? ib : ia;
-    x.a = c.a;
-    x.b = c.b;
-    out[slot] = x;
+    band[e] = x;
+}
+
+// The band's first T - nBelow entries by (FP64 projected distance, i, j) join out,
+// each placed by its rank among them; *np becomes T.
+__global__ void __launch_bounds__(128)
+k_cut_fill(const PairExact *__restrict__ band, unsigned long long cap, unsigned long long T, PairCand *__restrict__ out,
+           unsigned long long *__restrict__ np, CutState *__restrict__ st)
+{
+    __shared__ ulonglong2 s[128];   // distance bits (>= +0: they order like it), ids i 2^32 + j
+    const unsigned long long nBand = st->nBand, nBelow = st->nBelow;
+    if (nBand > cap || nBelow > T || nBelow + nBand < T) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) st->err = 1;
+        return;   // (uniform over the grid)
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        st->fp64 += nBand;
+        *np = T;
+    }
+    const unsigned long long need = T - nBelow, e = blockIdx.x * 128ull + threadIdx.x;
+    if (blockIdx.x * 128ull >= nBand) return;   // block-uniform
+    auto key = [](const PairExact &x) {
+        return make_ulonglong2((unsigned long long)__double_as_longlong(x.dist),
+                               ((unsigned long long)x.i << 32) | (unsigned long long)x.j);
+    };
+    const bool v = e < nBand;
+    const PairExact x = band[v ? e : 0];
+    const ulonglong2 kx = key(x);
+    unsigned int rank = 0;
+    for (unsigned long long f0 = 0; f0 < nBand; f0 += 128) {
+        __syncthreads();
+        s[threadIdx.x] = f0 + threadIdx.x < nBand ? key(band[f0 + threadIdx.x]) : make_ulonglong2(~0ull, ~0ull);
+        __syncthreads();
+#pragma unroll 4
+        for (int f = 0; f < 128; f++) rank += s[f].x < kx.x || (s[f].x == kx.x && s[f].y < kx.y) ? 1 : 0;
+    }
+    if (v && rank < need) {
+        PairCand pc;
+        pc.key = 0.f;
+        pc.a = x.a;
+        pc.b = x.b;
+        out[nBelow + rank] = pc;
+    }
 }
 
 template <class T> pmlsh_status dalloc(T **p, size_t count)
@@ -855,6 +1196,17 @@ pmlsh_status pair_kth(const PairCand *p, int64_t n, int64_t rank, unsigned int *
     return PMLSH_OK;
 }
 
+// Entries of p[0, n) with key <= thr into out (at most cap, counted in cnt) with
+// their FP64 distance (original space, or projected) and ids.
+void launch_pair_collect(const pmlsh_index *ix, const PairCand *p, int64_t n, float thr, int useProj, PairExact *out,
+                         unsigned long long *cnt, unsigned long long cap, cudaStream_t st)
+{
+    const unsigned grid = (unsigned)std::min<int64_t>((n + 255) / 256, 16 * 152);
+    PM_LAUNCH("k_pair_pick", st, k_pair_pick<<<grid, 256, 0, st>>>(p, n, thr, out, cnt, cap));
+    PM_LAUNCH("k_pair_exact", st, k_pair_exact<<<(unsigned)((cap + 31) / 32), 32, 0, st>>>(
+        ix->X, ix->ld, ix->d, ix->O64, ix->m, useProj, ix->perm, out, cnt, cap));
+}
+
 // Exact top-k merge: the current list `top` (sorted by (dist, i, j), FP64
 // distances, size kc <= k) and the candidate buffer p[0, n) with FP32
 // original-space squared distances.  A candidate can enter only if its FP32
@@ -884,8 +1236,7 @@ pmlsh_status pair_merge(TopK &top, int k, const PairCand *p, int64_t n, const pm
     if (!std::isinf(thr) && (double)thr32 < thr) thr32 = nextafterf(thr32, INFINITY);
     PM_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), st));
     const unsigned long long cap = PAIR_SORT_CAP - (unsigned long long)top.v.size();
-    PM_LAUNCH("k_pair_collect", st, k_pair_collect<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-        p, n, thr32, ix->X, ix->ld, ix->d, ix->O64, ix->m, 0, ix->perm, scratch + top.v.size(), cnt, cap));
+    launch_pair_collect(ix, p, n, thr32, 0, scratch + top.v.size(), cnt, cap, st);
     PM_CUDA(cudaGetLastError());
     unsigned long long got = 0;
     PM_CUDA(cudaMemcpyAsync(&got, cnt, sizeof(got), cudaMemcpyDeviceToHost, st));
@@ -923,9 +1274,7 @@ pmlsh_status pair_truncate(PairCand *p, int64_t n, int64_t need, const pmlsh_ind
     const double eps = 0x1.0p-22 * ix->maxNorm + 0x1.0p-19 * tau + 1e-300;
     const float hiK = (float)((tau + 2 * eps) * (tau + 2 * eps));
     PM_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), st));
-    PM_LAUNCH("k_pair_collect", st, k_pair_collect<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-        p, n, nextafterf(hiK, INFINITY), ix->X, ix->ld, ix->d, ix->O64, ix->m, 1, ix->perm, scratch, cnt,
-        PAIR_SORT_CAP));
+    launch_pair_collect(ix, p, n, nextafterf(hiK, INFINITY), 1, scratch, cnt, PAIR_SORT_CAP, st);
     unsigned long long got = 0;
     PM_CUDA(cudaMemcpyAsync(&got, cnt, sizeof(got), cudaMemcpyDeviceToHost, st));
     PM_CUDA(cudaStreamSynchronize(st));
@@ -952,62 +1301,6 @@ pmlsh_status pair_truncate(PairCand *p, int64_t n, int64_t need, const pmlsh_ind
     return PMLSH_OK;
 }
 
-
-// The T candidates of p[0, n) with the smallest (FP64 projected distance,
-// i, j) go to out[0, T) (any order): the T-th FP32 key by radix select;
-// keys below its FP32 band are in, keys inside the band are ordered by
-// (FP64 projected distance, i, j) and the first ones fill up to T.  tauHi:
-// an upper bound of the T-th FP64 projected distance.
-pmlsh_status pair_select(const PairCand *p, int64_t n, int64_t T, PairCand *out, const pmlsh_index *ix,
-                         unsigned int *hist, PairExact *scratch, unsigned long long *cnt, int64_t *fp64,
-                         double *tauHi, cudaStream_t st)
-{
-    float K;
-    PM_TRY(pair_kth(p, n, T, hist, &K, st));
-    const double tau = std::sqrt((double)K);
-    const double eps = 0x1.0p-22 * ix->maxNorm + 0x1.0p-19 * tau + 1e-300;
-    const double loD = tau - 2 * eps;
-    float lo = loD > 0 ? (float)(loD * loD) : 0.f;
-    if (loD > 0 && (double)lo > loD * loD) lo = nextafterf(lo, -INFINITY);
-    if (!(loD > 0)) lo = 0.f;
-    float hi = (float)((tau + 2 * eps) * (tau + 2 * eps));
-    if ((double)hi < (tau + 2 * eps) * (tau + 2 * eps)) hi = nextafterf(hi, INFINITY);
-    PM_CUDA(cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), st));
-    if (loD > 0)
-        PM_LAUNCH("k_pair_below", st, k_pair_below<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(p, n, lo, out, cnt));
-    PM_LAUNCH("k_pair_band", st, k_pair_band<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-        p, n, loD > 0 ? lo : -INFINITY, hi, ix->O64, ix->m, ix->perm, scratch, cnt + 1, PAIR_SORT_CAP));
-    PM_CUDA(cudaGetLastError());
-    unsigned long long hc[2];
-    PM_CUDA(cudaMemcpyAsync(hc, cnt, sizeof(hc), cudaMemcpyDeviceToHost, st));
-    PM_CUDA(cudaStreamSynchronize(st));
-    const int64_t nBelow = (int64_t)hc[0], nBand = (int64_t)hc[1];
-    if (nBand > PAIR_SORT_CAP || nBelow > T || nBelow + nBand < T) {
-        pm_set_error("closest pairs: %lld candidates inside the FP32 band at the T-th projected distance "
-                     "(capacity %d)", (long long)nBand, PAIR_SORT_CAP);
-        return PMLSH_EINTERNAL;
-    }
-    *fp64 += nBand;
-    int P = 1;
-    while (P < (int)nBand) P <<= 1;
-    if (nBand > 0)
-        PM_LAUNCH("k_pair_sort", st, k_pair_sort<<<1, 1024, (size_t)P * sizeof(PairExact), st>>>(scratch, (int)nBand));
-    std::vector<PairExact> v(nBand);
-    PM_CUDA(cudaMemcpyAsync(v.data(), scratch, nBand * sizeof(PairExact), cudaMemcpyDeviceToHost, st));
-    PM_CUDA(cudaStreamSynchronize(st));
-    const int64_t need = T - nBelow;
-    std::vector<PairCand> kept(need);
-    for (int64_t e = 0; e < need; e++) {
-        kept[e].key = 0.f;
-        kept[e].a = v[e].a;
-        kept[e].b = v[e].b;
-    }
-    if (need > 0)
-        PM_CUDA(cudaMemcpyAsync(out + nBelow, kept.data(), need * sizeof(PairCand), cudaMemcpyHostToDevice, st));
-    PM_CUDA(cudaStreamSynchronize(st));
-    *tauHi = tau + eps;
-    return PMLSH_OK;
-}
 
 }  // namespace
 
@@ -1446,9 +1739,13 @@ pmlsh_status pm_closest_pair_bnb(pmlsh_index *ix, const pmlsh_cp_opts *o, int64_
     unsigned int *hist;
     PairExact *scratch;
     unsigned long long *cnt;
+    CutState *state;
+    BatchPlan *planD;
     PM_TRY(mem.get(&hist, 2048));
     PM_TRY(mem.get(&scratch, PAIR_SORT_CAP));
     PM_TRY(mem.get(&cnt, 4));
+    PM_TRY(mem.get(&state, 1));
+    PM_TRY(mem.get(&planD, 1));
     PM_TRY(pm_allow_max_dyn_smem((const void *)k_pair_sort));
     // 1. self-joins
     std::vector<int64_t> pairOff(L + 1, 0);
@@ -1457,29 +1754,64 @@ pmlsh_status pm_closest_pair_bnb(pmlsh_index *ix, const pmlsh_cp_opts *o, int64_
         pairOff[l + 1] = pairOff[l] + s * (s - 1) / 2;
     }
     const int64_t nSelf = pairOff[L];
-    // candidate buffer: up to T kept pairs followed by a batch
+    // two candidate buffers, each up to T kept pairs followed by a batch: a cut
+    // reads one and writes the other.  cnt[0]: pairs in the current one.
     const int64_t batchCap = std::max<int64_t>((int64_t)1 << 24, nSelf);
-    PairCand *buf, *sel;
+    PairCand *buf, *other;
     int64_t *dPairOff;
     PM_TRY(mem.get(&buf, (size_t)(T + batchCap)));
-    PM_TRY(mem.get(&sel, (size_t)T));
+    PM_TRY(mem.get(&other, (size_t)(T + batchCap)));
     PM_TRY(mem.get(&dPairOff, L + 1));
     PM_CUDA(cudaMemcpyAsync(dPairOff, pairOff.data(), (L + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, st));
     if (nSelf > 0)
         PM_LAUNCH("k_bnb_selfjoin", st, k_bnb_selfjoin<<<(unsigned)L, 128, 0, st>>>(ix->O32, ix->leafOff, dPairOff, buf));
     PM_CUDA(cudaGetLastError());
-    int64_t nBuf = nSelf, fp64 = 0;
+    CutState state0;
+    std::memset(&state0, 0, sizeof(state0));
+    state0.dT = INFINITY;
+    const unsigned long long nSelfU = (unsigned long long)nSelf;
+    PM_CUDA(cudaMemcpyAsync(state, &state0, sizeof(state0), cudaMemcpyHostToDevice, st));
+    PM_CUDA(cudaMemcpyAsync(cnt, &nSelfU, sizeof(nSelfU), cudaMemcpyHostToDevice, st));
+    PM_CUDA(cudaMemsetAsync(hist, 0, 2048 * sizeof(unsigned int), st));
+    int64_t nBuf = nSelf, fp64 = 0;   // (the pairs in buf before any that a cut's band left out)
     double dT = INFINITY;   // upper bound of the T-th projected distance
+    bool cutDone = false;
+    // the T pairs of buf with the smallest (FP64 projected distance, i, j), entirely
+    // on the device (its bound dT and errors are read with the next batch's plan)
     auto cut = [&]() -> pmlsh_status {
         if (nBuf <= T) return PMLSH_OK;
-        double tauHi = INFINITY;
-        PM_TRY(pair_select(buf, nBuf, T, sel, ix, hist, scratch, cnt, &fp64, &tauHi, st));
-        PM_CUDA(cudaMemcpyAsync(buf, sel, T * sizeof(PairCand), cudaMemcpyDeviceToDevice, st));
+        const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>(8 * 152, (nBuf + 2047) / 2048));
+        for (int pass = 0; pass < 3; pass++) {
+            PM_LAUNCH("k_cut_hist", st, k_cut_hist<<<g, 256, 0, st>>>(buf, cnt, pass, state, hist));
+            PM_LAUNCH("k_cut_bin", st, k_cut_bin<<<1, 1024, 0, st>>>(hist, pass, (unsigned long long)T, ix->maxNorm, state));
+        }
+        PM_LAUNCH("k_cut_split", st, k_cut_split<<<g, 256, 0, st>>>(buf, cnt, other, scratch, PAIR_SORT_CAP, state));
+        PM_LAUNCH("k_cut_band", st, k_cut_band<<<PAIR_SORT_CAP / 32, 32, 0, st>>>(scratch, PAIR_SORT_CAP, ix->O64, ix->m,
+                                                                                 ix->perm, state));
+        PM_LAUNCH("k_cut_fill", st, k_cut_fill<<<PAIR_SORT_CAP / 128, 128, 0, st>>>(scratch, PAIR_SORT_CAP,
+                                                                    (unsigned long long)T, other, cnt, state));
+        PM_CUDA(cudaGetLastError());
+        std::swap(buf, other);
         nBuf = T;
-        dT = std::min(dT, tauHi);
+        cutDone = true;
+        return PMLSH_OK;
+    };
+    // the device's dT, band decisions and errors
+    auto read_state = [&]() -> pmlsh_status {
+        CutState h;
+        PM_CUDA(cudaMemcpyAsync(&h, state, sizeof(h), cudaMemcpyDeviceToHost, st));
+        PM_CUDA(cudaStreamSynchronize(st));
+        dT = h.dT;
+        fp64 = (int64_t)h.fp64;
+        if (h.err) {
+            pm_set_error("closest pairs: %lld candidates inside the FP32 band at the T-th projected distance "
+                         "(capacity %d)", (long long)h.nBand, PAIR_SORT_CAP);
+            return PMLSH_EINTERNAL;
+        }
         return PMLSH_OK;
     };
     PM_TRY(cut());
+    PM_TRY(read_state());
     // 2./3. leaf pairs in bands of Mindist, (lo, hi]: each band's pairs in
     // ascending (Mindist, l1, l2), cut to the T nearest after each batch;
     // the search ends at the first leaf pair whose Mindist exceeds the T-th
@@ -1489,114 +1821,128 @@ pmlsh_status pm_closest_pair_bnb(pmlsh_index *ix, const pmlsh_cp_opts *o, int64_
     // distance), so that the leaf pairs listed stay few; each further band
     // quadruples the quantile.
     std::vector<double> F;
-    PM_TRY(pm_distance_sample(ix, (int64_t)1 << 16, ix->seed + 8, F, st));
+    PM_TRY(pm_distance_sample(ix, (int64_t)1 << 16, ix->seed + 8, F, st, false));
     const double pT = (double)T / (double)P;
     double pBand = std::min(1.0, 4.0 * pT + 64.0 / (double)F.size());
     auto quantile = [&](double p) -> double {
         if (p >= 1.0 || F.empty()) return INFINITY;
         const int64_t r = std::min<int64_t>((int64_t)F.size() - 1, (int64_t)std::ceil(p * (double)F.size()));
+        std::nth_element(F.begin(), F.begin() + r, F.end());
         return F[r];
     };
     double bandHi = quantile(pBand);
     float lo32 = -INFINITY;   // FP32 end of the previous band: bands are disjoint in FP32
-    LeafPair *dlp;
-    const unsigned long long lpCap = (unsigned long long)std::max<int64_t>(1, L * (L - 1) / 2);
-    PM_TRY(mem.get(&dlp, (size_t)lpCap));
-    int2 *dPairs;
-    int64_t *dOff;
-    const size_t lpBatch = (size_t)1 << 16;
-    PM_TRY(mem.get(&dPairs, lpBatch));
-    PM_TRY(mem.get(&dOff, lpBatch));
-    unsigned long long *keyA = nullptr, *keyB = nullptr;   // device sort of the listed leaf pairs
+    const int64_t lpBatch = (int64_t)1 << 16;
+    // per listed leaf pair: the pair, two sort keys, the prefix of the cross pairs
+    LeafPair *dlp = nullptr;
+    unsigned long long *keyA = nullptr, *keyB = nullptr;
     unsigned int *rsHist = nullptr;
-    unsigned long long keyCap = 0;
-    int64_t examined = 0, crossPairs = 0, listed = 0;
+    int64_t *pre = nullptr, *blk = nullptr;
+    unsigned long long lpCap = 0, keyCap = 0;
+    const dim3 mdGrid((unsigned)((L + BM_T - 1) / BM_T),
+                      (unsigned)std::max<int64_t>(1, std::min<int64_t>(64, 16 * 152 / ((L + BM_T - 1) / BM_T))));
+    int64_t examined = 0, listed = 0;
     for (;;) {
         const double hiCut = std::min(bandHi, dT);
-        PM_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), st));
         // the band is (lo32, hi32] in FP32 Mindist, hi32 >= hiCut
         const float hi32 = std::isinf(hiCut) ? INFINITY : nextafterf((float)hiCut, INFINITY);
-        if (L > 1)
-            PM_LAUNCH("k_bnb_mindist", st, k_bnb_mindist<<<(unsigned)L, 256, 0, st>>>(ix->leafMeta, ix->s, L, lo32,
-                                                                                       hi32, dlp, cnt, lpCap));
-        PM_CUDA(cudaGetLastError());
+        // listed up to the buffer's size, and again into one of the band's size if
+        // that was too short (a list for every leaf pair took 12 bytes times
+        // L (L - 1) / 2)
         unsigned long long nlp = 0;
-        PM_CUDA(cudaMemcpyAsync(&nlp, cnt, sizeof(nlp), cudaMemcpyDeviceToHost, st));
-        PM_CUDA(cudaStreamSynchronize(st));
-        const bool gpuSort = L <= LP_GPU_MAX_L && nlp > 1;
-        if (gpuSort) {
-            // ascending (Mindist, l1, l2) by the device radix sort
-            if (nlp > keyCap) {
-                PM_TRY(mem.get(&keyA, (size_t)nlp));
-                PM_TRY(mem.get(&keyB, (size_t)nlp));
-                PM_TRY(mem.get(&rsHist, (size_t)256 * ((nlp + RS_THREADS * RS_ITEMS - 1) / (RS_THREADS * RS_ITEMS))));
-                keyCap = nlp;
-            }
-            const int64_t nl = (int64_t)nlp;
-            const int nb = (int)((nl + RS_THREADS * RS_ITEMS - 1) / (RS_THREADS * RS_ITEMS));
-            const unsigned g = (unsigned)((nl + 255) / 256);
-            PM_LAUNCH("k_lp_key", st, k_lp_key<<<g, 256, 0, st>>>(dlp, nl, L, keyA));
-            unsigned long long *src = keyA, *dst = keyB;
-            for (int shift = 0; shift < 64; shift += 8) {
-                PM_LAUNCH("k_rs_hist", st, k_rs_hist<<<(unsigned)nb, RS_THREADS, 0, st>>>(src, nl, shift, rsHist, nb));
-                PM_LAUNCH("k_rs_scan", st, k_rs_scan<<<1, 1024, 0, st>>>(rsHist, (int64_t)256 * nb));
-                PM_LAUNCH("k_rs_scatter", st, k_rs_scatter<<<(unsigned)nb, RS_THREADS, 0, st>>>(src, dst, nl, shift,
-                                                                                              rsHist, nb));
-                std::swap(src, dst);
+        for (int attempt = 0; L > 1 && attempt < 2; attempt++) {
+            if (!dlp || attempt == 1) {
+                lpCap = attempt == 1 ? nlp : (unsigned long long)std::min<int64_t>(L * (L - 1) / 2, (int64_t)1 << 23);
+                PM_TRY(mem.get(&dlp, (size_t)lpCap));
             }
             PM_CUDA(cudaMemsetAsync(cnt + 1, 0, sizeof(unsigned long long), st));
-            PM_LAUNCH("k_lp_decode", st, k_lp_decode<<<g, 256, 0, st>>>(src, nl, L, dlp, (int *)(cnt + 1)));
+            PM_LAUNCH("k_bnb_mindist", st, k_bnb_mindist<<<mdGrid, BM_T, 0, st>>>(ix->leafMeta, ix->s, L, lo32, hi32,
+                                                                                  dlp, cnt + 1, lpCap));
+            PM_CUDA(cudaGetLastError());
+            PM_CUDA(cudaMemcpyAsync(&nlp, cnt + 1, sizeof(nlp), cudaMemcpyDeviceToHost, st));
+            PM_CUDA(cudaStreamSynchronize(st));
+            if (nlp <= lpCap) break;
+        }
+        const int64_t nl = (int64_t)nlp;
+        const bool gpuSort = L <= LP_GPU_MAX_L;
+        if (nlp > keyCap) {
+            PM_TRY(mem.get(&pre, (size_t)nlp));
+            PM_TRY(mem.get(&blk, (size_t)(nl + 1023) / 1024));
+            if (gpuSort) {
+                PM_TRY(mem.get(&keyA, (size_t)nlp));
+                PM_TRY(mem.get(&keyB, (size_t)nlp));
+                PM_TRY(mem.get(&rsHist, (size_t)256 * ((nlp + RS_THREADS * RS_ITEMS - 1) / (RS_THREADS * RS_ITEMS)) + 256));
+            }
+            keyCap = nlp;
+        }
+        if (nl > 0) {
+            if (gpuSort) {
+                // ascending (Mindist, l1, l2) by the device radix sort
+                const int nb = (int)((nl + RS_THREADS * RS_ITEMS - 1) / (RS_THREADS * RS_ITEMS));
+                const unsigned g = (unsigned)((nl + 255) / 256);
+                unsigned int *total = rsHist + (size_t)256 * nb;
+                PM_LAUNCH("k_lp_key", st, k_lp_key<<<g, 256, 0, st>>>(dlp, nl, L, keyA));
+                unsigned long long *src = keyA, *dst = keyB;
+                for (int shift = 0; shift < 64; shift += 8) {
+                    // (digits of the pair's rank that no rank reaches)
+                    if (shift < 32 && (uint64_t)(L * (L - 1) / 2) <= ((uint64_t)1 << shift)) continue;
+                    PM_LAUNCH("k_rs_hist", st, k_rs_hist<<<(unsigned)nb, RS_THREADS, 0, st>>>(src, nl, shift, rsHist, nb));
+                    PM_LAUNCH("k_rs_scan", st, k_rs_scan<<<256, 256, 0, st>>>(rsHist, nb, total));
+                    PM_LAUNCH("k_rs_scatter", st, k_rs_scatter<<<(unsigned)nb, RS_THREADS, 0, st>>>(src, dst, nl, shift,
+                                                                                                  rsHist, total, nb));
+                    std::swap(src, dst);
+                }
+                PM_CUDA(cudaMemsetAsync(cnt + 3, 0, sizeof(unsigned long long), st));
+                PM_LAUNCH("k_lp_decode", st, k_lp_decode<<<g, 256, 0, st>>>(src, nl, L, dlp, (int *)(cnt + 3)));
+                PM_CUDA(cudaGetLastError());
+                unsigned long long badH = 0;
+                PM_CUDA(cudaMemcpyAsync(&badH, cnt + 3, sizeof(badH), cudaMemcpyDeviceToHost, st));
+                PM_CUDA(cudaStreamSynchronize(st));
+                if (badH != 0) {
+                    pm_set_error("closest pairs: the device sort of %llu leaf pairs failed its check (%llu)", nlp, badH);
+                    return PMLSH_EINTERNAL;
+                }
+            } else {
+                std::vector<LeafPair> lps(nlp);
+                PM_CUDA(cudaMemcpyAsync(lps.data(), dlp, nlp * sizeof(LeafPair), cudaMemcpyDeviceToHost, st));
+                PM_CUDA(cudaStreamSynchronize(st));
+                std::sort(lps.begin(), lps.end(), [](const LeafPair &x, const LeafPair &y) {
+                    if (x.md != y.md) return x.md < y.md;
+                    if (x.l1 != y.l1) return x.l1 < y.l1;
+                    return x.l2 < y.l2;
+                });
+                PM_CUDA(cudaMemcpyAsync(dlp, lps.data(), nlp * sizeof(LeafPair), cudaMemcpyHostToDevice, st));
+                PM_CUDA(cudaStreamSynchronize(st));
+            }
+            PM_LAUNCH("k_lp_size", st, k_lp_size<<<(unsigned)((nl + 1023) / 1024), 1024, 0, st>>>(dlp, nl, ix->leafOff, pre, blk));
+            PM_LAUNCH("k_lp_scan", st, k_lp_scan<<<1, 1024, 0, st>>>(blk, (int)((nl + 1023) / 1024)));
             PM_CUDA(cudaGetLastError());
         }
-        std::vector<LeafPair> lps(nlp);
-        PM_CUDA(cudaMemcpyAsync(lps.data(), dlp, nlp * sizeof(LeafPair), cudaMemcpyDeviceToHost, st));
-        if (gpuSort) {
-            unsigned long long badH = 0;
-            PM_CUDA(cudaMemcpyAsync(&badH, cnt + 1, sizeof(badH), cudaMemcpyDeviceToHost, st));
-            PM_CUDA(cudaStreamSynchronize(st));
-            if (badH != 0) {
-                pm_set_error("closest pairs: the device sort of %llu leaf pairs failed its check (%llu)", nlp, badH);
-                return PMLSH_EINTERNAL;
-            }
-        } else {
-            PM_CUDA(cudaStreamSynchronize(st));
-            std::sort(lps.begin(), lps.end(), [](const LeafPair &x, const LeafPair &y) {
-                if (x.md != y.md) return x.md < y.md;
-                if (x.l1 != y.l1) return x.l1 < y.l1;
-                return x.l2 < y.l2;
-            });
-        }
-        listed += (int64_t)nlp;
-        size_t next = 0;
+        listed += nl;
         bool stop = false;
-        while (next < lps.size()) {
-            if ((double)lps[next].md > dT) { stop = true; break; }   // no pair under it can beat the T-th
-            std::vector<int2> bp;
-            std::vector<int64_t> bo;
-            int64_t tot = 0;
-            while (next < lps.size() && bp.size() < lpBatch && (double)lps[next].md <= dT) {
-                const int64_t na = ix->leafOffH[lps[next].l1 + 1] - ix->leafOffH[lps[next].l1];
-                const int64_t nb = ix->leafOffH[lps[next].l2 + 1] - ix->leafOffH[lps[next].l2];
-                if (tot > 0 && tot + na * nb > batchCap) break;
-                bp.push_back(make_int2(lps[next].l1, lps[next].l2));
-                bo.push_back(nBuf + tot);
-                tot += na * nb;
-                next++;
-            }
-            if (tot > batchCap) {
+        for (int64_t next = 0; next < nl;) {
+            // the next batch (one read of the device's decisions)
+            BatchPlan plan;
+            PM_LAUNCH("k_bnb_plan", st, k_bnb_plan<<<1, 32, 0, st>>>(dlp, pre, blk, ix->leafOff, nl, next, lpBatch,
+                                                                     batchCap, state, planD));
+            PM_CUDA(cudaMemcpyAsync(&plan, planD, sizeof(plan), cudaMemcpyDeviceToHost, st));
+            PM_CUDA(cudaStreamSynchronize(st));
+            dT = plan.dT;
+            if (plan.err) return read_state();
+            if (plan.stop) { stop = true; break; }   // no pair under it can beat the T-th
+            if (plan.tot > batchCap) {
                 pm_set_error("closest pairs: one leaf pair holds more pairs than the batch capacity");
                 return PMLSH_EINTERNAL;
             }
-            PM_CUDA(cudaMemcpyAsync(dPairs, bp.data(), bp.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
-            PM_CUDA(cudaMemcpyAsync(dOff, bo.data(), bo.size() * sizeof(int64_t), cudaMemcpyHostToDevice, st));
-            PM_LAUNCH("k_bnb_cross", st, k_bnb_cross<<<(unsigned)bp.size(), 256, 0, st>>>(ix->O32, ix->leafOff, dPairs,
-                                                                                            dOff, buf));
+            PM_LAUNCH("k_bnb_cross", st, k_bnb_cross<<<(unsigned)((plan.end - next + 7) / 8), 256, 0, st>>>(
+                ix->O32, ix->leafOff, dlp, next, plan.end, cutDone ? 1 : 0, state, buf, cnt));
             PM_CUDA(cudaGetLastError());
-            nBuf += tot;
-            examined += (int64_t)bp.size();
-            crossPairs += tot;
+            nBuf += plan.tot;
+            examined += plan.end - next;
+            next = plan.end;
             PM_TRY(cut());
         }
+        PM_TRY(read_state());
         // done when this band reached dT (every later pair has Mindist > dT)
         // or covered everything
         if (stop || std::isinf(bandHi) || dT <= bandHi) break;
@@ -1631,6 +1977,5 @@ pmlsh_status pm_closest_pair_bnb(pmlsh_index *ix, const pmlsh_cp_opts *o, int64_
         stats->T = T;
         stats->gamma = o->gamma;
     }
-    (void)crossPairs;
     return PMLSH_OK;
 }

@@ -202,9 +202,10 @@ pmlsh_status pm_closest_pair_bnb(pmlsh_index *ix, const pmlsh_cp_opts *o, int64_
                              pmlsh_cp_stats *stats, cudaStream_t st);
 
 // Cost model of Sec. 4.2 (cost.cu)
-// Sorted FP64 projected distances of `npairs` sampled pairs (host vector).
+// FP64 projected distances of `npairs` sampled pairs (host vector), sorted or in
+// the order of the sample.
 pmlsh_status pm_distance_sample(const pmlsh_index *ix, int64_t npairs, uint64_t seed, std::vector<double> &out,
-                                cudaStream_t st);
+                                cudaStream_t st, bool sorted = true);
 // CC and sum of Pr[e] over the leaves for each radius rq[r]; F and rq on the
 // host, F sorted ascending.
 pmlsh_status pm_cost_model(const pmlsh_index *ix, const double *F, int64_t nF, const double *rq, int64_t nr,

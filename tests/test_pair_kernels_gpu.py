@@ -61,3 +61,25 @@ def test_more_entrants_than_the_list_holds():
     X = rng.standard_normal((900, 6)).astype(np.float32)
     A = oracle.gen_projection(4, 6, 6).astype(np.float32)
     _check(X, A, 1024, math.inf, 10 ** 9, 16)
+
+
+def _bnb(X, A, k, T, leaf):
+    ix = pm.Index(torch.from_numpy(X).cuda(), m=A.shape[0], leaf_size=leaf, proj=A)
+    got = ix.closest_pairs_bnb(k=k, T=T)
+    ix.close()
+    rp, rd = oracle.cp_bnb(X, A, T, k)[:2]
+    return got, np.asarray(rp), np.asarray(rd)
+
+
+# leaf counts around the 128 x 32 tiles of Mindist; T below, at and above the self
+# pairs (a first cut, none, cuts in the batches)
+@pytest.mark.parametrize("n,clusters,leaf,T", [
+    (40, 2, 16, 30), (300, 5, 16, 200), (700, 3, 16, 1500), (1500, 6, 16, 4000), (1500, 6, 128, 4000),
+])
+def test_branch_and_bound_tiles(n, clusters, leaf, T):
+    X, _, _, _ = datagen.mixture(n, 10, clusters, 1.0, seed=n)
+    A = oracle.gen_projection(6, 15, 10).astype(np.float32)
+    got, rp, rd = _bnb(X, A, 12, T, leaf)
+    assert got["pairs"].tolist() == rp.tolist()
+    assert np.array_equal(got["dists"], rd.astype(np.float32))
+    assert got["stats"]["count"] == T
