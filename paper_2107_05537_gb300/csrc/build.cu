@@ -970,14 +970,15 @@ void pm_free_index(pmlsh_index *ix)
 void pm_release_work(KnnWork &w)
 {
     DevBuf *bufs[] = {&w.Qd, &w.qp32, &w.qp64, &w.qnorm, &w.qpiv, &w.order, &w.keys,
-                      &w.keys2, &w.vals2, &w.sortTmp, &w.qstate, &w.thr, &w.blkCnt,
-                      &w.blkLeaves, &w.cntSure, &w.cntBand, &w.bandQ, &w.bandPos,
-                      &w.bandIn, &w.bandCnt, &w.partD, &w.partI, &w.partSeen, &w.bandInQ,
-                      &w.outD64, &w.outIds, &w.outErr, &w.dk, &w.flags, &w.selBuf,
+                      &w.vals2, &w.sortTmp, &w.qstate, &w.thr, &w.blkCnt,
+                      &w.blkLeaves, &w.cntSure, &w.bandQ, &w.bandPos,
+                      &w.bandIn, &w.partD, &w.partI, &w.partSeen, &w.bandInQ,
+                      &w.outIds, &w.dk, &w.flags, &w.selBuf,
                       &w.selOff, &w.selCnt, &w.selTau, &w.active, &w.misc, &w.blkMask,
-                      &w.recheck, &w.leafBits, &w.fullBits, &w.cntPart, &w.cntTight, &w.subIdx, &w.subThr, &w.subBits, &w.qpca};
+                      &w.recheck, &w.leafBits, &w.fullBits, &w.cntTight, &w.subIdx, &w.subThr, &w.subBits, &w.qpca};
     for (DevBuf *b : bufs) b->release();
     w.stage.release();
+    w.outStage.release();
 }
 
 pmlsh_status HostBuf::reserve(size_t b)

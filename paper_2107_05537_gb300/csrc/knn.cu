@@ -2370,13 +2370,11 @@ void knn_work_needs(const pmlsh_index *ix, int64_t nq, int k, int precision,
         {&KnnWork::Qd, nq * ld * 4}, {&KnnWork::qp64, nq * PM_MP * 8}, {&KnnWork::qp32, nq * PM_MP * 4},
         {&KnnWork::qnorm, nq * 8}, {&KnnWork::qpiv, nq * PM_MAX_PIVOTS * 4}, {&KnnWork::keys, nq * 4},
         {&KnnWork::order, nq * 4}, {&KnnWork::qpca, nq * (PM_PCA + 1) * 4},
-        {&KnnWork::qstate, nq * 8}, {&KnnWork::outIds, nq * k * 8}, {&KnnWork::outD64, nq * k * 4},
-        {&KnnWork::outErr, nq * k * 4}, {&KnnWork::active, nq * 4}, {&KnnWork::thr, nq * (int64_t)sizeof(Thr)},
-        {&KnnWork::cntSure, nq * 4}, {&KnnWork::cntBand, nq * 4}, {&KnnWork::cntPart, nq * 4},
-        {&KnnWork::cntTight, nq * 8},
-        {&KnnWork::bandCnt, nq * 4}, {&KnnWork::bandIn, nq * 4}, {&KnnWork::bandInQ, nq * BCAP * 4},
+        {&KnnWork::qstate, nq * 8}, {&KnnWork::outIds, nq * k * 16}, {&KnnWork::active, nq * 4}, {&KnnWork::thr, nq * (int64_t)sizeof(Thr)},
+        {&KnnWork::cntSure, 4 * nq * 4}, {&KnnWork::cntTight, nq * 8},
+        {&KnnWork::bandIn, nq * 4}, {&KnnWork::bandInQ, nq * BCAP * 4},
         {&KnnWork::bandQ, ((int64_t)1 << 20) * 4}, {&KnnWork::bandPos, ((int64_t)1 << 20) * 4},
-        {&KnnWork::flags, (nq + 8) * 4}, {&KnnWork::dk, nq * 8}, {&KnnWork::leafBits, nq * W32 * 4},
+        {&KnnWork::flags, (nq + 8) * 4}, {&KnnWork::dk, 2 * nq * 8}, {&KnnWork::leafBits, nq * W32 * 4},
         {&KnnWork::fullBits, nq * W32 * 4},
         {&KnnWork::recheck, tc ? ((int64_t)1 << 23) * 8 : 0},
         {&KnnWork::blkCnt, nlist * 4}, {&KnnWork::blkLeaves, nlist * L * 16},
@@ -2416,12 +2414,12 @@ int64_t pm_knn_work_growth(const pmlsh_index *ix, int64_t nq, int k, int precisi
 
 int64_t pm_work_resident(const KnnWork &w)
 {
-    const DevBuf *bufs[] = {&w.Qd, &w.qp32, &w.qp64, &w.qnorm, &w.qpiv, &w.order, &w.keys, &w.keys2, &w.vals2,
-                            &w.sortTmp, &w.qstate, &w.thr, &w.blkCnt, &w.blkLeaves, &w.cntSure, &w.cntBand,
-                            &w.bandQ, &w.bandPos, &w.bandIn, &w.bandCnt, &w.partD, &w.partI, &w.partSeen,
-                            &w.bandInQ, &w.outD64, &w.outIds, &w.outErr, &w.dk, &w.flags, &w.selBuf, &w.selOff,
+    const DevBuf *bufs[] = {&w.Qd, &w.qp32, &w.qp64, &w.qnorm, &w.qpiv, &w.order, &w.keys, &w.vals2,
+                            &w.sortTmp, &w.qstate, &w.thr, &w.blkCnt, &w.blkLeaves, &w.cntSure, 
+                            &w.bandQ, &w.bandPos, &w.bandIn, &w.partD, &w.partI, &w.partSeen,
+                            &w.bandInQ, &w.outIds, &w.dk, &w.flags, &w.selBuf, &w.selOff,
                             &w.selCnt, &w.selTau, &w.active, &w.misc, &w.blkMask, &w.recheck, &w.leafBits,
-                            &w.fullBits, &w.cntPart, &w.cntTight, &w.subIdx, &w.subThr, &w.subBits, &w.qpca};
+                            &w.fullBits, &w.cntTight, &w.subIdx, &w.subThr, &w.subBits, &w.qpca};
     int64_t b = 0;
     for (const DevBuf *p : bufs) b += (int64_t)p->bytes;
     return b;
@@ -2489,22 +2487,29 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
     // memory, else to scratch copied out at the end
     const bool idev = pm_is_device_ptr(ids), ddev = pm_is_device_ptr(dists);
     const bool edev = err != nullptr && pm_is_device_ptr(err);
-    int64_t *oIds = idev ? ids : grow<int64_t>(w.outIds, (size_t)nq * k, s);
-    float *oD = ddev ? dists : grow<float>(w.outD64, (size_t)nq * k, s);
-    float *oE = edev ? err : grow<float>(w.outErr, (size_t)nq * k, s);
+    // (one buffer: ids, distances, errors)
+    const size_t nk = (size_t)nq * k, outBytes = nk * (8 + 4 + 4);
+    int64_t *oBuf = grow<int64_t>(w.outIds, nk * 2, s);
+    int64_t *oIds = idev ? ids : oBuf;
+    float *oD = ddev ? dists : (float *)(oBuf + nk);
+    float *oE = edev ? err : (float *)(oBuf + nk) + nk;
+    // host results up to 4 MB: copied to pinned memory before each round's wait
+    const bool outPinned = !idev && !ddev && !edev && !rcbc && outBytes <= ((size_t)4 << 20);
+    if (outPinned && s == PMLSH_OK) s = w.outStage.reserve(outBytes);
     if (s != PMLSH_OK) return s;
-    // pinned staging of the per-round decisions: order [nq], bounds [2 nq],
-    // verification outputs (k-th distance [nq] f64, fp64/verified/leaves
-    // counts [3 nq], error flag)
-    // (plus the radii [nq] f64 and an active or straddling list [nq] sent to
-    // the device, so that every copy is asynchronous)
-    PM_TRY(w.stage.reserve((size_t)nq * (8 + 4 * 8 + 8 + 8 + 4) + 64));
+    // pinned staging of the per-round decisions, so that every copy is asynchronous:
+    // k-th distances [nq] f64 followed by the verified and visited counts [2 nq]
+    // (one copy), radii [nq] f64, tight bounds [nq], the four round counters [4 nq],
+    // FP64 decisions with the flags after them [nq + 8], order, verification order,
+    // first-pass fallbacks, an active or straddling list [nq] each, flags
+    PM_TRY(w.stage.reserve((size_t)nq * (16 + 8 + 8 + 16 + 4 + 16) + 128));
     double *stDk = (double *)w.stage.p;
-    double *stR = stDk + nq;
+    int *stNv = (int *)(stDk + nq);   // (visited counts follow the verified ones)
+    double *stR = (double *)(stNv + 2 * nq);
     int2 *stTight = (int2 *)(stR + nq);
-    int32_t *stOrder = (int32_t *)(stTight + nq);
-    int *stHs = stOrder + nq, *stHp = stHs + nq, *stFp = stHp + nq, *stNv = stFp + nq, *stNl = stNv + nq,
-        *stVo = stNl + nq, *stRedo = stVo + nq, *stList = stRedo + nq, *stErr = stList + nq;
+    int *stHs = (int *)(stTight + nq), *stFp = stHs + 4 * nq;
+    int32_t *stOrder = stFp + nq + 8;
+    int *stVo = stOrder + nq, *stRedo = stVo + nq, *stList = stRedo + nq, *stErr = stList + nq;
     std::vector<int32_t> orderH;   // host copy, read after the first round's sync
 
     // host round state
@@ -2517,17 +2522,18 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
     const int bandCap = 1 << 20;
     int *actBuf = grow<int32_t>(w.active, nq, s);
     Thr *thr = grow<Thr>(w.thr, nq, s);
-    int *cntSure = grow<int>(w.cntSure, nq, s);
-    int *cntBand = grow<int>(w.cntBand, nq, s);
-    int *cntPart = grow<int>(w.cntPart, nq, s);
+    // the round's counters [nq] each, in one buffer so that the host reads them in
+    // one copy: whole-leaf members, partial leaves' members, band points, band points
+    // inside (a gathered sub-batch has the same order)
+    int *cntSure = grow<int>(w.cntSure, (size_t)4 * nq, s);
+    int *cntPart = cntSure + nq, *cntBand = cntSure + 2 * nq, *inTrue = cntSure + 3 * nq;
     int2 *cntTight = grow<int2>(w.cntTight, nq, s);
-    int *inTrue = grow<int>(w.bandCnt, nq, s);
     int *inN = grow<int>(w.bandIn, nq, s);
     int *inPos = grow<int>(w.bandInQ, (size_t)nq * BCAP, s);
     int *bandA = grow<int>(w.bandQ, bandCap, s);
     int *bandPos = grow<int>(w.bandPos, bandCap, s);
     int *fpc = grow<int>(w.flags, nq + 8, s);
-    double *dk = grow<double>(w.dk, nq, s);
+    double *dk = grow<double>(w.dk, (size_t)2 * nq, s);   // [nq], then the verification's counts [2 nq] int
     if (s != PMLSH_OK) return s;
     int *bandN = fpc + nq;       // counters after the per-query array
     int *errFlag = fpc + nq + 1;
@@ -2632,6 +2638,7 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
             uint32_t *fullBits;   // whole-leaf bits for the verification, or null
             int2 *cntTight;       // partial leaves' members surely / possibly inside (radial profiles), or null
             const int32_t *amb;   // a gathered sub-batch: its rows in the batch (lists from the batch's bits)
+            int64_t stride;       // entries between cntSure, cntPart, cntBand and inTrue
         };
         const int64_t Tdec = std::min<int64_t>(B, n);
         auto class_phase = [&](bool tc, const CountIO &io, ZeroList z, bool zeroed) -> pmlsh_status {
@@ -2746,14 +2753,14 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
                                                        io.fpc, errFlag));
                 PM_CUDA(cudaGetLastError());
                 // (pinned staging: copies to pageable memory would each wait)
+                // io's four counters lie `io.stride` apart
+                const int64_t cs = io.stride;
                 PM_CUDA(cudaMemcpyAsync(stErr, bandN, 3 * sizeof(int), cudaMemcpyDeviceToHost, st));
-                PM_CUDA(cudaMemcpyAsync(stHs, io.cntSure, io.na * sizeof(int), cudaMemcpyDeviceToHost, st));
-                PM_CUDA(cudaMemcpyAsync(stHp, io.cntBand, io.na * sizeof(int), cudaMemcpyDeviceToHost, st));
-                PM_CUDA(cudaMemcpyAsync(stNl, io.inTrue, io.na * sizeof(int), cudaMemcpyDeviceToHost, st));
+                PM_CUDA(cudaMemcpyAsync(stHs, io.cntSure, (3 * cs + io.na) * sizeof(int), cudaMemcpyDeviceToHost, st));
                 PM_CUDA(cudaStreamSynchronize(st));
                 es.assign(stHs, stHs + io.na);
-                eb.assign(stHp, stHp + io.na);
-                ein.assign(stNl, stNl + io.na);
+                eb.assign(stHs + 2 * cs, stHs + 2 * cs + io.na);
+                ein.assign(stHs + 3 * cs, stHs + 3 * cs + io.na);
                 for (int i = 0; i < 3; i++) hN[i] = stErr[i];
                 if (!(tcp && hN[2] > recheckCap)) break;
             }
@@ -2764,7 +2771,7 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
             return PMLSH_OK;
         };
         const CountIO full{act, na, thr, cntSure, cntPart, cntBand, inTrue, inN, inPos, fpc, leafBits, fullBits,
-                           stats == nullptr ? cntTight : nullptr, nullptr};
+                           stats == nullptr ? cntTight : nullptr, nullptr, nq};
         {
             // this round's per-query counters and the error and list counters
             // after them (fpc [nq + 8]) start at zero
@@ -2776,12 +2783,11 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
         std::vector<int2> ht;
         const bool needExact = stats != nullptr;
         if (!needExact) {
-            PM_CUDA(cudaMemcpyAsync(stHs, cntSure, na * sizeof(int), cudaMemcpyDeviceToHost, st));
-            PM_CUDA(cudaMemcpyAsync(stHp, cntPart, na * sizeof(int), cudaMemcpyDeviceToHost, st));
+            PM_CUDA(cudaMemcpyAsync(stHs, cntSure, (nq + na) * sizeof(int), cudaMemcpyDeviceToHost, st));
             if (full.cntTight) PM_CUDA(cudaMemcpyAsync(stTight, cntTight, na * sizeof(int2), cudaMemcpyDeviceToHost, st));
             PM_CUDA(cudaStreamSynchronize(st));
             hs.assign(stHs, stHs + na);
-            hp.assign(stHp, stHp + na);
+            hp.assign(stHs + nq, stHs + nq + na);
             hb.assign(na, 0);
             hin.assign(na, 0);
             if (full.cntTight) ht.assign(stTight, stTight + na);
@@ -2823,11 +2829,15 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
         // grouped kernel takes groups of GV_WARPS consecutive active queries
         // (locality order), a group's cost class being its costliest
         // member's.
-        int *nverD = grow<int>(w.partSeen, (size_t)4 * na + 8, s);
-        int *vOrder = nverD + 2 * na + 8;
+        int *vOrder = grow<int>(w.partSeen, (size_t)2 * na, s);
         int *redoD = vOrder + na;   // queries left by the BF16 first pass
+        int *nverD = (int *)(dk + nq);
+        // (a block per query with every block resident needs no order)
+        const bool vblock = !grouped && na <= vp.blockMax;
+        const int vbW = na <= 2 * nsm ? 8 : 4;
+        const bool vOrdered = !(vblock && na <= 16 / vbW * nsm);
         const int ngroups = (na + GV_WARPS - 1) / GV_WARPS;
-        {
+        if (vOrdered) {
             const int nunits = grouped ? ngroups : na;
             std::vector<int32_t> cls(nunits, 31);
             int64_t hist[33] = {0};
@@ -2856,7 +2866,7 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
             PM_CUDA(cudaMemcpyAsync(amb, stList, na2 * sizeof(int32_t), cudaMemcpyHostToDevice, st));
             PM_LAUNCH("k_gather_sub", st, k_gather_sub<<<(na2 + 255) / 256, 256, 0, st>>>(amb, na2, act, thr, act2, thr2));
             const CountIO subIO{act2, na2, thr2, s2Sure, s2Part, s2Band, s2In, s2InN, s2InPos, s2Fp, bits2, nullptr,
-                                nullptr, amb};
+                                nullptr, amb, na2};
             PM_TRY(class_phase(tensor, subIO, ZeroList(), false));   // zeroes inTrue, inN, fp64 of the sub-batch
             std::vector<int> es, eb, ein;
             PM_TRY(exact_count(subIO, es, eb, ein));
@@ -2906,7 +2916,6 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
         }
         // verification (order uploaded above): best-first over candidate
         // leaves, guard set, FP64
-        PM_CUDA(cudaMemsetAsync(nverD + 2 * na, 0, 8 * sizeof(int), st));
         if (grouped) {
             const int gGrid = std::max(1, std::min(ngroups, gvPerSM * nsm));
             uint32_t *ukey = grow<uint32_t>(w.partD, (size_t)gGrid * L * 9 / 4 + 16, s);
@@ -2918,7 +2927,7 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
             ga.KP = KP; ga.k = k;
             ga.inN = inN; ga.inPos = inPos; ga.perm = ix->perm; ga.outIds = oIds; ga.outD = oD; ga.outErr = oE;
             ga.dk = dk; ga.fp64cnt = fpc; ga.nverOut = nverD; ga.nleafOut = nverD + na; ga.errFlag = errFlag;
-            ga.workCtr = nverD + 2 * na; ga.dbg = nverD + 2 * na + 1; ga.n = n;
+            ga.workCtr = fpc + nq + 3; ga.dbg = fpc + nq + 4; ga.n = n;
             ga.leafBits = leafBits; ga.W32 = W32;
             ga.O64 = ix->O64; ga.qp64 = qp64; ga.m = m; ga.inlineBand = needExact ? 0 : 1;
             ga.leafPmu = ix->leafPmu; ga.qpca = qpca; ga.qnx = qnx;
@@ -2932,8 +2941,6 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
         } else {
             // a block per query (eight warps while one wave of two blocks per SM
             // holds the batch, else four), or a warp per query
-            const bool vblock = na <= vp.blockMax;
-            const int vbW = na <= 2 * nsm ? 8 : 4;
             const int vGrid = vblock ? std::min(na, 16 / vbW * nsm)
                                      : std::max(1, std::min((na + vWarps - 1) / vWarps, vPerSM * nsm));
             int2 *vLists = grow<int2>(w.partD, (size_t)vGrid * (vblock ? 1 : vWarps) * L, s);
@@ -2945,8 +2952,8 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
             va.leafOff = ix->leafOff; va.leafChunk = ix->leafChunk; va.chunkMu = ix->chunkMu; va.chunkRx = ix->chunkRx; va.KP = KP; va.k = k;
             va.inN = inN; va.inPos = inPos; va.perm = ix->perm; va.outIds = oIds; va.outD = oD; va.outErr = oE;
             va.dk = dk; va.fp64cnt = fpc; va.nverOut = nverD; va.nleafOut = nverD + na; va.errFlag = errFlag;
-            va.workCtr = nverD + 2 * na; va.dbg = nverD + 2 * na + 1; va.n = n; va.lists = vLists;
-            va.order = vOrder;
+            va.workCtr = fpc + nq + 3; va.dbg = fpc + nq + 4; va.n = n; va.lists = vLists;
+            va.order = vOrdered ? vOrder : nullptr;
             va.leafBits = leafBits; va.fullBits = fullBits; va.W32 = W32;
             va.O64 = ix->O64; va.qp64 = qp64; va.m = m; va.inlineBand = needExact ? 0 : 1;
             va.leafPmu = ix->leafPmu; va.qpca = qpca; va.qnx = qnx;
@@ -2964,19 +2971,22 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
         }
         PM_CUDA(cudaGetLastError());
         if (stats) {
-            PM_CUDA(cudaMemcpyAsync(stNl, nverD + na, na * sizeof(int), cudaMemcpyDeviceToHost, st));
-            PM_CUDA(cudaMemcpyAsync(stNv, nverD, na * sizeof(int), cudaMemcpyDeviceToHost, st));
-            PM_CUDA(cudaMemcpyAsync(stFp, fpc, na * sizeof(int), cudaMemcpyDeviceToHost, st));
+            // k-th distances with the counts after them; FP64 decisions with the flags
+            PM_CUDA(cudaMemcpyAsync(stDk, dk, nq * sizeof(double) + 2 * na * sizeof(int), cudaMemcpyDeviceToHost, st));
+            PM_CUDA(cudaMemcpyAsync(stFp, fpc, (nq + 8) * sizeof(int), cudaMemcpyDeviceToHost, st));
+        } else {
+            PM_CUDA(cudaMemcpyAsync(stDk, dk, na * sizeof(double), cudaMemcpyDeviceToHost, st));
+            PM_CUDA(cudaMemcpyAsync(stFp + nq, fpc + nq, 8 * sizeof(int), cudaMemcpyDeviceToHost, st));
         }
-        PM_CUDA(cudaMemcpyAsync(stDk, dk, na * sizeof(double), cudaMemcpyDeviceToHost, st));
-        PM_CUDA(cudaMemcpyAsync(stErr, errFlag, sizeof(int), cudaMemcpyDeviceToHost, st));
+        // small results for host arrays travel with the round's decisions (a round is
+        // mostly the last one)
+        if (outPinned) PM_CUDA(cudaMemcpyAsync(w.outStage.p, oIds, outBytes, cudaMemcpyDeviceToHost, st));
         if (bf16v) PM_CUDA(cudaMemcpyAsync(stRedo, redoD, na * sizeof(int), cudaMemcpyDeviceToHost, st));
         PM_CUDA(cudaStreamSynchronize(st));
         const double *dkH = stDk;
-        const int errH = *stErr;
+        const int errH = stFp[nq + 1];
         if (errH) {
-            int dbgH[3] = {0, 0, 0};
-            cudaMemcpy(dbgH, nverD + 2 * na + 1, sizeof(dbgH), cudaMemcpyDeviceToHost);
+            const int *dbgH = stFp + nq + 4;
             pm_set_error("internal error flags %d (index check %d value %d query %d); flags 2, 4, 8, 16, 32, "
                          "64: more points tied within one FP32 error band than an internal capacity; 128: a "
                          "staged copy timed out; 256/512: layout capacity", errH, dbgH[0], dbgH[1], dbgH[2]);
@@ -2991,7 +3001,7 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
             if (stats) {
                 fp64[q] += stFp[a];
                 nver[q] += stNv[a];
-                nleaf[q] += stNl[a];
+                nleaf[q] += stNv[na + a];
                 if (bf16v) fallback[q] += stRedo[a];
             }
             if (rcbc) {
@@ -3038,9 +3048,16 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
         }
     }
     // results held in scratch (host arrays of the caller)
-    if (!idev) PM_CUDA(cudaMemcpyAsync(ids, oIds, (size_t)nq * k * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    if (!ddev) PM_CUDA(cudaMemcpyAsync(dists, oD, (size_t)nq * k * sizeof(float), cudaMemcpyDeviceToHost, st));
-    if (err && !edev) PM_CUDA(cudaMemcpyAsync(err, oE, (size_t)nq * k * sizeof(float), cudaMemcpyDeviceToHost, st));
+    if (outPinned) {
+        const char *h = (const char *)w.outStage.p;
+        std::memcpy(ids, h, nk * 8);
+        std::memcpy(dists, h + nk * 8, nk * 4);
+        if (err) std::memcpy(err, h + nk * 12, nk * 4);
+    } else {
+        if (!idev) PM_CUDA(cudaMemcpyAsync(ids, oIds, nk * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+        if (!ddev) PM_CUDA(cudaMemcpyAsync(dists, oD, nk * sizeof(float), cudaMemcpyDeviceToHost, st));
+        if (err && !edev) PM_CUDA(cudaMemcpyAsync(err, oE, nk * sizeof(float), cudaMemcpyDeviceToHost, st));
+    }
     if (stats) {
         std::vector<pmlsh_query_stats> sv(nq);
         for (int64_t q = 0; q < nq; q++) {
@@ -3053,11 +3070,14 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
             sv[q].n_verified = nver[q];
             sv[q].first_pass_fallbacks = fallback[q];
         }
-        PM_CUDA(cudaMemcpyAsync(stats, sv.data(), nq * sizeof(pmlsh_query_stats),
-                                pm_is_device_ptr(stats) ? cudaMemcpyHostToDevice : cudaMemcpyHostToHost, st));
-        PM_CUDA(cudaStreamSynchronize(st));
+        if (pm_is_device_ptr(stats)) {
+            PM_CUDA(cudaMemcpyAsync(stats, sv.data(), nq * sizeof(pmlsh_query_stats), cudaMemcpyHostToDevice, st));
+            PM_CUDA(cudaStreamSynchronize(st));
+        } else {
+            std::memcpy(stats, sv.data(), nq * sizeof(pmlsh_query_stats));
+        }
     }
-    if (!idev || !ddev || (err && !edev)) PM_CUDA(cudaStreamSynchronize(st));
+    if (!outPinned && (!idev || !ddev || (err && !edev))) PM_CUDA(cudaStreamSynchronize(st));
     return PMLSH_OK;
 }
 

@@ -66,13 +66,14 @@ struct HostBuf {
 // Per-call scratch buffers of the query path (kept in the index, grown on
 // demand, reused across calls).
 struct KnnWork {
-    DevBuf Qd, qp32, qp64, qnorm, qpiv, order, keys, keys2, vals2, sortTmp;
-    DevBuf qstate, thr, blkCnt, blkLeaves, blkMask, cntSure, cntBand, bandQ, bandPos,
-        bandIn, bandCnt;
-    DevBuf partD, partI, partSeen, bandInQ, outD64, outIds, outErr, dk, flags;
+    DevBuf Qd, qp32, qp64, qnorm, qpiv, order, keys, vals2, sortTmp;
+    DevBuf qstate, thr, blkCnt, blkLeaves, blkMask, cntSure, bandQ, bandPos,
+        bandIn;
+    DevBuf partD, partI, partSeen, bandInQ, outIds, dk, flags;
     DevBuf selBuf, selOff, selCnt, selTau;
-    DevBuf active, misc, recheck, leafBits, fullBits, cntPart, cntTight, subIdx, subThr, subBits, qpca;
+    DevBuf active, misc, recheck, leafBits, fullBits, cntTight, subIdx, subThr, subBits, qpca;
     HostBuf stage;   // per-round decisions read by the host
+    HostBuf outStage;   // small results on their way to host arrays (up to 4 MB)
 };
 
 struct pmlsh_index {

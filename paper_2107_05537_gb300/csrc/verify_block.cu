@@ -301,16 +301,18 @@ k_verify_block(VwArgs A)
     const double epsv = (double)(ld + 8) * 0x1.0p-24;
     const float lbMulF = __double2float_rd(1.0 - epsv), cutF = __double2float_ru(1.0 + 3.0 * epsv);
     const float lbSlack = 1.f - (float)((ld + 8) * 0x1.0p-24) - 1e-6f;
-    for (;;) {
+    // the first query by the block's number, the others from the counter
+    for (int turn = 0;; turn++) {
         __syncthreads();
         if (tid == 0) {
-            S.work = atomicAdd(A.workCtr, 1);
+            S.work = turn == 0 ? (int)blockIdx.x
+                               : (A.nwork > (int)gridDim.x ? (int)gridDim.x + atomicAdd(A.workCtr, 1) : A.nwork);
             S.cnt = 0;
         }
         __syncthreads();
         int a = S.work;
         if (a >= A.nwork) break;
-        a = A.order[a];
+        if (A.order) a = A.order[a];
         if (!VW_CHECK(a >= 0, 7, a)) break;   // (block-uniform)
         const int q = A.act[a];
         const Thr Th = A.thr[a];
