@@ -477,7 +477,6 @@ struct Bisect {
     std::vector<int32_t> pre;   // [N] index of the node's segment for the refinement, -1 if inner
     std::vector<int64_t> preLo, preHi;
     std::vector<double> key;
-    std::vector<unsigned char> side;   // by position: the 2-means side of a segment the team splits
     // the final layout (assemble): leaf-index ranges of the nodes, leaves, chunks
     std::vector<int64_t> nlo, nhi;
     std::vector<int64_t> leafOff{0};
@@ -529,18 +528,60 @@ struct Bisect {
         });
     }
 
-    // The first point of perm[lo, hi) farthest from c.
-    int64_t farthest(HostTeam *team, const double *c, int64_t lo, int64_t hi) const
+    // A segment's coordinates in position order, by rows and by columns (copied once
+    // per split): the distances run over a column at a time, so that the compiler's
+    // vectors hold several points, each with its own sum in the order of the
+    // coordinates; only the sums over points walk the rows.
+    struct Points {
+        int64_t n = 0;
+        std::vector<float> row, col;
+        std::vector<unsigned char> side;
+    };
+    void load(HostTeam *team, Points &p, int64_t lo, int64_t hi) const
+    {
+        p.n = hi - lo;
+        p.row.resize((size_t)p.n * PM_MP);
+        p.col.resize((size_t)p.n * PM_MP);
+        p.side.resize((size_t)p.n);
+        parts(team, 0, p.n, [&](int, int64_t a, int64_t b) {
+            for (int64_t e = a; e < b; e++) {
+                const float *x = pt(perm[lo + e]);
+                for (int j = 0; j < PM_MP; j++) {
+                    p.row[(size_t)e * PM_MP + j] = x[j];
+                    p.col[(size_t)j * p.n + e] = x[j];
+                }
+            }
+        });
+    }
+    static constexpr int BLK = 256;
+    // d2(c, .) of the points [e, e + m), m <= BLK
+    static void d2_block(const Points &p, const double *c, int64_t e, int m, double *out)
+    {
+        for (int i = 0; i < m; i++) out[i] = 0.0;
+        for (int j = 0; j < PM_MP; j++) {
+            const float *x = p.col.data() + (size_t)j * p.n + e;
+            const double cj = c[j];
+            for (int i = 0; i < m; i++) {
+                const double t = cj - (double)x[i];
+                out[i] += t * t;
+            }
+        }
+    }
+
+    // The first point farthest from c.
+    static int64_t farthest(HostTeam *team, const Points &p, const double *c)
     {
         const int n = team ? team->threads() : 1;
         std::vector<double> best(n, -1.0);
-        std::vector<int64_t> at(n, lo);
-        parts(team, lo, hi, [&](int t, int64_t a, int64_t b) {
-            double v0 = -1.0;
+        std::vector<int64_t> at(n, 0);
+        parts(team, 0, p.n, [&](int t, int64_t a, int64_t b) {
+            double d[BLK], v0 = -1.0;
             int64_t i0 = a;
-            for (int64_t e = a; e < b; e++) {
-                const double v = d2(c, pt(perm[e]));
-                if (v > v0) { v0 = v; i0 = e; }
+            for (int64_t e = a; e < b; e += BLK) {
+                const int m = (int)std::min<int64_t>(BLK, b - e);
+                d2_block(p, c, e, m, d);
+                for (int i = 0; i < m; i++)
+                    if (d[i] > v0) { v0 = d[i]; i0 = e + i; }
             }
             best[t] = v0;
             at[t] = i0;
@@ -551,50 +592,65 @@ struct Bisect {
         return at[k];
     }
 
-    // 2-means of perm[lo, hi) started from a farthest pair; returns the
-    // hyperplane (w, t) separating the two means.  The sums run in the order of
-    // the points whatever the threads: the team divides the distances by points
-    // and the sums by coordinates.
-    void two_means(HostTeam *team, int64_t lo, int64_t hi, double *w, double &t)
+    // 2-means started from a farthest pair; returns the hyperplane (w, t) separating
+    // the two means.  The sums run in the order of the points whatever the threads:
+    // the team divides the distances by points and the sums by coordinates.
+    static void two_means(HostTeam *team, Points &p, double *w, double &t)
     {
         double c0[PM_MP], a[PM_MP], b[PM_MP];
-        for (int j = 0; j < PM_MP; j++) c0[j] = pt(perm[lo])[j];
-        const int64_t ia = farthest(team, c0, lo, hi);
-        for (int j = 0; j < PM_MP; j++) a[j] = pt(perm[ia])[j];
-        const int64_t ib = farthest(team, a, lo, hi);
-        for (int j = 0; j < PM_MP; j++) b[j] = pt(perm[ib])[j];
+        for (int j = 0; j < PM_MP; j++) c0[j] = p.row[j];
+        const int64_t ia = farthest(team, p, c0);
+        for (int j = 0; j < PM_MP; j++) a[j] = p.row[(size_t)ia * PM_MP + j];
+        const int64_t ib = farthest(team, p, a);
+        for (int j = 0; j < PM_MP; j++) b[j] = p.row[(size_t)ib * PM_MP + j];
         for (int it = 0; it < 6; it++) {
             double sa[PM_MP] = {0}, sb[PM_MP] = {0};
-            int64_t na = 0, nb = 0;
+            std::vector<int64_t> cb(team ? team->threads() : 1, 0);
+            parts(team, 0, p.n, [&](int part, int64_t x, int64_t y) {
+                double da[BLK], db[BLK];
+                int64_t c = 0;
+                for (int64_t e = x; e < y; e += BLK) {
+                    const int m = (int)std::min<int64_t>(BLK, y - e);
+                    d2_block(p, a, e, m, da);
+                    d2_block(p, b, e, m, db);
+                    for (int i = 0; i < m; i++) {
+                        p.side[e + i] = db[i] < da[i];
+                        c += p.side[e + i];
+                    }
+                }
+                cb[part] = c;
+            });
+            int64_t nb = 0;
+            for (int64_t c : cb) nb += c;
+            const int64_t na = p.n - nb;
             if (!team) {
-                for (int64_t e = lo; e < hi; e++) {
-                    const float *p = pt(perm[e]);
-                    if (d2(b, p) < d2(a, p)) { nb++; for (int j = 0; j < PM_MP; j++) sb[j] += p[j]; }
-                    else { na++; for (int j = 0; j < PM_MP; j++) sa[j] += p[j]; }
+                for (int64_t e = 0; e < p.n; e++) {
+                    const float *x = p.row.data() + (size_t)e * PM_MP;
+                    double *acc = p.side[e] ? sb : sa;
+                    for (int j = 0; j < PM_MP; j++) acc[j] += x[j];
                 }
             } else {
-                std::vector<int64_t> cb(team->threads(), 0);
-                parts(team, lo, hi, [&](int part, int64_t x, int64_t y) {
-                    int64_t c = 0;
-                    for (int64_t e = x; e < y; e++) {
-                        const float *p = pt(perm[e]);
-                        side[e] = d2(b, p) < d2(a, p);
-                        c += side[e];
-                    }
-                    cb[part] = c;
-                });
-                for (int64_t c : cb) nb += c;
-                na = hi - lo - nb;
                 parts(team, 0, PM_MP, [&](int, int64_t x, int64_t y) {
-                    double u[PM_MP] = {0}, v[PM_MP] = {0};
-                    for (int64_t e = lo; e < hi; e++) {
-                        const float *p = pt(perm[e]);
-                        double *acc = side[e] ? v : u;
-                        for (int64_t j = x; j < y; j++) acc[j] += p[j];
-                    }
                     for (int64_t j = x; j < y; j++) {
-                        sa[j] = u[j];
-                        sb[j] = v[j];
+                        const float *v = p.col.data() + (size_t)j * p.n;
+                        double u0 = 0.0, u1 = 0.0;
+                        // the other side's terms as +0, by masks: adding +0 to a sum
+                        // that began as +0 leaves it as it is, and a branch on the
+                        // side would be mispredicted every other point
+                        for (int64_t e = 0; e < p.n; e++) {
+                            const double x = (double)v[e];
+                            uint64_t bits, m1 = 0 - (uint64_t)p.side[e], b0, b1;
+                            std::memcpy(&bits, &x, 8);
+                            b0 = bits & ~m1;
+                            b1 = bits & m1;
+                            double x0, x1;
+                            std::memcpy(&x0, &b0, 8);
+                            std::memcpy(&x1, &b1, 8);
+                            u0 += x0;
+                            u1 += x1;
+                        }
+                        sa[j] = u0;
+                        sb[j] = u1;
                     }
                 });
             }
@@ -616,6 +672,35 @@ struct Bisect {
             bb += b[j] * b[j];
         }
         t = 0.5 * (bb - aa);
+    }
+
+    // The left points (key < t) of perm[lo, hi) to the front: the k-th right point
+    // among the first `left` positions changes places with the k-th left point
+    // beyond them, counted from the end -- std::partition's result, which a segment
+    // split by one thread gets from there.
+    void move_left(HostTeam &team, int64_t lo, int64_t hi, int64_t left, double t)
+    {
+        const int n = team.threads();
+        std::vector<std::vector<int64_t>> wrongL(n), wrongR(n);
+        parts(&team, lo, lo + left, [&](int part, int64_t a, int64_t b) {
+            for (int64_t e = a; e < b; e++)
+                if (!(key[perm[e]] < t)) wrongL[part].push_back(e);
+        });
+        parts(&team, lo + left, hi, [&](int part, int64_t a, int64_t b) {
+            for (int64_t e = b; e-- > a;)
+                if (key[perm[e]] < t) wrongR[part].push_back(e);
+        });
+        int pr = n - 1;
+        size_t ir = 0;
+        for (int pl = 0; pl < n; pl++)
+            for (int64_t e : wrongL[pl]) {
+                while (pr >= 0 && ir == wrongR[pr].size()) {
+                    pr--;
+                    ir = 0;
+                }
+                if (pr < 0) return;   // (as many of one kind as of the other)
+                std::swap(perm[e], perm[wrongR[pr][ir++]]);
+            }
     }
 
     int32_t new_node(int64_t lo, int64_t hi)
@@ -657,21 +742,29 @@ struct Bisect {
     // leaf does not straddle groups (c.mid stays -1 where it is not split).  A
     // degenerate 2-means split of a large segment falls back to the median along
     // the same direction.
-    void cut(HostTeam *team, Cut &c)
+    void cut(HostTeam *team, Cut &c, Points &p)
     {
         const int64_t lo = c.lo, hi = c.hi, size = hi - lo;
         if (size <= 8) return;
         double w[PM_MP], t;
-        two_means(team, lo, hi, w, t);
+        load(team, p, lo, hi);
+        two_means(team, p, w, t);
         std::vector<int64_t> right(team ? team->threads() : 1, 0);
-        parts(team, lo, hi, [&](int part, int64_t a, int64_t b) {
+        parts(team, 0, p.n, [&](int part, int64_t a, int64_t b) {
             int64_t r = 0;
-            for (int64_t e = a; e < b; e++) {
-                const float *p = pt(perm[e]);
-                double s = 0.0;
-                for (int j = 0; j < PM_MP; j++) s += w[j] * (double)p[j];
-                key[perm[e]] = s;
-                r += s >= t;
+            double s[BLK];
+            for (int64_t e = a; e < b; e += BLK) {
+                const int m = (int)std::min<int64_t>(BLK, b - e);
+                for (int i = 0; i < m; i++) s[i] = 0.0;
+                for (int j = 0; j < PM_MP; j++) {
+                    const float *x = p.col.data() + (size_t)j * p.n + e;
+                    const double wj = w[j];
+                    for (int i = 0; i < m; i++) s[i] += wj * (double)x[i];
+                }
+                for (int i = 0; i < m; i++) {
+                    key[perm[lo + e + i]] = s[i];
+                    r += s[i] >= t;
+                }
             }
             right[part] = r;
         });
@@ -684,6 +777,8 @@ struct Bisect {
                 left = size / 2;
                 std::nth_element(perm.begin() + lo, perm.begin() + lo + left, perm.begin() + hi, less);
                 t = K[perm[lo + left]];
+            } else if (team) {
+                move_left(*team, lo, hi, left, t);
             } else {
                 std::partition(perm.begin() + lo, perm.begin() + hi, [K, t](int32_t a) { return K[a] < t; });
             }
@@ -720,6 +815,7 @@ struct Bisect {
             return &pool.back();
         };
         Cut *root = make(0, n);
+        Points points;
         std::vector<Cut *> todo, large{root};
         while (!large.empty()) {
             Cut *c = large.back();
@@ -728,7 +824,7 @@ struct Bisect {
                 todo.push_back(c);
                 continue;
             }
-            cut(&team, *c);
+            cut(&team, *c, points);
             if (c->mid < 0) continue;
             c->left = make(c->lo, c->mid);
             c->right = make(c->mid, c->hi);
@@ -740,6 +836,7 @@ struct Bisect {
         std::atomic<int64_t> open{(int64_t)todo.size()};   // segments listed or in work
         team.run([&](int) {
             std::vector<Cut *> own;
+            Points mine_points;
             for (;;) {
                 Cut *c = nullptr;
                 if (!own.empty()) {
@@ -757,7 +854,7 @@ struct Bisect {
                     std::this_thread::yield();
                     continue;
                 }
-                cut(nullptr, *c);
+                cut(nullptr, *c, mine_points);
                 const bool mine = c->hi - c->lo <= small;   // (its children stay with this thread)
                 if (c->mid >= 0) {
                     {
@@ -1115,7 +1212,6 @@ pmlsh_status pm_build_index(pmlsh_index *ix, const float *X, bool x_on_device,
     bs.M = ix->M;
     bs.perm.resize(n);
     bs.key.resize(n);
-    bs.side.resize(n);
     std::iota(bs.perm.begin(), bs.perm.end(), 0);
     bs.split_all(n);
     // original-space refinement of the segments on the device, over the
