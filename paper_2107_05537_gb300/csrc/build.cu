@@ -1260,15 +1260,16 @@ pmlsh_status pm_build_index(pmlsh_index *ix, const float *X, bool x_on_device,
     PM_CUDA(cudaMemcpyAsync(ix->perm, ix->permH.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     PM_TRY(dalloc(&ix->leafOff, L + 1));
     PM_CUDA(cudaMemcpyAsync(ix->leafOff, ix->leafOffH.data(), (L + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, st));
+    PM_TRY(dalloc(&ix->O32, (size_t)n * PM_MP));
     PM_TRY(dalloc(&ix->O64, (size_t)n * PM_MP));
     if (layoutOnly) {
+        PM_LAUNCH("k_gather_rows", st, k_gather_rows<float><<<2048, 256, 0, st>>>(O32o, ix->O32, ix->perm, n, PM_MP));
         PM_LAUNCH("k_gather_rows", st, k_gather_rows<double><<<2048, 256, 0, st>>>(O64o, ix->O64, ix->perm, n, PM_MP));
         PM_CUDA(cudaGetLastError());
         PM_CUDA(cudaStreamSynchronize(st));
         return PMLSH_OK;
     }
     PM_TRY(dalloc(&ix->X, (size_t)n * ld));
-    PM_TRY(dalloc(&ix->O32, (size_t)n * PM_MP));
     PM_LAUNCH("k_gather_rows", st, k_gather_rows<float><<<2048, 256, 0, st>>>(Xo, ix->X, ix->perm, n, ld));
     PM_LAUNCH("k_gather_rows", st, k_gather_rows<float><<<2048, 256, 0, st>>>(O32o, ix->O32, ix->perm, n, PM_MP));
     PM_LAUNCH("k_gather_rows", st, k_gather_rows<double><<<2048, 256, 0, st>>>(O64o, ix->O64, ix->perm, n, PM_MP));

@@ -185,6 +185,144 @@ __global__ void k_gamma_ratio(const double *__restrict__ O64, int64_t n, int m, 
     }
 }
 
+// The same ratios in FP32, to find the few whose FP64 value can be the wanted rank.
+// Block a walks to its leaf once and keeps the ranges and radii of the nodes on the
+// way in shared memory: the lowest common node of (a, b), b > a, is the deepest one
+// that ends beyond b's leaf (k_gamma_ratio descends from the root for every pair and
+// divides in FP64: 50 M pairs 5.9 ms, here 0.85 ms for both passes).
+// LIST = false: v [pair] = R / d' approximately.  LIST = true, for a window [P, Q]:
+// with |sqrt(d'^2_32) - d'_64| <= eps = e0 + 2^-19 d' the ratio lies in
+// [R / (d' + eps), R / (d' - eps)]; pairs that lie below P by that are counted, those
+// above Q dropped, the rest listed with their node.  err bit 2: a path of more than
+// GP_DEPTH nodes.
+constexpr int GP_DEPTH = 1024;
+struct GammaPair {
+    int32_t a, b, node;
+};
+template <bool LIST>
+__global__ void __launch_bounds__(256)
+k_gamma_scan(const float *__restrict__ O32, int64_t n, const int32_t *__restrict__ leafOf,
+             const int64_t *__restrict__ node, const double *__restrict__ rad, float *__restrict__ v, float e0, float P,
+             float Q, unsigned long long *__restrict__ below, unsigned long long *__restrict__ nList,
+             unsigned long long cap, GammaPair *__restrict__ list, int *__restrict__ err)
+{
+    __shared__ int sEnd[GP_DEPTH], sNode[GP_DEPTH];
+    __shared__ float2 sR[GP_DEPTH];   // the radius rounded down and up
+    __shared__ int sDepth;
+    const int64_t a = blockIdx.x;
+    const int lane = threadIdx.x & 31;
+    const int la = leafOf[a];
+    if (threadIdx.x == 0) {
+        int64_t e = 0;
+        int depth = 0;
+        for (; depth < GP_DEPTH; depth++) {
+            sNode[depth] = (int)e;
+            sEnd[depth] = (int)node[e * 4 + 3];
+            const int64_t x = node[e * 4], y = node[e * 4 + 1];
+            if (x < 0) break;
+            e = la < node[x * 4 + 3] ? x : y;
+        }
+        if (depth == GP_DEPTH) atomicOr(err, 2);
+        sDepth = depth == GP_DEPTH ? GP_DEPTH - 1 : depth;   // the leaf's place
+    }
+    __syncthreads();
+    const int depth = sDepth;
+    for (int i = threadIdx.x; i <= depth; i += blockDim.x) {
+        const double r = rad[sNode[i]];
+        sR[i] = make_float2(__double2float_rd(r), __double2float_ru(r));
+    }
+    float oa[PM_MP];
+#pragma unroll
+    for (int j = 0; j < PM_MP; j++) oa[j] = O32[a * PM_MP + j];
+    __syncthreads();
+    const int64_t base = a * n - a * (a + 1) / 2 - a - 1;
+    unsigned long long mine = 0;
+    for (int64_t b0 = a + 1; b0 < n; b0 += blockDim.x) {
+        const int64_t b = b0 + threadIdx.x;
+        const bool ok = b < n;
+        float d = 0.f;
+        float2 R = make_float2(0.f, 0.f);
+        int at = 0;
+        if (ok) {
+            const int lb = leafOf[b];
+            // ends fall along the path: the last one beyond lb
+            int lo = 0, hi = depth;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (sEnd[mid] > lb) lo = mid;
+                else hi = mid - 1;
+            }
+            at = lo;
+            R = sR[lo];
+            float o[PM_MP];
+#pragma unroll
+            for (int j4 = 0; j4 < PM_MP / 4; j4++) {
+                const float4 x = __ldg((const float4 *)(O32 + b * PM_MP) + j4);
+                o[4 * j4] = x.x;
+                o[4 * j4 + 1] = x.y;
+                o[4 * j4 + 2] = x.z;
+                o[4 * j4 + 3] = x.w;
+            }
+            d = __fsqrt_rn(pm_pd2_32(oa, o));
+        }
+        if (!LIST) {
+            if (ok) v[base + b] = d > 0.f ? __fdividef(R.y, d) : (R.y > 0.f ? INFINITY : 0.f);
+        } else {
+            const float eps = __fmaf_ru(0x1.0p-19f, d, e0);
+            // a radius of 0 gives the ratio 0 at any distance
+            const bool under = R.y == 0.f ? P > 0.f : R.y < __fmul_rd(P, __fsub_rd(d, eps));
+            const bool over = R.x > __fmul_ru(Q, __fadd_ru(d, eps));
+            mine += ok && under ? 1 : 0;
+            if (ok && !under && !over) {
+                const unsigned long long slot = atomicAdd(nList, 1ull);
+                if (slot < cap) {
+                    GammaPair g;
+                    g.a = (int32_t)a;
+                    g.b = (int32_t)b;
+                    g.node = sNode[at];
+                    list[slot] = g;
+                }
+            }
+        }
+    }
+    if (LIST) {
+        for (int o = 16; o; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+        if (lane == 0 && mine) atomicAdd(below, mine);
+    }
+}
+
+// Exact ratios of the listed pairs (k_gamma_ratio's arithmetic).
+__global__ void __launch_bounds__(32)
+k_gamma_exact(const double *__restrict__ O64, int m, const GammaPair *__restrict__ list,
+              const unsigned long long *__restrict__ nList, unsigned long long cap, const double *__restrict__ rad,
+              double *__restrict__ out)
+{
+    const unsigned long long n = *nList < cap ? *nList : cap, e = blockIdx.x * 32ull + threadIdx.x;
+    if (e >= n) return;
+    const GammaPair g = list[e];
+    const double R = rad[g.node];
+    const double dv = pm_pdist64(O64 + (int64_t)g.a * PM_MP, O64 + (int64_t)g.b * PM_MP, m);
+    out[e] = dv > 0.0 ? __ddiv_rn(R, dv) : (R > 0.0 ? (double)INFINITY : 0.0);
+}
+
+// Histogram of w bits at `shift` of non-negative FP32 keys (their bits order like
+// them) that share the bits above.
+__global__ void __launch_bounds__(256)
+k_gamma_hist32(const float *__restrict__ v, int64_t N, int shift, int w, unsigned int hiMask, unsigned int prefix,
+               unsigned int *__restrict__ hist)
+{
+    __shared__ unsigned int h[2048];
+    for (int i = threadIdx.x; i < (1 << w); i += blockDim.x) h[i] = 0u;
+    __syncthreads();
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < N; e += (int64_t)gridDim.x * blockDim.x) {
+        const unsigned int k = __float_as_uint(v[e]);
+        if ((k & hiMask) == prefix) atomicAdd(&h[(k >> shift) & ((1u << w) - 1u)], 1u);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < (1 << w); i += blockDim.x)
+        if (h[i]) atomicAdd(&hist[i], h[i]);
+}
+
 // 256-bin histogram of 8 bits at `shift` of the keys whose bits above them
 // equal `prefix` (non-negative doubles and +inf order like their bits).
 __global__ void k_gamma_hist(const unsigned long long *__restrict__ v, int64_t N, int shift,
@@ -1328,19 +1466,84 @@ static pmlsh_status gamma_of_layout(const pmlsh_index *lx, double pr, double *ga
     int *err;
     PM_TRY(mem.get(&dNode, (size_t)N * 4));
     PM_TRY(mem.get(&dLeafOf, n));
-    PM_TRY(mem.get(&ratio, (size_t)npairs));
-    PM_TRY(mem.get(&hist, 256));
+    PM_TRY(mem.get(&hist, 2048));
     PM_TRY(mem.get(&err, 1));
     PM_CUDA(cudaMemcpyAsync(dNode, nodeH.data(), N * 4 * sizeof(int64_t), cudaMemcpyHostToDevice, st));
     PM_CUDA(cudaMemcpyAsync(dLeafOf, lof.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     PM_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
     PM_TRY(node_radii(lx, false, mem, &dRad, st));
+    int64_t rank = (int64_t)std::ceil(pr * (double)npairs - 1e-9);
+    rank = std::max<int64_t>(1, std::min<int64_t>(npairs, rank));
+    // 1. the ranked ratio in FP32, then the FP64 values of the pairs around it.  It
+    // stands if the rank falls among those and its value inside their window: every
+    // pair counted below is smaller, every one left out larger.
+    {
+        constexpr unsigned long long GL = 1ull << 16;
+        float *v;
+        unsigned long long *ctr;
+        GammaPair *list;
+        double *ex;
+        PM_TRY(mem.get(&v, (size_t)npairs));
+        PM_TRY(mem.get(&ctr, 2));
+        PM_TRY(mem.get(&list, (size_t)GL));
+        PM_TRY(mem.get(&ex, (size_t)GL));
+        PM_LAUNCH("k_gamma_scan", st, k_gamma_scan<false><<<(unsigned)(n - 1), 256, 0, st>>>(
+            lx->O32, n, dLeafOf, dNode, dRad, v, 0.f, 0.f, 0.f, nullptr, nullptr, 0, nullptr, err));
+        PM_CUDA(cudaGetLastError());
+        unsigned int prefix = 0;
+        int64_t need = rank;
+        const int shifts[3] = {21, 10, 0}, widths[3] = {11, 11, 10};
+        std::vector<unsigned int> hh(2048);
+        const int grid = (int)std::min<int64_t>(16 * 152, (npairs + 255) / 256);
+        for (int pass = 0; pass < 3; pass++) {
+            const unsigned int hiMask = pass == 0 ? 0u : (0xffffffffu << (shifts[pass] + widths[pass]));
+            PM_CUDA(cudaMemsetAsync(hist, 0, 2048 * sizeof(unsigned int), st));
+            PM_LAUNCH("k_gamma_hist32", st, k_gamma_hist32<<<grid, 256, 0, st>>>(v, npairs, shifts[pass], widths[pass],
+                                                                                hiMask, prefix, hist));
+            PM_CUDA(cudaMemcpyAsync(hh.data(), hist, sizeof(unsigned int) << widths[pass], cudaMemcpyDeviceToHost, st));
+            PM_CUDA(cudaStreamSynchronize(st));
+            int bin = 0;
+            while (bin < (1 << widths[pass]) - 1 && need > (int64_t)hh[bin]) need -= hh[bin++];
+            prefix |= (unsigned int)bin << shifts[pass];
+        }
+        float K;
+        std::memcpy(&K, &prefix, sizeof(K));
+        int herr = 0;
+        PM_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
+        PM_CUDA(cudaStreamSynchronize(st));
+        if (herr == 0 && K > 0.f && K < 1e30f) {
+            const float Pw = K * (1.f - 0x1.0p-16f), Qw = K * (1.f + 0x1.0p-16f);
+            const float e0 = nextafterf((float)(0x1.0p-22 * lx->maxNorm), INFINITY) + 1e-30f;
+            PM_CUDA(cudaMemsetAsync(ctr, 0, 2 * sizeof(unsigned long long), st));
+            PM_LAUNCH("k_gamma_scan", st, k_gamma_scan<true><<<(unsigned)(n - 1), 256, 0, st>>>(
+                lx->O32, n, dLeafOf, dNode, dRad, nullptr, e0, Pw, Qw, ctr, ctr + 1, GL, list, err));
+            PM_LAUNCH("k_gamma_exact", st, k_gamma_exact<<<(unsigned)(GL / 32), 32, 0, st>>>(lx->O64, lx->m, list, ctr + 1,
+                                                                                            GL, dRad, ex));
+            PM_CUDA(cudaGetLastError());
+            unsigned long long hc[2];
+            PM_CUDA(cudaMemcpyAsync(hc, ctr, sizeof(hc), cudaMemcpyDeviceToHost, st));
+            PM_CUDA(cudaStreamSynchronize(st));
+            const int64_t r = rank - (int64_t)hc[0];
+            if (hc[1] <= GL && r >= 1 && r <= (int64_t)hc[1]) {
+                std::vector<double> x((size_t)hc[1]);
+                PM_CUDA(cudaMemcpyAsync(x.data(), ex, x.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
+                PM_CUDA(cudaStreamSynchronize(st));
+                std::nth_element(x.begin(), x.begin() + (r - 1), x.end());
+                const double g = x[r - 1];
+                if (g >= (double)Pw && g <= (double)Qw) {
+                    *gamma = g;
+                    return PMLSH_OK;
+                }
+            }
+        }
+        PM_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
+    }
+    // 2. otherwise (many equal ratios, or none finite) every ratio in FP64
+    PM_TRY(mem.get(&ratio, (size_t)npairs));
     PM_LAUNCH("k_gamma_ratio", st, k_gamma_ratio<<<(unsigned)(n - 1), 256, 0, st>>>(lx->O64, n, lx->m, dLeafOf, dNode,
                                                                                      dRad, ratio, err));
     PM_CUDA(cudaGetLastError());
     // exact rank-th smallest ratio: radix select, 8 passes of 8 bits
-    int64_t rank = (int64_t)std::ceil(pr * (double)npairs - 1e-9);
-    rank = std::max<int64_t>(1, std::min<int64_t>(npairs, rank));
     unsigned long long prefix = 0, hiMask = 0;
     unsigned int hh[256];
     const int grid = (int)std::min<int64_t>(4096, (npairs + 255) / 256);

@@ -133,8 +133,8 @@ struct pmlsh_index {
     KnnWork work;
 };
 
-// Build helpers (build.cu).  layoutOnly: the leaf hierarchy and the FP64
-// projected points in leaf order only (no structure that queries read).
+// Build helpers (build.cu).  layoutOnly: the leaf hierarchy and the projected
+// points in leaf order only (no structure that queries read).
 pmlsh_status pm_build_index(pmlsh_index *ix, const float *X, bool x_on_device,
                             const pmlsh_build_opts *o, cudaStream_t st, bool layoutOnly = false);
 void pm_free_index(pmlsh_index *ix);

@@ -83,3 +83,26 @@ def test_branch_and_bound_tiles(n, clusters, leaf, T):
     assert got["pairs"].tolist() == rp.tolist()
     assert np.array_equal(got["dists"], rd.astype(np.float32))
     assert got["stats"]["count"] == T
+
+
+# the FP32 window around the wanted rank, and the data that leave it: equal ratios by
+# the thousand (copies, a grid), ranks at both ends
+@pytest.mark.parametrize("kind", ["mixture", "copies", "grid", "line"])
+@pytest.mark.parametrize("pr", [1e-9, 0.02, 0.5, 0.85, 1.0])
+def test_gamma_rank(kind, pr):
+    if kind == "mixture":
+        X, _, _, _ = datagen.mixture(900, 12, 9, 1.0, seed=3)
+    elif kind == "copies":
+        X = np.repeat(datagen.gaussian(60, 12, seed=5), 15, axis=0)
+    elif kind == "grid":
+        X = np.stack(np.meshgrid(*[np.arange(6.0)] * 3), -1).reshape(-1, 3).astype(np.float32)
+        X = np.concatenate([X, np.zeros((len(X), 9), np.float32)], 1)
+    else:
+        X = np.zeros((700, 12), np.float32)
+        X[:, 0] = 2.0 ** np.arange(700).clip(0, 60) + np.arange(700)
+    A = oracle.gen_projection(2, 15, 12).astype(np.float32)
+    ix = pm.Index(torch.from_numpy(X).cuda(), leaf_size=16, proj=A)
+    got = ix.gamma_calibrate(pr=pr)
+    ref = oracle.gamma_calibrate(ix.projected(), ix.layout(), pr)
+    ix.close()
+    assert got == ref or (math.isinf(got) and math.isinf(ref))
