@@ -27,6 +27,7 @@
 #include <cstring>
 #include <type_traits>
 
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include "knn_shared.cuh"
@@ -34,6 +35,7 @@
 namespace {
 
 using namespace pmk;
+namespace cg = cooperative_groups;
 
 
 // ------------------------------------------------------------ prep kernels
@@ -832,10 +834,12 @@ __global__ void k_band64(const int *__restrict__ bandN, int bandCap, const int *
 // --------------------------------------------------------- budget (rule 2)
 
 // Collects (FP32 d'^2, position) of every point with d'^2 <= hi for one
-// budget query.  Grid (budget query, leaf slice): a warp classifies 32
-// leaves at once (leaf_class, a lane per leaf), then takes the kept ones in
-// turn, its lanes testing 32 points at once (rows read together), and
-// appends the selected points with one atomic on the query's counter.
+// budget query.  Grid (budget query, leaf slice, share): a warp classifies 32
+// leaves at once (leaf_class, a lane per leaf), then takes the kept ones whose
+// rank falls to its share (gridDim.z shares: few queries need more warps than
+// there are sets of 32 leaves; four queries over 5,019 leaves 115 us in one share,
+// 38 in fifteen) in turn, its lanes testing 32 points at once (rows read together),
+// and appends the selected points with one atomic on the query's counter.
 __global__ void __launch_bounds__(256)
 k_collect(const int32_t *__restrict__ sel, const int32_t *__restrict__ act,
           const Thr *__restrict__ thr, const float *__restrict__ qp32,
@@ -862,9 +866,10 @@ k_collect(const int32_t *__restrict__ sel, const int32_t *__restrict__ act,
         const int64_t lme = l0 + lane;
         const unsigned char cme = lme < L ? leaf_class(qv, qpv, s, Rin, Rout, meta + lme * PM_LEAF_STRIDE) : CL_OUT;
         unsigned kept = __ballot_sync(0xffffffffu, cme != CL_OUT);
-        while (kept) {
+        for (int turn = 0; kept; turn++) {
             const int src = __ffs(kept) - 1;
             kept &= kept - 1;
+            if (turn % (int)gridDim.z != (int)blockIdx.z) continue;
             const int64_t l = l0 + src;
             const unsigned char c = (unsigned char)__shfl_sync(0xffffffffu, (int)cme, src);
             const int64_t p0 = off[l], p1 = off[l + 1];
@@ -894,8 +899,12 @@ k_collect(const int32_t *__restrict__ sel, const int32_t *__restrict__ act,
 
 // Radix select of the B-th smallest FP32 key, then the FP64-resolved cut:
 // keys < LO are surely among the B nearest, keys in [LO, HI] are ordered by
-// (FP64 d', id) and the first B - |{key < LO}| of them join.  One block of
-// 1024 threads per budget query.
+// (FP64 d', id) and the first B - |{key < LO}| of them join.  A cluster of one to
+// eight blocks of 1024 threads per budget query: each block counts its share of the
+// keys, the histograms are added through distributed shared memory (every block does
+// so, and so knows the digit), and the band meets in the first block, which orders
+// it.  Bound by the passes over the keys: four queries of 70,000 to 90,000 keys took
+// 102 us on one block each, 36 on eight.
 __global__ void __launch_bounds__(1024)
 k_select(const int32_t *__restrict__ sel, const int32_t *__restrict__ act, Thr *__restrict__ thr,
          const int64_t *__restrict__ selOff, const int *__restrict__ selCnt,
@@ -905,20 +914,27 @@ k_select(const int32_t *__restrict__ sel, const int32_t *__restrict__ act, Thr *
          int *__restrict__ inN, int *__restrict__ inPos, int *__restrict__ fp64cnt,
          int *__restrict__ errFlag)
 {
-    __shared__ unsigned int hist[2048];
+    __shared__ __align__(8) unsigned int hist[2048];
     __shared__ unsigned int sPrefix, sNeed;
     __shared__ double bd[SELBAND];
     __shared__ int bpos[SELBAND];
     __shared__ int bid[SELBAND];
     __shared__ int sSure, sBand;
     __shared__ unsigned int sWarp[32];
-    const int si = blockIdx.x;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int C = (int)cluster.num_blocks(), cr = (int)cluster.block_rank();
+    const int si = blockIdx.x / C;
     const int a = sel[si];
     const int q = act[a];
     const int64_t base = selOff[si];
     const int cnt = min(selCnt[si], (int)(selOff[si + 1] - selOff[si]));
     const unsigned int *keys = (const unsigned int *)(selKey + base);
-    if (threadIdx.x == 0) { sPrefix = 0; sNeed = (unsigned int)B; }
+    if (threadIdx.x == 0) {
+        sPrefix = 0;
+        sNeed = (unsigned int)B;
+        sSure = 0;
+        sBand = 0;
+    }
     const int shifts[3] = {21, 10, 0};
     const int widths[3] = {11, 11, 10};
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
@@ -931,7 +947,7 @@ k_select(const int32_t *__restrict__ sel, const int32_t *__restrict__ act, Thr *
         const unsigned int need = sNeed;
         // histogram: lanes with the same bin add once (keys of one query
         // share their leading bits, so bins are few and hot)
-        for (int e0 = wid * 32; e0 < cnt; e0 += nwarp * 32) {
+        for (int e0 = (cr * nwarp + wid) * 32; e0 < cnt; e0 += C * nwarp * 32) {
             const int e = e0 + lane;
             unsigned int bin = 0xFFFFFFFFu;
             if (e < cnt) {
@@ -941,12 +957,18 @@ k_select(const int32_t *__restrict__ sel, const int32_t *__restrict__ act, Thr *
             const unsigned int peers = __match_any_sync(0xffffffffu, bin);
             if (bin != 0xFFFFFFFFu && lane == __ffs(peers) - 1) atomicAdd(&hist[bin], (unsigned int)__popc(peers));
         }
-        __syncthreads();
+        cluster.sync();
         // the bin holding the need-th key: block-wide prefix over the bins
-        // (two per thread), the thread whose range holds it records it
+        // (two per thread, the cluster's counts added), the thread whose range
+        // holds it records it
         const int nbins = 1 << widths[pass];
         const int b0 = 2 * threadIdx.x;
-        const unsigned int h0 = b0 < nbins ? hist[b0] : 0u, h1 = b0 + 1 < nbins ? hist[b0 + 1] : 0u;
+        unsigned int h0 = 0u, h1 = 0u;
+        for (int r = 0; r < C && b0 < nbins; r++) {
+            const uint2 x = *(const uint2 *)(cluster.map_shared_rank(hist, r) + b0);
+            h0 += x.x;
+            h1 += x.y;
+        }
         unsigned int incl = h0 + h1;
         for (int o = 1; o < 32; o <<= 1) {
             const unsigned int t = __shfl_up_sync(0xffffffffu, incl, o);
@@ -969,32 +991,35 @@ k_select(const int32_t *__restrict__ sel, const int32_t *__restrict__ act, Thr *
             sNeed = need - ex - (first ? 0u : h0);
             sPrefix = pre | ((unsigned int)(first ? b0 : b0 + 1) << sh);
         }
-        __syncthreads();
+        cluster.sync();   // (the histograms are read)
     }
     const float tau32 = __uint_as_float(sPrefix);
     const double tau = sqrt((double)tau32);
     const double eps = band_eps(tau, maxNorm, qnorm[q]);
     const float LO = tau - 2.0 * eps > 0.0 ? __double2float_rd((tau - 2.0 * eps) * (tau - 2.0 * eps)) : 0.f;
     const float HI = __double2float_ru((tau + 2.0 * eps) * (tau + 2.0 * eps));
-    if (threadIdx.x == 0) { sSure = 0; sBand = 0; }
-    __syncthreads();
+    // keys below the band counted, those inside it listed, in the first block
+    int *rSure = cluster.map_shared_rank(&sSure, 0), *rBand = cluster.map_shared_rank(&sBand, 0);
+    double *rbd = cluster.map_shared_rank(bd, 0);
+    int *rbpos = cluster.map_shared_rank(bpos, 0), *rbid = cluster.map_shared_rank(bid, 0);
     int mySure = 0;
-    for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
+    for (int e = cr * blockDim.x + threadIdx.x; e < cnt; e += C * blockDim.x) {
         float v = selKey[base + e];
         if (v < LO) mySure++;
         else if (v <= HI) {
-            int slot = atomicAdd(&sBand, 1);
+            int slot = atomicAdd(rBand, 1);
             if (slot < SELBAND) {
                 int64_t pos = selPos[base + e];
-                bd[slot] = pm_pdist64(O64 + pos * PM_MP, qp64 + (int64_t)q * PM_MP, m);
-                bpos[slot] = (int)pos;
-                bid[slot] = perm[pos];
+                rbd[slot] = pm_pdist64(O64 + pos * PM_MP, qp64 + (int64_t)q * PM_MP, m);
+                rbpos[slot] = (int)pos;
+                rbid[slot] = perm[pos];
             }
         }
     }
     mySure = __reduce_add_sync(0xffffffffu, mySure);
-    if (lane == 0 && mySure) atomicAdd(&sSure, mySure);
-    __syncthreads();
+    if (lane == 0 && mySure) atomicAdd(rSure, mySure);
+    cluster.sync();
+    if (cr != 0) return;
     const int nband = sBand;
     const int need = (int)B - sSure;
     if (nband > SELBAND || need < 0 || need > nband) {
@@ -2907,11 +2932,34 @@ pmlsh_status pm_knn(pmlsh_index *ix, const float *Q, int64_t nq, const pmlsh_knn
             PM_CUDA(cudaMemsetAsync(selCnt, 0, ns * sizeof(int), st));
             // about eight 256-thread blocks per SM over all budget queries
             const int64_t gyc = std::max<int64_t>(1, std::min<int64_t>((L + 255) / 256, ((int64_t)8 * nsm + ns - 1) / ns));
-            PM_LAUNCH("k_collect", st, k_collect<<<dim3(ns, (unsigned)gyc), 256, 0, st>>>(
+            const int64_t gzc = std::max<int64_t>(1, std::min<int64_t>(32, (int64_t)8 * nsm / (ns * gyc)));
+            PM_LAUNCH("k_collect", st, k_collect<<<dim3(ns, (unsigned)gyc, (unsigned)gzc), 256, 0, st>>>(
                 sel, act, thr, qp32, qpiv, ix->s, ix->leafMeta, ix->leafOff, L, ix->O32, selOff,
                 selOff + ns + 1, selCnt, selKey, selPos, errFlag));
-            PM_LAUNCH("k_select", st, k_select<<<ns, 1024, 0, st>>>(sel, act, thr, selOff, selCnt, selKey, selPos, B, ix->maxNorm,
-                                          qnorm, ix->O64, qp64, m, ix->perm, inN, inPos, fpc, errFlag));
+            // as many blocks per query (a portable cluster size) as leave every block
+            // resident, two per SM, and 10,240 keys or more to each: with fewer the
+            // cluster's barriers cost more than the passes (139 queries of some 8,000
+            // keys: 42 us by two blocks, 21 by one)
+            int csel = 8;
+            while (csel > 1 && ((int64_t)ns * csel > 2 * nsm || selTotal / ns < (int64_t)csel * 10240)) csel >>= 1;
+            cudaLaunchConfig_t lc = {};
+            cudaLaunchAttribute la[1];
+            la[0].id = cudaLaunchAttributeClusterDimension;
+            la[0].val.clusterDim.x = (unsigned)csel;
+            la[0].val.clusterDim.y = 1;
+            la[0].val.clusterDim.z = 1;
+            lc.gridDim = dim3((unsigned)(ns * csel));
+            lc.blockDim = dim3(1024);
+            lc.stream = st;
+            lc.attrs = la;
+            lc.numAttrs = 1;
+            cudaError_t le = cudaSuccess;
+            PM_LAUNCH("k_select", st, le = cudaLaunchKernelEx(&lc, k_select, (const int32_t *)sel, (const int32_t *)act, thr,
+                                          (const int64_t *)selOff, (const int *)selCnt, (const float *)selKey,
+                                          (const int *)selPos, B, ix->maxNorm, (const double *)qnorm,
+                                          (const double *)ix->O64, (const double *)qp64, m,
+                                          (const int32_t *)ix->perm, inN, inPos, fpc, errFlag));
+            PM_CUDA(le);
             PM_CUDA(cudaGetLastError());
         }
         // verification (order uploaded above): best-first over candidate
