@@ -31,3 +31,24 @@ def test_counts_by_leaf_size(leaf, nq):
         for f in ("ncand", "rounds", "rule"):
             assert np.array_equal(got["stats"][f], ref[f])
     ix.close()
+
+
+# tensor cores: one M-tile, exactly one, and two of them per leaf (128 queries each), as
+# well as leaves that alternate between the two; leaves below, at and past a tile of
+# 128 points.  Every query of a tight bundle covers the same leaves partially.
+@pytest.mark.parametrize("leaf", [16, 128, 129, 600])
+@pytest.mark.parametrize("nq", [1, 127, 128, 129, 256, 257, 400])
+def test_tensor_counts_by_queries_per_leaf(leaf, nq):
+    X, Q, _, _ = datagen.mixture(2600, 24, 2, 4.0, seed=leaf, nq=nq)
+    rng = np.random.default_rng(nq)
+    Q[: (nq + 1) // 2] = Q[0] + rng.standard_normal(((nq + 1) // 2, 24)).astype(np.float32) * np.float32(0.01)
+    A = oracle.gen_projection(2, 13, 24).astype(np.float32)
+    t, _, _ = oracle.params(13, 1.5, 1 / math.e)
+    ix = pm.Index(torch.from_numpy(X).cuda(), m=13, leaf_size=leaf, proj=A)
+    for r in (3.0, 12.0, 25.0):
+        got = ix.knn(torch.from_numpy(Q).cuda(), k=3, beta=0.9, r_min=r, t=t, precision=pm.PMLSH_BF16_TENSOR)
+        ref = oracle.knn(X, A, Q, 3, 1.5, t, oracle.budget(len(X), 0.9, 3), r, 0)
+        assert np.array_equal(got["ids"].cpu().numpy(), ref["ids"])
+        for f in ("ncand", "rounds", "rule"):
+            assert np.array_equal(got["stats"][f], ref[f])
+    ix.close()
