@@ -68,7 +68,7 @@ __device__ __forceinline__ float vb_unkey(unsigned int k)
 {
     return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
 }
-// A finite stand-in that keeps the order: NaN (no bound) first.
+// A finite stand-in for a distance bound that keeps the order: NaN (no bound) first.
 __device__ __forceinline__ float vb_finite(float f)
 {
     return f != f ? -1e30f : fminf(fmaxf(f, -1e30f), 1e30f);
@@ -142,8 +142,9 @@ __device__ __noinline__ bool vb_band(const double *o, const double *q, int m, do
 }
 
 // Selection of the smallest values by the block: v[e stride], e < n, taking part
-// if valid[e stride] >= 0 (valid not null) and not above lim; NaN and values above
-// 1e30 count as 1e30.  Finds lo, hi and S.bin such that the values with v < lo, or
+// if valid[e stride] >= 0 (valid not null) and not above lim; NaN and infinity
+// count as the largest finite value (squared distances reach it; bounds stay within
+// +-1e30, so that a range never overflows).  Finds lo, hi and S.bin such that the values with v < lo, or
 // v <= hi and vb_bin(v) <= S.bin, are at least `want` (or all) and, unless values
 // tie, either at most `cap` in all or at most `capBin` in that bin (S.in; S.below
 // before it).  Bins are linear in the value and monotone under rounding.  Not
@@ -156,7 +157,7 @@ __device__ __forceinline__ int vb_bin(float v, float lo, float scale)
 {
     return min(VB_BINS - 1, (int)((v - lo) * scale));
 }
-__device__ __forceinline__ float vb_val(float v) { return fminf(v, 1e30f); }
+__device__ __forceinline__ float vb_val(float v) { return fminf(v, FLT_MAX); }
 
 __device__ __noinline__ VbCut vb_select(VbShared &S, const float *vals, const int *valid, int stride, int n, float lim,
                                         int want, int cap, int capBin)

@@ -91,3 +91,13 @@ def test_large_batch(d, k, precision):
     X, Q, _, _ = datagen.mixture(1500, d, 6, 1.0, seed=d, nq=64)
     A = oracle.gen_projection(8, 15, d).astype(np.float32)
     _check(X, Q, A, k, copies=80, precision=precision, with_stats=precision != 3)
+
+
+# squared distances far below and above 1 (at 1e16, above 1e33)
+@pytest.mark.parametrize("scale", [1e-6, 1e13, 1e16])
+@pytest.mark.parametrize("nq", [2, 130])
+def test_scales(scale, nq):
+    X, Q, _, _ = datagen.mixture(2503, 24, 2, 4.0, seed=9, nq=nq)
+    A = oracle.gen_projection(2, 13, 24).astype(np.float32)
+    _check((X * np.float32(scale)).astype(np.float32), (Q * np.float32(scale)).astype(np.float32), A, 3, leaf=100,
+           beta=0.9, r_min=25.0 * scale)
