@@ -319,7 +319,9 @@ constexpr float CL_INV_HI = 1.0f / (1.f + SLACK) * (1.f - 1e-7f);   // <= 1 / (1
 // that some query of the warp keeps.  The warps' masks of a tile meet in
 // shared memory (double-buffered, one barrier per tile), where the tile's
 // partially covered leaves are listed.  Queries beyond the batch sit at
-// +1e18 on every coordinate, so the centre test excludes them.
+// +1e18 on every coordinate, where the centre test excludes them at once unless
+// the points lie as far out; the masks leave them out in any case (k_count has
+// no thresholds for them).
 // NWD = 8 writes a query's bits as whole 32-byte sectors; NWD = 1 cuts the leaves
 // into eight times as many tiles, for batches whose larger tiles leave SMs idle.
 constexpr int CQ_LT = 256;   // leaf bit sets are padded to whole tiles of 256 leaves (32-byte sectors)
@@ -375,6 +377,7 @@ k_class(const int32_t *__restrict__ act, int na, const Thr *__restrict__ thr,
     float lowT[PM_MAX_PIVOTS], highT[PM_MAX_PIVOTS];
     float roL = 0.f, rinLo = -1.f;   // Rout (1 + SLACK) CL_INV_LO rounded up; Rin (1 - SLACK) rounded down
     const bool qv_ok = t < nb;
+    const uint32_t vm = __ballot_sync(VW_FULL, qv_ok);   // the warp's queries of the batch
     if (qv_ok) {
         const int q = act[a0 + t];
         const float4 *src = (const float4 *)(qp32 + (int64_t)q * PM_MP);
@@ -467,7 +470,7 @@ k_class(const int32_t *__restrict__ act, int na, const Thr *__restrict__ thr,
                             bits |= 1u << jj;
                         }
                     }
-                    const uint32_t m = __ballot_sync(VW_FULL, c == CL_PART);
+                    const uint32_t m = __ballot_sync(VW_FULL, c == CL_PART) & vm;
                     if (lane == 0) sM[buf][j][wp] = m;
                 }
             }

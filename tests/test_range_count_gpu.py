@@ -52,3 +52,23 @@ def test_tensor_counts_by_queries_per_leaf(leaf, nq):
         for f in ("ncand", "rounds", "rule"):
             assert np.array_equal(got["stats"][f], ref[f])
     ix.close()
+
+
+# points around the place of the leaf test's stand-in for queries beyond the batch
+# (+1e18 on every coordinate): a block's absent queries take part in nothing
+@pytest.mark.parametrize("nq", [3, 65, 300])
+@pytest.mark.parametrize("precision", [pm.PMLSH_FP32_PLAIN, pm.PMLSH_BF16_TENSOR])
+def test_points_at_the_absent_queries(nq, precision):
+    rng = np.random.default_rng(5)
+    X = (1e18 + 1e16 * rng.standard_normal((2500, 15))).astype(np.float32)
+    Q = (1e18 + 1e16 * rng.standard_normal((nq, 15))).astype(np.float32)
+    A = np.eye(15, dtype=np.float32)
+    t, _, _ = oracle.params(15, 1.5, 1 / math.e)
+    ix = pm.Index(torch.from_numpy(X).cuda(), leaf_size=64, proj=A)
+    for r in (1e16, 2e16):
+        got = ix.knn(torch.from_numpy(Q).cuda(), k=3, beta=0.9, r_min=r, t=t, precision=precision)
+        ref = oracle.knn(X, A, Q, 3, 1.5, t, oracle.budget(len(X), 0.9, 3), r, 0)
+        assert np.array_equal(got["ids"].cpu().numpy(), ref["ids"])
+        for f in ("ncand", "rounds", "rule"):
+            assert np.array_equal(got["stats"][f], ref[f])
+    ix.close()
