@@ -693,12 +693,20 @@ k_sublists(const int32_t *__restrict__ amb, int na2, const uint32_t *__restrict_
 // Per-point test in partially covered leaves (the queries of the block's
 // list mask).  Grid (block, split); a warp per listed leaf, up to four of its
 // points per lane in registers, so that a leaf of any size fills its lanes (a block
-// per leaf ran eight warps over leaves of 92 points on average).  Points go in
-// pairs through the packed arithmetic: each half is pm_pd2_32's sequence of
-// operations on that point, bit for bit.  Bound by FP32 issue, 32 operations per
-// pair of a query and a point; a query's coordinates are read once per 128 points
-// and its two counts leave the warp in one reduction.  5,000 queries on 300,000
-// points: 0.76 ms, 1.67 with a block per leaf and a point per thread.
+// per leaf ran eight warps over leaves of 92 points on average), two points to a
+// packed operation.  The decision is pm_pd2_32's against lo and hi.  It is taken
+// from x = ||o~||^2 - 2 q~.o~ where that is far enough from both: o~ = o' - g and q~ = q' - g
+// for the mean g of the block's queries, so that the norms are about as large as
+// the distances whatever the data's offset.  With u = 2^-24 and n the squared norms of
+// o~ and q~, x + n_q differs from d'^2 by at most
+//   u (4 (n_o + n_q) + 18 n_o + 17 n_q + 17 (2 n_o + n_q))
+// (coordinates rounded; the norms' sums; the 16 steps of the chain, whose partial sums
+// stay below 2 n_o + n_q), pm_pd2_32 from it by 18 u d'^2; u (80 n_o + 60 n_q + 32 hi)
+// holds both, with n_o the largest of the warp's points.  A query and 128 points with any pair in between (or not a number) are taken
+// again in pm_pd2_32's own operations, each half of a pair bit for bit.
+// Bound by FP32 issue: 16 operations per pair of a query and a point instead of 32.
+// 5,000 queries on 300,000 points: 0.61 ms; 0.74 with pm_pd2_32 for every pair, 1.67 with a
+// block per leaf and a point per thread.
 constexpr int CT_PTS = 4;   // points per lane
 __global__ void __launch_bounds__(256, 2)
 k_count(const int32_t *__restrict__ act, int na, const Thr *__restrict__ thr,
@@ -708,22 +716,45 @@ k_count(const int32_t *__restrict__ act, int na, const Thr *__restrict__ thr,
         int *__restrict__ cntSure, int *__restrict__ cntBand,
         int *__restrict__ bandN, int bandCap, int *__restrict__ bandA, int *__restrict__ bandPos)
 {
-    __shared__ __align__(16) unsigned long long sq[QB][PM_MP];   // (q_j, q_j)
-    __shared__ float2 sT[QB];                                    // lo, hi
+    __shared__ __align__(16) unsigned long long sq[QB][PM_MP];   // (-2 q~_j, -2 q~_j)
+    __shared__ float2 sT[QB];                                    // x <= .x: d'^2 <= lo; x > .y: d'^2 > hi
+    __shared__ float sRef[PM_MP][PM_MP + 1];                     // the mean's partial sums; row 0: g
     __shared__ int sSure[QB], sBand[QB];
     const int b = blockIdx.x;
     const int a0 = b * QB;
     const int nb = min(QB, na - a0);
     const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+    {
+        const int j = threadIdx.x % PM_MP, part = threadIdx.x / PM_MP;
+        float v = 0.f;
+        for (int qq = part; qq < nb; qq += 16) v += qp32[(int64_t)act[a0 + qq] * PM_MP + j];
+        sRef[part][j] = v;
+        __syncthreads();
+        if (part == 0) {
+            v = 0.f;
+            for (int i = 0; i < 16; i++) v += sRef[i][j];
+            sRef[0][j] = v / (float)nb;
+        }
+        __syncthreads();
+    }
     for (int e = threadIdx.x; e < QB * PM_MP; e += blockDim.x) {
         const int qq = e / PM_MP, j = e % PM_MP;
-        const float v = qq < nb ? qp32[(int64_t)act[a0 + qq] * PM_MP + j] : 0.f;
+        const float v = qq < nb ? -2.f * (qp32[(int64_t)act[a0 + qq] * PM_MP + j] - sRef[0][j]) : 0.f;
         sq[qq][j] = f32x2_pack(v, v);
     }
+    __syncthreads();
     for (int qq = threadIdx.x; qq < QB; qq += blockDim.x) {
         if (qq < nb) {
             const Thr T = thr[a0 + qq];
-            sT[qq] = make_float2(T.lo, T.hi);
+            float nq = 0.f;
+            for (int j = 0; j < PM_MP; j++) {
+                const float v = 0.5f * __uint_as_float((unsigned)sq[qq][j]);
+                nq = __fmaf_rn(v, v, nq);
+            }
+            const float E = __fmaf_ru(0x1.0p-24f, __fmaf_ru(60.f, nq, __fmul_ru(32.f, fmaxf(T.hi, 0.f))), 1e-30f);
+            // norms that could overflow below: not a number, every pair goes the exact way
+            const float bad = nq < 1e30f ? 0.f : __int_as_float(0x7fffffff);
+            sT[qq] = make_float2(__fsub_rd(__fsub_rd(T.lo, nq), E) + bad, __fadd_ru(__fsub_ru(T.hi, nq), E) + bad);
         }
         sSure[qq] = 0;
         sBand[qq] = 0;
@@ -738,22 +769,37 @@ k_count(const int32_t *__restrict__ act, int na, const Thr *__restrict__ thr,
         // NP pairs of points per lane: positions base + 32 u + lane
         auto run = [&](auto np, int64_t base, int64_t p1) {
             constexpr int NP = decltype(np)::value;
-            unsigned long long o[NP][PM_MP];
+            unsigned long long o[NP][PM_MP], no[NP];
+            float nmax = 0.f;
 #pragma unroll
             for (int u = 0; u < NP; u++) {
                 const int64_t pa = base + 64 * u + lane, pb = pa + 32;
-                // positions past the leaf: NaN, which no comparison takes
-                const float nan = __int_as_float(0x7fffffff);
+                no[u] = 0ull;
 #pragma unroll
                 for (int j4 = 0; j4 < PM_MP / 4; j4++) {
-                    const float4 x = pa < p1 ? __ldg((const float4 *)(O32 + pa * PM_MP) + j4) : make_float4(nan, nan, nan, nan);
-                    const float4 y = pb < p1 ? __ldg((const float4 *)(O32 + pb * PM_MP) + j4) : make_float4(nan, nan, nan, nan);
+                    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+                    const float4 x = pa < p1 ? __ldg((const float4 *)(O32 + pa * PM_MP) + j4) : z;
+                    const float4 y = pb < p1 ? __ldg((const float4 *)(O32 + pb * PM_MP) + j4) : z;
                     o[u][4 * j4] = f32x2_pack(x.x, y.x);
                     o[u][4 * j4 + 1] = f32x2_pack(x.y, y.y);
                     o[u][4 * j4 + 2] = f32x2_pack(x.z, y.z);
                     o[u][4 * j4 + 3] = f32x2_pack(x.w, y.w);
                 }
+#pragma unroll
+                for (int j = 0; j < PM_MP; j++) {
+                    o[u][j] = f32x2_add(o[u][j], f32x2_pack(-sRef[0][j], -sRef[0][j]));
+                    no[u] = f32x2_fma(o[u][j], o[u][j], no[u]);
+                }
+                // positions past the leaf: infinitely far
+                const float na2 = pa < p1 ? __uint_as_float((unsigned)no[u]) : INFINITY;
+                const float nb2 = pb < p1 ? __uint_as_float((unsigned)(no[u] >> 32)) : INFINITY;
+                if (pa < p1) nmax = fmaxf(nmax, na2);
+                if (pb < p1) nmax = fmaxf(nmax, nb2);
+                no[u] = f32x2_pack(na2, nb2);
             }
+            // (all non-negative or NaN, whose patterns order alike as integers)
+            nmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(nmax)));
+            const float El = nmax < 1e30f ? __fmul_ru(80.f * 0x1.0p-24f, nmax) : __int_as_float(0x7fffffff);
             unsigned long long bits = part;
             while (bits) {
                 const int qq = __ffsll(bits) - 1;
@@ -761,40 +807,68 @@ k_count(const int32_t *__restrict__ act, int na, const Thr *__restrict__ thr,
                 const ulonglong2 *qv = (const ulonglong2 *)sq[qq];
                 unsigned long long acc[NP];
 #pragma unroll
-                for (int u = 0; u < NP; u++) acc[u] = 0ull;
+                for (int u = 0; u < NP; u++) acc[u] = no[u];
 #pragma unroll
                 for (int j2 = 0; j2 < PM_MP / 2; j2++) {
                     const ulonglong2 x = qv[j2];
 #pragma unroll
                     for (int u = 0; u < NP; u++) {
-                        f32x2_sqdiff_acc(acc[u], o[u][2 * j2], x.x);
-                        f32x2_sqdiff_acc(acc[u], o[u][2 * j2 + 1], x.y);
+                        acc[u] = f32x2_fma(o[u][2 * j2], x.x, acc[u]);
+                        acc[u] = f32x2_fma(o[u][2 * j2 + 1], x.y, acc[u]);
                     }
                 }
                 const float2 T = sT[qq];
-                int c = 0;   // points <= lo, points <= hi (upper half)
+                const float tIn = __fsub_rd(T.x, El), tOut = __fadd_ru(T.y, El);
+                int c = 0;
+                bool open = false;
 #pragma unroll
                 for (int u = 0; u < NP; u++) {
                     const float v0 = __uint_as_float((unsigned)acc[u]), v1 = __uint_as_float((unsigned)(acc[u] >> 32));
-                    c += (v0 <= T.x ? 1 : 0) + (v1 <= T.x ? 1 : 0) + (v0 <= T.y ? 0x10000 : 0) + (v1 <= T.y ? 0x10000 : 0);
+                    c += (v0 <= tIn ? 1 : 0) + (v1 <= tIn ? 1 : 0);
+                    open |= !(v0 <= tIn || v0 > tOut) || !(v1 <= tIn || v1 > tOut);
                 }
-                c = __reduce_add_sync(0xffffffffu, c);
-                const int sure = c & 0xFFFF, band = (c >> 16) - sure;
-                if (lane == 0 && sure) atomicAdd(&sSure[qq], sure);
-                if (band) {   // (warp-uniform)
-                    if (lane == 0) atomicAdd(&sBand[qq], band);
+                if (!__any_sync(0xffffffffu, open)) {
+                    c = __reduce_add_sync(0xffffffffu, c);
+                    if (lane == 0 && c) atomicAdd(&sSure[qq], c);
+                    continue;
+                }
+                const Thr Te = thr[a0 + qq];
+                const float4 *qr = (const float4 *)(qp32 + (int64_t)act[a0 + qq] * PM_MP);
+                c = 0;   // points <= lo, points <= hi (upper half)
 #pragma unroll
-                    for (int u = 0; u < 2 * NP; u++) {
-                        const float v = __uint_as_float((unsigned)(u & 1 ? acc[u >> 1] >> 32 : acc[u >> 1]));
-                        if (v > T.x && v <= T.y) {
-                            const int e2 = atomicAdd(bandN, 1);
-                            if (e2 < bandCap) {
-                                bandA[e2] = a0 + qq;
-                                bandPos[e2] = (int)(base + 32 * u + lane);
+                for (int u = 0; u < NP; u++) {
+                    const int64_t pa = base + 64 * u + lane, pb = pa + 32;
+                    unsigned long long ex = 0ull;
+#pragma unroll
+                    for (int j4 = 0; j4 < PM_MP / 4; j4++) {
+                        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f), q4 = __ldg(qr + j4);
+                        const float4 x = pa < p1 ? __ldg((const float4 *)(O32 + pa * PM_MP) + j4) : z;
+                        const float4 y = pb < p1 ? __ldg((const float4 *)(O32 + pb * PM_MP) + j4) : z;
+                        f32x2_sqdiff_acc(ex, f32x2_pack(x.x, y.x), f32x2_pack(q4.x, q4.x));
+                        f32x2_sqdiff_acc(ex, f32x2_pack(x.y, y.y), f32x2_pack(q4.y, q4.y));
+                        f32x2_sqdiff_acc(ex, f32x2_pack(x.z, y.z), f32x2_pack(q4.z, q4.z));
+                        f32x2_sqdiff_acc(ex, f32x2_pack(x.w, y.w), f32x2_pack(q4.w, q4.w));
+                    }
+#pragma unroll
+                    for (int h = 0; h < 2; h++) {
+                        const float v = __uint_as_float((unsigned)(h ? ex >> 32 : ex));
+                        const int64_t pos = h ? pb : pa;
+                        if (pos < p1 && v <= Te.hi) {
+                            c += 0x10000 + (v <= Te.lo ? 1 : 0);
+                            if (!(v <= Te.lo)) {
+                                const int e2 = atomicAdd(bandN, 1);
+                                if (e2 < bandCap) {
+                                    bandA[e2] = a0 + qq;
+                                    bandPos[e2] = (int)pos;
+                                }
                             }
                         }
                     }
                 }
+                c = __reduce_add_sync(0xffffffffu, c);
+                const int sure = c & 0xFFFF, band = (c >> 16) - sure;
+                if (lane == 0 && sure) atomicAdd(&sSure[qq], sure);
+                if (lane == 0 && band) atomicAdd(&sBand[qq], band);
             }
         };
         const int64_t p1 = (int64_t)ent.y + ent.z;

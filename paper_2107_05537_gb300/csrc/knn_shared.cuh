@@ -161,6 +161,21 @@ __device__ __forceinline__ unsigned long long f32x2_pack(float lo, float hi)
     return ((unsigned long long)__float_as_uint(hi) << 32) | __float_as_uint(lo);
 }
 
+__device__ __forceinline__ unsigned long long f32x2_add(unsigned long long a, unsigned long long b)
+{
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ unsigned long long f32x2_fma(unsigned long long a, unsigned long long b,
+                                                        unsigned long long c)
+{
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
 // acc += (q - x)^2 for two coordinates at once: each half is a separate
 // round-to-nearest subtraction and fused multiply-add (the scalar
 // __fsub_rn / __fmaf_rn of that coordinate).

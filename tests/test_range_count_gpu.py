@@ -33,6 +33,26 @@ def test_counts_by_leaf_size(leaf, nq):
     ix.close()
 
 
+# the same far from the origin, where norms dwarf the distances, and at scales whose
+# squared norms are tiny or too large for the expanded form; a last leaf of few points
+@pytest.mark.parametrize("scale,offset", [(1.0, 1000.0), (1.0, -40.0), (1e-6, 0.0), (1e16, 0.0)])
+@pytest.mark.parametrize("nq", [2, 130])
+def test_counts_by_scale_and_offset(scale, offset, nq):
+    X, Q, _, _ = datagen.mixture(2500 + 3, 24, 2, 4.0, seed=9, nq=nq)
+    X = ((X + np.float32(offset)) * np.float32(scale)).astype(np.float32)
+    Q = ((Q + np.float32(offset)) * np.float32(scale)).astype(np.float32)
+    A = oracle.gen_projection(2, 13, 24).astype(np.float32)
+    t, _, _ = oracle.params(13, 1.5, 1 / math.e)
+    ix = pm.Index(torch.from_numpy(X).cuda(), m=13, leaf_size=100, proj=A)
+    for r in (3.0 * scale, 12.0 * scale, 25.0 * scale):
+        got = ix.knn(torch.from_numpy(Q).cuda(), k=3, beta=0.9, r_min=r, t=t, precision=pm.PMLSH_FP32_PLAIN)
+        ref = oracle.knn(X, A, Q, 3, 1.5, t, oracle.budget(len(X), 0.9, 3), r, 0)
+        assert np.array_equal(got["ids"].cpu().numpy(), ref["ids"])
+        for f in ("ncand", "rounds", "rule"):
+            assert np.array_equal(got["stats"][f], ref[f])
+    ix.close()
+
+
 # tensor cores: one M-tile, exactly one, and two of them per leaf (128 queries each), as
 # well as leaves that alternate between the two; leaves below, at and past a tile of
 # 128 points.  Every query of a tight bundle covers the same leaves partially.
