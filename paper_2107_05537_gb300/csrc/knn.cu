@@ -1,8 +1,10 @@
 // (c,k)-ANN query path: Algorithm 2 over a batch of queries.
 //
 // One round of Algorithm 2 for every still-active query is a fixed sequence
-// of kernels:
-//   k_thresholds   radius R = t r and the FP32 classification thresholds
+// of kernels (before the first, k_query_prep and k_order prepare the queries and
+// put them in locality order):
+//   k_thresholds   radius R = t r and the FP32 classification thresholds (in the
+//                  first round part of k_query_prep)
 //   k_class        Eq. 5 leaf test for (query block x leaf); counts whole-leaf
 //                  members and lists, per query block, the leaves that some
 //                  query covers partially, with the bit mask of those queries
@@ -1978,7 +1980,7 @@ __device__ __forceinline__ bool mbar_wait_or_fail(uint64_t *bar, uint32_t ph, vo
 // ||o'||^2 + ||q'||^2 - 2 q'.o' (split and accumulation error, FP32 rounding
 // of the norms, the CUDA-core computation's own error), d'^2~ <= lo - E is
 // surely in and > hi + E surely out; the pairs in between go to a recheck
-// list that k_recheck decides exactly as k_count does.  Counts and band
+// list that k_recheck decides by pm_pd2_32, as k_count does.  Counts and band
 // lists therefore equal k_count's.
 //
 // Roles: warp 0 streams point tiles (operand ring) and their norms (job
@@ -2382,7 +2384,7 @@ k_count_tc(const int32_t *__restrict__ act, int na, const Thr *__restrict__ thr,
 }
 
 // Exact decision of the pairs the tensor-core count left inside its error
-// band, in k_count's arithmetic: surely in -> count, band -> band list.
+// band, by pm_pd2_32: surely in -> count, band -> band list.
 __global__ void k_recheck(const int *__restrict__ recheckN, int recheckCap, const int2 *__restrict__ recheck,
                           const int32_t *__restrict__ act, const Thr *__restrict__ thr,
                           const float *__restrict__ qp32, const float *__restrict__ O32,
