@@ -221,43 +221,59 @@ __device__ __forceinline__ float warp_d2x2(const float4 *__restrict__ q4, const 
     return __shfl_sync(VW_FULL, keep, ((lane & 3) << 3) | (lane >> 2));
 }
 
-// warp_d2x2 with four lanes per row: eight rows per round and four rounds,
-// each lane's loads of a round issued together (nf4 / 4 float4 per lane), so
-// that half as many dependent load rounds stand between the rows and their
-// distances; each lane sums its coordinates in two packed partial sums, the
-// four lanes of a row are added by a butterfly.  Requires nf4 % 4 == 0.
-__device__ __forceinline__ float warp_d2x4(const float4 *__restrict__ q4, const float *p, int nf4, int lane)
+// Squared FP32 distances of the query to rows `row` of base (one per lane; -1: none,
+// the lane then gets 0), four lanes per row, sixteen rows per round and two rounds;
+// each lane sums its coordinates in two packed partial sums, the four lanes of a row
+// are added by a butterfly.  Requires nf4 % 8 == 0.  With 32 warps on an SM the data
+// pipe of shared memory and L1 bounds it (64% busy), not the loads in flight: a lane
+// takes two rows together, so that the query's coordinates are read once for both
+// (10,000 queries of 128: k_verify 1.92 -> 1.79 ms; a row at a time with eight loads in
+// flight before; four rows at a time spill, 1.89), and rows come as numbers (pointers
+// take twice the shuffles and registers, 1.84).
+__device__ __forceinline__ float warp_d2x4(const float4 *__restrict__ q4, const float *__restrict__ base, int row, int nf4,
+                                           int lane)
 {
     const int grp = lane >> 2, g = lane & 3;
     float keep = 0.f;
 #pragma unroll 1
-    for (int j = 0; j < 4; j++) {
-        const float4 *x4 = (const float4 *)__shfl_sync(VW_FULL, (unsigned long long)p, grp + 8 * j);
-        unsigned long long acc = 0ull;
-        if (x4 != nullptr) {
-            int t = g;
-            for (; t + 28 < nf4; t += 32) {
-                float4 x[8];
+    for (int j = 0; j < 4; j += 2) {
+        // (a missing row of a pair reads the other one)
+        int r[2];
+        const float4 *x[2];
 #pragma unroll
-                for (int u = 0; u < 8; u++) x[u] = __ldg(x4 + t + 4 * u);
+        for (int k = 0; k < 2; k++) r[k] = __shfl_sync(VW_FULL, row, grp + 8 * (j + k));
+        const int some = max(r[0], r[1]);
 #pragma unroll
-                for (int u = 0; u < 8; u++) {
+        for (int k = 0; k < 2; k++) x[k] = (const float4 *)base + (int64_t)(r[k] >= 0 ? r[k] : some) * nf4;
+        unsigned long long acc[2];
+#pragma unroll
+        for (int k = 0; k < 2; k++) acc[k] = 0ull;
+        if (some >= 0) {
+            for (int t = g; t < nf4; t += 8) {
+                float4 v[2][2];
+#pragma unroll
+                for (int u = 0; u < 2; u++)
+#pragma unroll
+                    for (int k = 0; k < 2; k++) v[k][u] = __ldg(x[k] + t + 4 * u);
+#pragma unroll
+                for (int u = 0; u < 2; u++) {
                     const float4 qv = q4[t + 4 * u];
-                    f32x2_sqdiff_acc(acc, f32x2_pack(qv.x, qv.y), f32x2_pack(x[u].x, x[u].y));
-                    f32x2_sqdiff_acc(acc, f32x2_pack(qv.z, qv.w), f32x2_pack(x[u].z, x[u].w));
+                    const unsigned long long q0 = f32x2_pack(qv.x, qv.y), q1 = f32x2_pack(qv.z, qv.w);
+#pragma unroll
+                    for (int k = 0; k < 2; k++) {
+                        f32x2_sqdiff_acc(acc[k], q0, f32x2_pack(v[k][u].x, v[k][u].y));
+                        f32x2_sqdiff_acc(acc[k], q1, f32x2_pack(v[k][u].z, v[k][u].w));
+                    }
                 }
             }
-            for (; t < nf4; t += 4) {
-                const float4 x = __ldg(x4 + t);
-                const float4 qv = q4[t];
-                f32x2_sqdiff_acc(acc, f32x2_pack(qv.x, qv.y), f32x2_pack(x.x, x.y));
-                f32x2_sqdiff_acc(acc, f32x2_pack(qv.z, qv.w), f32x2_pack(x.z, x.w));
-            }
         }
-        float a = __fadd_rn(__uint_as_float((unsigned)acc), __uint_as_float((unsigned)(acc >> 32)));
-        a = __fadd_rn(a, __shfl_xor_sync(VW_FULL, a, 1));
-        a = __fadd_rn(a, __shfl_xor_sync(VW_FULL, a, 2));
-        if (g == j) keep = a;
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            float a = __fadd_rn(__uint_as_float((unsigned)acc[k]), __uint_as_float((unsigned)(acc[k] >> 32)));
+            a = __fadd_rn(a, __shfl_xor_sync(VW_FULL, a, 1));
+            a = __fadd_rn(a, __shfl_xor_sync(VW_FULL, a, 2));
+            if (g == j + k) keep = a;
+        }
     }
     // lane (grp, g) holds row grp + 8 g; row v sits at lane 4 (v % 8) + v / 8
     return __shfl_sync(VW_FULL, keep, ((lane & 7) << 2) | (lane >> 3));
@@ -365,18 +381,18 @@ __device__ __forceinline__ double dist64_widen(const float *x, const float *y, i
 // sequential over the 16 coordinates, row minus query), float4 loads.
 __device__ __forceinline__ float pd2_row(const float *__restrict__ o, const float *__restrict__ qv)
 {
-    const float4 *o4 = (const float4 *)o;
+    const float4 *o4 = (const float4 *)o, *qv4 = (const float4 *)qv;   // (qv 16-byte aligned)
     float s = 0.f;
 #pragma unroll
     for (int j4 = 0; j4 < PM_MP / 4; j4++) {
-        const float4 x = __ldg(o4 + j4);
-        float t = __fsub_rn(x.x, qv[4 * j4]);
+        const float4 x = __ldg(o4 + j4), q = qv4[j4];
+        float t = __fsub_rn(x.x, q.x);
         s = __fmaf_rn(t, t, s);
-        t = __fsub_rn(x.y, qv[4 * j4 + 1]);
+        t = __fsub_rn(x.y, q.y);
         s = __fmaf_rn(t, t, s);
-        t = __fsub_rn(x.z, qv[4 * j4 + 2]);
+        t = __fsub_rn(x.z, q.z);
         s = __fmaf_rn(t, t, s);
-        t = __fsub_rn(x.w, qv[4 * j4 + 3]);
+        t = __fsub_rn(x.w, q.w);
         s = __fmaf_rn(t, t, s);
     }
     return s;

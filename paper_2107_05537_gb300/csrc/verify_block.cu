@@ -53,7 +53,8 @@ struct VbShared {
         VbWalk w;
         double sq64[2 * 32 * (VB_GR + 1)];   // squares of two steps of 32 coordinates, [coordinate][row]
     };
-    float sq[PM_MP], sp[PM_MAX_PIVOTS], sPq[PM_PCA];
+    alignas(16) float sq[PM_MP];
+    float sp[PM_MAX_PIVOTS], sPq[PM_PCA];
     unsigned int kMin, kMax;             // ordered keys of a minimum and a maximum
     int cnt, bin, below, in, work;
 };
